@@ -21,7 +21,7 @@ LIB = os.path.join(LIBDIR, "librubix.so")
 DEBUG_LIBDIR = os.path.join(HERE, "_lib_debug")
 DEBUG_LIB = os.path.join(DEBUG_LIBDIR, "librubix.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["api.cu", "engine.cu", "serve.cu", "sort.cu", "setup.cu", "deposit.cu", "rows.cu", "psf_lsf.cu", "adjoint.cu", "adjoint_tiles.cu", "noalloc.cu", "selftest.cu", "peak.cu"]
+SOURCES = ["api.cu", "engine.cu", "serve.cu", "sort.cu", "setup.cu", "deposit.cu", "deposit_k0.cu", "deposit_k1.cu", "deposit_k2.cu", "rows.cu", "psf_lsf.cu", "adjoint.cu", "adjoint_tiles.cu", "adjoint_k0.cu", "adjoint_k1.cu", "adjoint_k2.cu", "noalloc.cu", "selftest.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # Host code is compiled without floating-point contraction: the orientation
 # matrix and the key coordinates are defined with every product and sum

@@ -56,7 +56,7 @@ extern "C" rubix_status rubix_cube_create(const rubix_ssp_grid* ssp, const rubix
     if (!ssp || !tel) return fail(RUBIX_ERR_INVALID_ARG, "ssp or telescope is NULL");
     if (max_particles < 0 || max_particles > (1ll << 30)) return fail(RUBIX_ERR_INVALID_ARG, "max_particles out of range");
     rubix_cube* h = new rubix_cube();
-    rubix_status st = ssp_state_create(ssp, tel, &h->S);
+    rubix_status st = ssp_state_create(ssp, tel, true, &h->S);
     if (st == RUBIX_OK) st = plan_init(&h->P, h->S, tel, std::max<int64_t>(max_particles, 1), Alloc{}, false, true);
     if (st == RUBIX_OK && cudaDeviceSynchronize() != cudaSuccess)
         st = fail(RUBIX_ERR_CUDA, "create: %s", cudaGetErrorString(cudaGetLastError()));
@@ -155,7 +155,7 @@ extern "C" rubix_status rubix_cube_sorted(rubix_cube_t* h, int32_t* perm_out, in
     if (!h) return fail(RUBIX_ERR_INVALID_ARG, "NULL handle");
     const Plan& P = h->P;
     if (!P.have_forward) return fail(RUBIX_ERR_INVALID_ARG, "no forward has run on this handle");
-    const int nb = h->S->n_bands;
+    const int nb = h->S->geo.n_bands;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     CK(cudaSetDevice(h->S->device));
     if (perm_out && P.last_n > 0)
@@ -231,11 +231,11 @@ extern "C" rubix_status rubix_cube_stats(rubix_cube_t* h, int64_t* stats, int32_
     int n_in = 0;
     unsigned long long slow = 0;
     unsigned err = 0;
-    if (P.have_forward) CK(cudaMemcpy(&n_in, P.d_seg_off + (size_t)P.n_s * S.n_bands, 4, cudaMemcpyDeviceToHost));
+    if (P.have_forward) CK(cudaMemcpy(&n_in, P.d_seg_off + (size_t)P.n_s * S.geo.n_bands, 4, cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(&slow, S.d_slow, 8, cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(&err, S.d_err, 4, cudaMemcpyDeviceToHost));
     int64_t v[9] = {n_in, (int64_t)n_in * P.tel.n_lambda, (int64_t)slow, P.dep_launches, P.launches,
-                    (int64_t)err, S.tile_w, S.slab_w, S.n_bands};
+                    (int64_t)err, S.geo.tile_w, S.geo.slab_w, S.geo.n_bands};
     const int n = std::min<int>(*n_inout, 9);
     for (int i = 0; i < n; ++i) stats[i] = v[i];
     *n_inout = n;
@@ -332,7 +332,7 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
     A.seg_off = P.d_seg_off;
     A.sorted_keys = P.d_skeys;
     A.n_s = P.n_s;
-    A.n_bands = S.n_bands;
+    A.n_bands = S.geo.n_bands;
     A.n_lambda = P.tel.n_lambda;
     A.l0 = P.tel.lambda0;
     A.dl = P.tel.dlambda;
@@ -347,41 +347,27 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
     A.dv_dang = P.d_dvda;
     A.n_in = P.last_n;  // upper bound; the kernel reads the in-field count on the device
     // over the deposit's (tile, work item, age band) decomposition and slabs
-    launch_adjoint_setup(A, P.d_rec, P.d_wu, st);
+    launch_adjoint_setup(A, P.d_wu, st);
     AdjTileParams T{};
-    T.quad = S.d_quad;
-    T.quad16 = S.d_quad16;
-    T.qdt = S.qdt;
-    T.n_cells = S.n_cells;
-    T.n_ls = S.ssp.n_ls;
+    static_cast<SlabParams&>(T) = S.geo;
+    T.pair = S.d_pair_adj;
+    T.qdt = 0;
     T.rec = P.d_rec;
     T.wu = P.d_wu;
     T.items = P.d_items;
     T.item_off = P.d_item_off;
     T.seg_off = P.d_seg_off;
     T.n_s = P.n_s;
-    T.n_bands = S.n_bands;
-    for (int b = 0; b < kMaxBands; ++b) T.band_cell0[b] = S.band_cell0[b];
     T.G0 = G0;
     T.part = P.d_adjpart;
     T.n_cap = P.cap;
-    T.n_lambda = P.tel.n_lambda;
-    T.tile_w = S.tile_w;
-    T.n_tiles = S.n_tiles;
-    T.tile_klo = S.d_tile_klo;
-    T.slab_w = S.slab_w;
-    T.ncb = S.ncb;
-    T.box_w = S.box_w;
-    T.n_boxes = S.n_boxes;
-    T.cost_c0 = S.cost_c0;
     T.ls0_over = (float)(S.ssp.ls0 / S.ssp.dls);
     T.resample = P.tel.resample;
-    T.err = S.d_err;
-    if (launch_adjoint_tiles(T, &S.tmap, S.dep_ctas, RUBIX_ADJ_THREADS, S.dep_smem, st) < 0)
+    if (launch_adjoint_tiles(T, S.dep_ctas, RUBIX_ADJ_THREADS, S.dep_smem, st) < 0)
         return fail(RUBIX_ERR_CUDA, "adjoint launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    launch_adjoint_final(A, P.d_adjpart, S.n_tiles, P.cap, st);
+    launch_adjoint_final(A, P.d_adjpart, S.geo.n_tiles, P.cap, st);
     if (d_global)
-        launch_reduce_global(P.d_contrib, P.d_seg_off + (size_t)P.n_s * S.n_bands, d_global, P.d_red, st);
+        launch_reduce_global(P.d_contrib, P.d_seg_off + (size_t)P.n_s * S.geo.n_bands, d_global, P.d_red, st);
     CK(cudaGetLastError());
     return RUBIX_OK;
 }

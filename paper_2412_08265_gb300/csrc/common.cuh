@@ -76,12 +76,16 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
 }
 
-// 2-D tiled TMA load of box (c0 = innermost coordinate, c1 = row) into smem.
-__device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_addr(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(c0), "r"(c1)
-        : "memory");
+// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) from
+// global memory to the shared-space address dst.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
+                 : "memory");
+}
+
+__device__ __forceinline__ void sts_f4(uint32_t dst, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
 // 3-D tiled TMA load (c0 innermost).
@@ -171,7 +175,7 @@ __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
 // term j*a_lo is rounded.
 struct __align__(16) DepRec {
     float w[4];        // mass * flux_scale * bilinear weights: (ia,iz) (ia+1,iz) (ia,iz+1) (ia+1,iz+1)
-    int c0_bi;         // (SSP cell ia * max(n_Z - 1, 1) + iz) << 16 | (floor(t(0)) & 0xffff)
+    int c0_bi;         // (SSP cell ia * n_Z + iz) << 16 | (floor(t(0)) & 0xffff)
     float bf;          // t(0) - floor(t(0)), in [0, 1)
     float a_hi;        // dt/dj, high part
     float a_lo;        // dt/dj, low part

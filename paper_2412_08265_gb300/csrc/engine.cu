@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "engine.h"
+#include "tile.cuh"
 
 namespace rubix {
 
@@ -208,14 +209,15 @@ void ssp_state_destroy(SspState* S) {
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(S->device);
-    void* ptrs[] = {S->d_quad, S->d_quad16, S->d_la, S->d_lz, S->d_tile_klo, S->d_err, S->d_slow};
+    void* ptrs[] = {S->d_pair, S->d_pair_adj, S->d_la, S->d_lz, S->d_tile_klo, S->d_err, S->d_slow};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     cudaSetDevice(prev);
     delete S;
 }
 
-rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* tel, SspState** out) {
+rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* tel, bool with_adjoint,
+                              SspState** out) {
     *out = nullptr;
     rubix_status st = validate_ssp(ssp);
     if (st != RUBIX_OK) return st;
@@ -259,18 +261,102 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
         S.lz_nodes = h->d_lz;
     }
 
-    // ---- cell quads: for SSP cell (ia, iz) and node k, the four bilinear
-    // corners (ia,iz) (ia+1,iz) (ia,iz+1) (ia+1,iz+1), node-major
-    // [n_ls][n_cells], in the storage dtype: a float4 of FP32 values, or an
-    // 8-byte uint2 of BF16 / FP16 bit patterns (x = corner 0 | corner 1 << 16,
-    // y = corner 2 | corner 3 << 16) that the kernels widen to FP32 exactly ----
-    h->cz = std::max(S.n_Z - 1, 1);
+    // ---- deposit tiling: wavelength tiles and the slab staged per tile and age
+    // band: a band's age pairs (an odd number of 8-byte entries per node) over
+    // the nodes of the tile's R rounds plus a Doppler halo of
+    // +-RUBIX_DEP_VHALO. Among the band sizes that fit, take the one with the
+    // lowest estimated cost per particle: n_tiles * (per-particle setup + R
+    // rounds + bands). ----
     const int ca = std::max(S.n_age - 1, 1);
-    h->n_cells = ca * h->cz;
-    h->qdt = (S.dtype == RUBIX_F32) ? 0 : (S.dtype == RUBIX_BF16 ? 1 : 2);
+    const double A0 = tel->dlambda / ((1.0 + tel->z_cosmo) * S.dls);
+    const double beta = RUBIX_DEP_VHALO / kC_kms;
+    const double a_lo = A0 / (1.0 + beta), a_hi = A0 / (1.0 - beta);
+    const double lam_max = (tel->lambda0 + (tel->n_lambda - 1) * tel->dlambda) / (1.0 + tel->z_cosmo);
+    const int shift = (int)std::ceil(lam_max / S.dls * beta / (1.0 - beta));
+    const long long budget = ((long long)h->smem_optin - kDepHeader) / (long long)sizeof(float2);
+    const int nzc = std::max(S.n_Z, 2);  // entries per age cell and node
+    SlabParams& G = h->geo;
+    // kind 0 covers dt/dj in (30/31, 1] (and the two-read rounds just above 1)
+    // when the halo's range reaches it; kind 1 dt/dj in [1/2, 1); else kind 2
+    G.kind = (a_lo > 30.0 / 31.0 && a_lo < 1.0) ? 0 : ((a_lo >= 0.5 && a_hi < 0.999) ? 1 : 2);
+    const int B = kind_bins(G.kind);
+    struct Geo { int apb, bands, pitch, slab_w, R, need; double cost; };
+    Geo best{0, 0, 0, 0, 0, 0, 1e300};
+#define RUBIX_R(r) r,
+    const int rounds[] = {RUBIX_ROUNDS(RUBIX_R)};
+#undef RUBIX_R
+    for (int apb = ca; apb >= 1; --apb) {
+        const int bands = (ca + apb - 1) / apb;
+        if (bands > kMaxBands) break;
+        if (RUBIX_DEP_BANDS > 0 && bands != std::min(RUBIX_DEP_BANDS, ca)) continue;
+        const int pitch = (apb * nzc) | 1;
+        const int slab_w = (int)std::min<long long>(budget / pitch, 1 << 14) / 4 * 4;
+        for (int r : rounds) {
+            // bins of the last lane of the last round, deposit (also a mean
+            // round more) and adjoint (rounds of 32 bins, of 31 edges for means)
+            const int last = std::max({B * (r - 1) + 31, (B - 1) * r + r + 1, (B * r + 31) / 32 * 32 - 1});
+            const int need = (int)std::ceil((last + 1) * std::max(a_hi, 1.0)) + 3;
+            if (need + 2 * shift + 8 > slab_w) continue;
+            const int n_tiles = (tel->n_lambda + B * r - 1) / (B * r);
+            const double cost = n_tiles * (40.0 + 15.0 * r + 6.0 * bands);
+            if (cost < best.cost) best = Geo{apb, bands, pitch, slab_w, r, need, cost};
+        }
+    }
+    // no slab fits (very wide Doppler halo): global-memory path only (need = 0 =
+    // slab_w fails every kernel's test for a fast path)
+    if (best.R == 0) best = Geo{ca, 1, (ca * nzc) | 1, 0, 1, 0, 0.0};
+    h->apb = best.apb;
+    G.n_bands = best.bands;
+    G.pitch = best.pitch;
+    G.slab_w = best.slab_w;
+    G.need = best.need;
+    G.a_max = (float)a_hi;
+    G.tile_w = B * best.R;
+    G.n_tiles = (tel->n_lambda + G.tile_w - 1) / G.tile_w;
+    G.n_lambda = tel->n_lambda;
+    G.n_ls = S.n_ls;
+    G.es = S.n_Z > 1 ? 1 : 2;
+    G.pad = G.slab_w + 8;
+    G.ib = (float)std::floor(B * A0 + 0.5);
+    G.ib_mean = (float)std::floor((B - 1) * A0 + 0.5);
+    G.cost_c0 = RUBIX_DEP_COSTC0;
+    for (int b = 0; b < kMaxBands; ++b) G.band_e0[b] = std::min(b * best.apb, ca - 1) * nzc;
+    std::vector<int> klo(G.n_tiles, 0);
+    for (int t = 0; t < G.n_tiles; ++t) {
+        // nodes the tile's fast path reads: K0 .. K0 + need - 1 with K0 within
+        // +-shift of the zero-velocity position t00 of its first bin; slabs
+        // that would start beyond the templates' zero rows hold none of the
+        // tile's nodes
+        const int j0 = t * G.tile_w;
+        const double t00 = ((tel->lambda0 + j0 * tel->dlambda) / (1.0 + tel->z_cosmo) - S.ls0) / S.dls;
+        const double k = std::floor((t00 - shift - 1.0 - 0.5 * (G.slab_w - G.need - 2 * shift - 8)) / 4.0) * 4.0;
+        const double k_last = (S.n_ls + 3) / 4 * 4;
+        klo[t] = (int)std::max((double)-G.slab_w, std::min(k, k_last));
+    }
+    if (dalloc_sync(&h->d_tile_klo, G.n_tiles)) return bail(fail(RUBIX_ERR_OOM, "tile alloc"));
+    cudaMemcpy(h->d_tile_klo, klo.data(), klo.size() * 4, cudaMemcpyHostToDevice);
+    G.tile_klo = h->d_tile_klo;
+    h->dep_smem = deposit_smem_bytes(G.pitch, G.slab_w);
+    h->dep_ctas = h->n_sm;
+    G.err = h->d_err;
+
+    // ---- age pairs: entry (ia, iz) of node k holds templates (ia, iz) and
+    // (ia + 1, iz), so that a cell's four corners are entries iz and iz + 1 (a
+    // grid of one metallicity repeats its entry). One block per age band,
+    // node-major, pad zero node rows on both sides, in the storage dtype: FP32
+    // pairs, or two BF16 / FP16 bit patterns (first | second << 16) that the
+    // kernels widen to FP32 exactly ----
+    G.qdt = (S.dtype == RUBIX_F32) ? 0 : (S.dtype == RUBIX_BF16 ? 1 : 2);
+    static_assert(kDepHeader % 128 == 0, "slab must start 16-byte aligned");
     {
-        const int da = (S.n_age > 1) ? 1 : 0, dz = (S.n_Z > 1) ? 1 : 0;
-        auto tpl = [&](int ia, int iz, int k) { return (float)ssp->spectra[((size_t)ia * S.n_Z + iz) * S.n_ls + k]; };
+        const int da = (S.n_age > 1) ? 1 : 0;
+        const size_t rows = (size_t)S.n_ls + 2 * (size_t)G.pad;
+        G.band_stride = (long long)((rows * G.pitch + 3) / 4 * 4);
+        const size_t total = (size_t)G.band_stride * G.n_bands, entry = G.qdt ? 4 : 8;
+        std::vector<unsigned char> host(total * entry, 0);
+        // the adjoint's entries, FP32: the template and its difference to the
+        // next age's, so that its sums of age derivatives do not cancel
+        std::vector<float2> adj(with_adjoint ? total : 0, make_float2(0.f, 0.f));
         auto bits16 = [&](float f) -> uint32_t {
             if (S.dtype == RUBIX_BF16) return f32_to_bf16(f);
             const __half hv = __float2half_rn(f);
@@ -278,122 +364,64 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
             std::memcpy(&b, &hv, 2);
             return b;
         };
-        const size_t nq = (size_t)S.n_ls * h->n_cells;
-        if (h->qdt == 0) {
-            std::vector<float4> q(nq);
-            for (int ia = 0; ia < ca; ++ia)
-                for (int iz = 0; iz < h->cz; ++iz) {
-                    const int c = ia * h->cz + iz;
-                    for (int k = 0; k < S.n_ls; ++k)
-                        q[(size_t)k * h->n_cells + c] = make_float4(tpl(ia, iz, k), tpl(ia + da, iz, k),
-                                                                    tpl(ia, iz + dz, k), tpl(ia + da, iz + dz, k));
-                }
-            if (dalloc_sync(&h->d_quad, q.size())) return bail(fail(RUBIX_ERR_OOM, "quad alloc"));
-            if (cudaMemcpy(h->d_quad, q.data(), q.size() * sizeof(float4), cudaMemcpyHostToDevice) != cudaSuccess)
-                return bail(fail(RUBIX_ERR_CUDA, "quad copy"));
-        } else {
-            std::vector<uint2> q(nq);
-            for (int ia = 0; ia < ca; ++ia)
-                for (int iz = 0; iz < h->cz; ++iz) {
-                    const int c = ia * h->cz + iz;
-                    for (int k = 0; k < S.n_ls; ++k) {
-                        uint2 v;
-                        v.x = bits16(tpl(ia, iz, k)) | (bits16(tpl(ia + da, iz, k)) << 16);
-                        v.y = bits16(tpl(ia, iz + dz, k)) | (bits16(tpl(ia + da, iz + dz, k)) << 16);
-                        q[(size_t)k * h->n_cells + c] = v;
-                    }
-                }
-            if (dalloc_sync(&h->d_quad16, q.size())) return bail(fail(RUBIX_ERR_OOM, "quad alloc"));
-            if (cudaMemcpy(h->d_quad16, q.data(), q.size() * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
-                return bail(fail(RUBIX_ERR_CUDA, "quad copy"));
+        auto widen16 = [&](uint32_t u) -> float {
+            if (S.dtype == RUBIX_F16) {
+                const uint16_t h16 = (uint16_t)u;
+                __half hv;
+                std::memcpy(&hv, &h16, 2);
+                return __half2float(hv);
+            }
+            u <<= 16;
+            float f;
+            std::memcpy(&f, &u, 4);
+            return f;
+        };
+        // every template value once, as stored, then node by node (both passes
+        // write in order; the second reads n_age * n_Z streams)
+        const size_t nt = (size_t)S.n_age * S.n_Z;
+        std::vector<uint16_t> t16(G.qdt ? nt * S.n_ls : 0);
+        std::vector<float> tf(!G.qdt || with_adjoint ? nt * S.n_ls : 0);
+        for (size_t i = 0; i < nt * S.n_ls; ++i) {
+            float f = (float)ssp->spectra[i];
+            if (G.qdt) {
+                t16[i] = (uint16_t)bits16(f);
+                f = widen16(t16[i]);
+            }
+            if (!tf.empty()) tf[i] = f;
         }
-    }
-
-    // ---- deposit tiling: wavelength tiles and the quad slab staged per tile
-    // and age band. A band's slab holds ncb cells (odd) x slab_w nodes: the
-    // tile's R rounds of 31 bins plus a Doppler halo of +-RUBIX_DEP_VHALO.
-    // Among the band sizes that fit, take the one with the lowest estimated
-    // cost per particle: n_tiles * (per-particle setup + R rounds + bands). ----
-    const double A0 = tel->dlambda / ((1.0 + tel->z_cosmo) * S.dls);
-    const double v_halo = RUBIX_DEP_VHALO;
-    const double lam_max = (tel->lambda0 + (tel->n_lambda - 1) * tel->dlambda) / (1.0 + tel->z_cosmo);
-    const int shift = (int)std::ceil(lam_max / S.dls * (v_halo / kC_kms) / (1.0 - v_halo / kC_kms));
-    long long budget = (long long)h->smem_optin - kDepHeader;
-    if (RUBIX_DEP_CTAS > 1) {
-        int per_sm = 0;
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device);
-        budget = std::min<long long>(budget, per_sm / RUBIX_DEP_CTAS - 1024 - kDepHeader);  // 1 KB reserved per CTA
-    }
-    struct Geo { int apb, bands, ncb, box_w, n_boxes, slab_w, R; double cost; };
-    Geo best{0, 0, 0, 0, 0, 0, 0, 1e300};
-    const bool fast_A = A0 <= 1.0 && A0 > 1.0 - 1.0 / 31.0;
-    for (int apb = ca; apb >= 1; --apb) {
-        const int bands = (ca + apb - 1) / apb;
-        if (bands > kMaxBands) break;
-        if (RUBIX_DEP_BANDS > 0 && bands != std::min(RUBIX_DEP_BANDS, ca)) continue;
-        int ncb = apb * h->cz;
-        ncb += (ncb % 2 == 0) ? 1 : 0;
-        if (4 * ncb > 256) continue;  // TMA box: at most 256 elements per dimension
-        const long long wmax = budget / ((long long)ncb * (long long)sizeof(float4));
-        if (wmax < 64) continue;
-        // each box lands 128-byte aligned in shared memory (TMA destination
-        // rule): box_w * ncb * 16 bytes a multiple of 128, i.e. box_w % 8 == 0
-        const int n_boxes = (int)((wmax + 255) / 256);
-        const int box_w = (int)(wmax / n_boxes) / 8 * 8;
-        const int slab_w = n_boxes * box_w;
-        int R = 0;
-        for (int r = RUBIX_DEP_RMAX; r >= 1; --r)
-            if (31 * r + 1 + 2 * shift + 2 <= slab_w) { R = r; break; }
-        if (R == 0) continue;
-        if (!fast_A) R = std::min(R, 2);
-        const int n_tiles = (tel->n_lambda + 31 * R - 1) / (31 * R);
-        const double cost = n_tiles * (40.0 + 15.0 * R + 6.0 * bands);
-        if (cost < best.cost) best = Geo{apb, bands, ncb, box_w, n_boxes, slab_w, R, cost};
-    }
-    if (best.R == 0) {
-        // no slab fits (very wide Doppler halo): global-memory path only. ncb
-        // = 0 fails every kernel's "cell inside the slab" test, so that no
-        // particle takes a fast path into the (absent) slab.
-        best = Geo{ca, 1, 0, 0, 0, 0, 1, 0.0};
-    }
-    h->apb = best.apb;
-    h->n_bands = best.bands;
-    h->ncb = best.ncb;
-    h->box_w = best.box_w;
-    h->n_boxes = best.n_boxes;
-    h->slab_w = best.slab_w;
-    for (int b = 0; b < kMaxBands; ++b) h->band_cell0[b] = std::min(b * best.apb, ca - 1) * h->cz;
-    h->tile_w = 31 * best.R;
-    h->n_tiles = (tel->n_lambda + h->tile_w - 1) / h->tile_w;
-    std::vector<int> klo(h->n_tiles, 0);
-    for (int t = 0; t < h->n_tiles; ++t) {
-        // nodes the tile's fast path reads: K0 .. K0 + 31 R with K0 within
-        // +-shift of the zero-velocity position t00 of its first bin
-        const int j0 = t * h->tile_w;
-        const double t00 = ((tel->lambda0 + j0 * tel->dlambda) / (1.0 + tel->z_cosmo) - S.ls0) / S.dls;
-        const double need = 2.0 * shift + h->tile_w + 3.0;
-        const double k = std::floor(t00 - shift - 1.0 - 0.5 * (h->slab_w - need));
-        klo[t] = (int)std::max(-1e6, std::min(k, 1e6));
-    }
-    if (dalloc_sync(&h->d_tile_klo, h->n_tiles)) return bail(fail(RUBIX_ERR_OOM, "tile alloc"));
-    cudaMemcpy(h->d_tile_klo, klo.data(), klo.size() * 4, cudaMemcpyHostToDevice);
-    static_assert(kDepHeader % 128 == 0, "slab must start 128-byte aligned");
-    if ((h->box_w * h->ncb * (int)sizeof(float4)) % 128 != 0)
-        return bail(fail(RUBIX_ERR_CUDA, "internal: TMA box of %d x %d quads is not 128-byte aligned", h->box_w, h->ncb));
-    h->dep_smem = deposit_smem_bytes(h->ncb, h->slab_w);
-    h->dep_ctas = h->n_sm * RUBIX_DEP_CTAS;
-    if (h->slab_w > 0 && h->qdt == 0) {
-        PFN_encodeTiled_t enc = get_encode_tiled();
-        if (!enc) return bail(fail(RUBIX_ERR_CUDA, "cuTensorMapEncodeTiled unavailable"));
-        // 2-D view of the quads: x = 4 floats per cell (innermost), y = node
-        cuuint64_t gdim[2] = {(cuuint64_t)4 * h->n_cells, (cuuint64_t)S.n_ls};
-        cuuint64_t gstr[1] = {(cuuint64_t)h->n_cells * sizeof(float4)};
-        cuuint32_t box[2] = {(cuuint32_t)(4 * h->ncb), (cuuint32_t)h->box_w};
-        cuuint32_t es[2] = {1, 1};
-        CUresult r = enc(&h->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->d_quad, gdim, gstr, box, es,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return bail(fail(RUBIX_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r));
+        for (int b = 0; b < G.n_bands; ++b)
+            for (int k = 0; k < S.n_ls; ++k) {
+                size_t at = (size_t)b * G.band_stride + (size_t)(k + G.pad) * G.pitch;
+                for (int ia = b * best.apb; ia < std::min((b + 1) * best.apb, ca); ++ia)
+                    for (int z = 0; z < nzc; ++z, ++at) {
+                        const size_t t0 = ((size_t)ia * S.n_Z + std::min(z, S.n_Z - 1)) * S.n_ls + k;
+                        const size_t t1 = t0 + (size_t)da * S.n_Z * S.n_ls;
+                        if (G.qdt) {
+                            const uint32_t u = t16[t0] | ((uint32_t)t16[t1] << 16);
+                            std::memcpy(&host[at * 4], &u, 4);
+                        } else {
+                            const float v[2] = {tf[t0], tf[t1]};
+                            std::memcpy(&host[at * 8], v, 8);
+                        }
+                        if (with_adjoint) adj[at] = make_float2(tf[t0], tf[t1] - tf[t0]);
+                    }
+            }
+        if (cudaMalloc(&h->d_pair, total * entry) != cudaSuccess) {
+            h->d_pair = nullptr;
+            cudaGetLastError();
+            return bail(fail(RUBIX_ERR_OOM, "template alloc"));
+        }
+        if (cudaMemcpy(h->d_pair, host.data(), total * entry, cudaMemcpyHostToDevice) != cudaSuccess)
+            return bail(fail(RUBIX_ERR_CUDA, "template copy"));
+        G.pair = h->d_pair;
+        if (with_adjoint) {
+            if (dalloc_sync(&h->d_pair_adj, total)) {
+                cudaGetLastError();
+                return bail(fail(RUBIX_ERR_OOM, "template alloc"));
+            }
+            if (cudaMemcpy(h->d_pair_adj, adj.data(), total * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
+                return bail(fail(RUBIX_ERR_CUDA, "template copy"));
+        }
     }
     if (cudaDeviceSynchronize() != cudaSuccess)
         return bail(fail(RUBIX_ERR_CUDA, "SSP state: %s", cudaGetErrorString(cudaGetLastError())));
@@ -432,7 +460,7 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_items, sizeof(Item) * (size_t)item_cap}, {(void**)&P->d_rec, sizeof(DepRec) * N},
         {(void**)&P->d_prec, sizeof(PartRec) * N},
         {(void**)&P->d_partials, 4 * (size_t)part_cap * n_lambda},
-        {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.n_bands + 2)}, {(void**)&P->d_n_items, 4 * ((size_t)n_s + 1)},
+        {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.geo.n_bands + 2)}, {(void**)&P->d_n_items, 4 * ((size_t)n_s + 1)},
         {(void**)&P->d_n_parts, 4 * ((size_t)n_s + 1)}, {(void**)&P->d_item_off, 4 * ((size_t)n_s + 1)},
         {(void**)&P->d_part_off, 4 * ((size_t)n_s + 1)},
         {(void**)&P->d_scan_scratch, 4 * (scan_scratch_ints(n_s + 1) + 16)},
@@ -449,8 +477,8 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         v.push_back({(void**)&P->d_contrib, 8 * kGlobal * N});
         v.push_back({(void**)&P->d_dvda, 8 * N});
         v.push_back({(void**)&P->d_red, 8 * 1024});
-        v.push_back({(void**)&P->d_wu, 16 * N});
-        v.push_back({(void**)&P->d_adjpart, 16 * N * (size_t)std::max(S.n_tiles, 1)});
+        v.push_back({(void**)&P->d_wu, 8 * N});
+        v.push_back({(void**)&P->d_adjpart, 16 * N * (size_t)std::max(S.geo.n_tiles, 1)});
     }
     return v;
 }
@@ -702,12 +730,12 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         A.la_nodes = S.d_la;
         A.n_age = S.ssp.n_age;
         A.apb = S.apb;
-        A.n_bands = S.n_bands;
+        A.n_bands = S.geo.n_bands;
         P.launches += launch_assign(A, st);
-        P.launches += launch_sort_by_key(P.d_key, n, P.n_s * S.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
+        P.launches += launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
                                          P.d_perm, P.d_seg_off, P.d_sort_scratch, st);
     } else {
-        CK(cudaMemsetAsync(P.d_seg_off, 0, ((size_t)P.n_s * S.n_bands + 2) * sizeof(int), st));
+        CK(cudaMemsetAsync(P.d_seg_off, 0, ((size_t)P.n_s * S.geo.n_bands + 2) * sizeof(int), st));
     }
     if (ev) cudaEventRecord(ev[1], st);
     SetupParams SP{};
@@ -715,7 +743,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     SP.perm = P.d_perm;
     SP.seg_off = P.d_seg_off;
     SP.n_s = P.n_s;
-    SP.n_bands = S.n_bands;
+    SP.n_bands = S.geo.n_bands;
     SP.pin = P.d_pin;
     SP.l0 = P.tel.lambda0;
     SP.dl = P.tel.dlambda;
@@ -733,7 +761,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     ItemParams IP{};
     IP.seg_off = P.d_seg_off;
     IP.n_s = P.n_s;
-    IP.n_bands = S.n_bands;
+    IP.n_bands = S.geo.n_bands;
     IP.chunk = S.chunk;
     IP.n_items = P.d_n_items;
     IP.n_parts = P.d_n_parts;
@@ -770,35 +798,19 @@ int enqueue_deposit(const SspState& S, const DepJob* jobs, int n_jobs, long long
     NvtxRange nvtx("rubix: deposit");
     if (n_jobs < 1 || n_jobs > kMaxJobs) return -1;
     DepositParams DP{};
-    DP.quad = S.d_quad;
-    DP.quad16 = S.d_quad16;
-    DP.qdt = S.qdt;
-    DP.n_cells = S.n_cells;
-    DP.n_ls = S.ssp.n_ls;
+    static_cast<SlabParams&>(DP) = S.geo;
     for (int j = 0; j < n_jobs; ++j) DP.jobs[j] = jobs[j];
     DP.n_jobs = n_jobs;
     DP.job_cost = d_job_cost;
-    DP.n_bands = S.n_bands;
-    for (int b = 0; b < kMaxBands; ++b) DP.band_cell0[b] = S.band_cell0[b];
-    DP.n_lambda = S.n_lambda;
-    DP.tile_w = S.tile_w;
-    DP.n_tiles = S.n_tiles;
-    DP.tile_klo = S.d_tile_klo;
-    DP.slab_w = S.slab_w;
-    DP.ncb = S.ncb;
-    DP.box_w = S.box_w;
-    DP.n_boxes = S.n_boxes;
-    DP.cost_c0 = S.cost_c0;
-    DP.err = S.d_err;
     DP.slow_count = S.d_slow;
-    return launch_deposit(DP, &S.tmap, S.dep_ctas, S.dep_threads, S.dep_smem, st);
+    return launch_deposit(DP, S.dep_ctas, S.dep_threads, S.dep_smem, st);
 }
 
 int enqueue_post(Plan& P, float* target, float* out, uint64_t noise_seed, float noise_s2n, cudaStream_t st,
                  cudaEvent_t* ev) {
     NvtxRange nvtx("rubix: rows, PSF/LSF, noise");
     const int pitch = target == P.d_cube0 ? P.pitch0 : P.tel.n_lambda;
-    int l = launch_zero_empty(P.d_seg_off, P.n_s, P.S->n_bands, target, pitch, P.tel.n_lambda, st);
+    int l = launch_zero_empty(P.d_seg_off, P.n_s, P.S->geo.n_bands, target, pitch, P.tel.n_lambda, st);
     // d_n_parts (scanned into d_part_off by the item stage) is free here: the
     // combine's list of split spaxels
     l += launch_combine(P.d_part_off, P.n_s, P.tel.n_lambda, P.d_partials, target, pitch, P.d_n_parts, st);

@@ -30,35 +30,31 @@ rubix_status fail(rubix_status st, const char* fmt, ...);
 void set_last_error(const char* msg);
 
 // SSP templates on one device + the deposit tiling for one output wavelength
-// grid (n_lambda, lambda0, dlambda, z_cosmo): the cell quads the deposit and
-// adjoint read (the storage dtype's values), wavelength tiles,
-// the age bands and width of the shared-memory quad slab, and its TMA
-// descriptor.
+// grid (n_lambda, lambda0, dlambda, z_cosmo): the age pairs the deposit and
+// adjoint read (the storage dtype's values), wavelength tiles, and the age
+// bands and width of the shared-memory slab.
 struct SspState {
     int device = 0, n_sm = 0, smem_optin = 0;
     SspDev ssp{};
-    float4* d_quad = nullptr;   // [n_ls][n_cells] cell quads, FP32 templates
-    uint2* d_quad16 = nullptr;  // [n_ls][n_cells] cell quads, BF16 / FP16 templates (qdt 1 / 2)
-    int qdt = 0;
-    int n_cells = 0, cz = 1;    // cells = max(n_age-1,1) * cz, cz = max(n_Z-1,1)
+    void* d_pair = nullptr;     // age pairs of the templates, one block per age band (SlabParams)
+    float2* d_pair_adj = nullptr;  // the adjoint's form of them (null without backward): (T, T(ia + 1) - T)
+    SlabParams geo{};           // the deposit's tiles and slabs
     float* d_la = nullptr;
     float* d_lz = nullptr;
     int n_lambda = 0;
     double lambda0 = 0, dlambda = 0, z_cosmo = 0;
-    int tile_w = 31, n_tiles = 0, slab_w = 0, ncb = 1, box_w = 0, n_boxes = 0;
-    int n_bands = 1, apb = 1;
-    int band_cell0[kMaxBands] = {};
+    int apb = 1;                // age cells per band
     size_t dep_smem = 0;
     int* d_tile_klo = nullptr;
-    CUtensorMap tmap{};
-    int dep_ctas = 0, dep_threads = RUBIX_DEP_THREADS, chunk = RUBIX_DEP_CHUNK, cost_c0 = RUBIX_DEP_COSTC0;
+    int dep_ctas = 0, dep_threads = RUBIX_DEP_THREADS, chunk = RUBIX_DEP_CHUNK;
     unsigned* d_err = nullptr;              // device error word (kernel bit flags)
     unsigned long long* d_slow = nullptr;   // (particle, tile) pairs on the global-memory path
 };
 
 rubix_status validate_ssp(const rubix_ssp_grid* ssp);
 rubix_status validate_telescope(const rubix_telescope* tel, double ssp_dlambda);
-rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* wavelength_grid, SspState** out);
+rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* wavelength_grid, bool with_adjoint,
+                              SspState** out);
 void ssp_state_destroy(SspState* S);
 bool same_wavelength_grid(const SspState& S, const rubix_telescope* tel);
 // Spaxel rows the telescope's row window models (ny without a window).
@@ -118,7 +114,7 @@ struct Plan {
     long long* d_job_cost = nullptr;        // deposit launch scratch [kMaxJobs + 1]
     double *d_contrib = nullptr, *d_red = nullptr;
     float2* d_dvda = nullptr;               // backward: dv_los/d(inclination, azimuth) per particle [cap]
-    float4* d_wu = nullptr;                 // backward: unit-mass weights [cap]
+    float2* d_wu = nullptr;                 // backward: (ta, tz) in the SSP cell [cap]
     float4* d_adjpart = nullptr;            // backward: per (tile, particle) sums [n_tiles][cap]
     Alloc alloc;
     size_t bytes = 0;                       // device bytes held by the plan

@@ -23,26 +23,20 @@ int sm_count();
 #ifndef RUBIX_DEP_THREADS
 #define RUBIX_DEP_THREADS 896
 #endif
-// Deposit CTAs resident per SM (each gets 1/RUBIX_DEP_CTAS of the shared memory).
-#ifndef RUBIX_DEP_CTAS
-#define RUBIX_DEP_CTAS 1
-#endif
 // Deposit geometry: particles per work item, the line-of-sight speed (km/s)
-// the shared-memory slab's Doppler halo covers, the most 31-bin rounds per
-// wavelength tile, and a fixed number of age bands (0 = chosen by the cost
-// estimate).
+// the shared-memory slab's Doppler halo covers, and a fixed number of age
+// bands (0 = chosen by the cost estimate).
 #ifndef RUBIX_DEP_CHUNK
 #define RUBIX_DEP_CHUNK 256
 #endif
 #ifndef RUBIX_DEP_VHALO
 #define RUBIX_DEP_VHALO 800.0
 #endif
-#ifndef RUBIX_DEP_RMAX
-#define RUBIX_DEP_RMAX 12
-#endif
 #ifndef RUBIX_DEP_BANDS
 #define RUBIX_DEP_BANDS 0
 #endif
+// Rounds per wavelength tile that the deposit and the adjoint are built for.
+#define RUBIX_ROUNDS(X) X(1) X(2) X(3) X(4) X(6) X(8) X(10) X(11) X(12)
 // Cost of a work item in particle units, for the static split of the
 // (tile, item) cost space over CTAs.
 #ifndef RUBIX_DEP_COSTC0
@@ -153,30 +147,43 @@ struct DepJob {
     int pitch;               // cube row stride in floats (>= n_lambda)
     int resample;            // 1: bin means (records hold the bins' lower edges)
 };
-struct DepositParams {
-    const float4* quad;      // [n_ls][n_cells] SSP cell quads (the four bilinear corners per node), FP32
-    const uint2* quad16;     // the same as 16-bit values (qdt 1: BF16, 2: FP16; quad is then null)
+
+// Template slabs: the SSP grid's age pairs, one contiguous block per age band
+// ([pad + n_ls + pad] node rows of `pitch` entries; the pad rows are zero) of
+// FP32 float2 entries or, for 16-bit templates, uint32_t entries (qdt 1: BF16,
+// 2: FP16). The geometry of the wavelength tiles and of their shared-memory
+// slabs, shared by the deposit and the adjoint.
+struct SlabParams {
+    const void* pair;
     int qdt;
-    int n_cells, n_ls;
+    long long band_stride;      // entries per band block
+    int n_ls, pad, pitch, es;   // es: entries per cell index (tile.cuh)
+    int n_bands;
+    int band_e0[kMaxBands];     // first entry of each age band
+    int kind;                   // bins per round and how lanes reach their nodes (tile.cuh)
+    int n_lambda;
+    int tile_w;                 // output bins per tile = rounds x kind_bins(kind)
+    int n_tiles;
+    const int* tile_klo;        // [n_tiles] first SSP node of each tile's slab (a multiple of 4)
+    int slab_w;                 // nodes per slab (0 = no slab: global path only)
+    float a_max;                // largest dt/dj of the fast rounds, and
+    int need;                   // the nodes they read from a particle's first
+    float ib, ib_mean;  // whole nodes per round (LanePos::base steps)
+    int cost_c0;                // per-item cost in particle units
+    unsigned* err;
+};
+inline __host__ __device__ const void* band_ptr(const void* pair, int qdt, long long band_stride, int band) {
+    return static_cast<const char*>(pair) + (long long)band * band_stride * (qdt ? 4 : 8);
+}
+
+struct DepositParams : SlabParams {
     DepJob jobs[kMaxJobs];
     int n_jobs;
     long long* job_cost;     // [n_jobs + 1] device scratch: exclusive prefix of the jobs' per-tile cost
-    int n_bands;
-    int band_cell0[kMaxBands];  // first cell of each age band's slab
-    int n_lambda;
-    int tile_w;              // output bins per tile = 31 * rounds (1..12)
-    int n_tiles;
-    const int* tile_klo;     // [n_tiles] first SSP node of each tile's slab
-    int slab_w;              // nodes per slab (0 = no slab: global path only)
-    int ncb;                 // cells per slab node (odd)
-    int box_w, n_boxes;      // TMA boxes of box_w nodes covering the slab
-    int cost_c0;             // per-item cost in particle units
-    unsigned* err;
     unsigned long long* slow_count;
 };
-int launch_deposit(const DepositParams& P, const CUtensorMap* tmap, int n_ctas, int threads, size_t smem,
-                   cudaStream_t st);
-size_t deposit_smem_bytes(int ncb, int slab_w);
+int launch_deposit(const DepositParams& P, int n_ctas, int threads, size_t smem, cudaStream_t st);
+size_t deposit_smem_bytes(int pitch, int slab_w);
 
 // Zero rows of the spaxels without particles (no work item covers them).
 int launch_zero_empty(const int* seg_off, int n_s, int nb, float* cube, int pitch, int n_lambda, cudaStream_t st);
@@ -231,33 +238,22 @@ struct AdjointParams {
 // decomposition: per (tile, particle) the four sums
 //   part = (sum_j G S, sum_j G dS/dta', sum_j G dS/dtz', sum_j G dS/dt * t_abs)
 // over the tile's bins (unit mass), from the same shared-memory quad slabs.
-struct AdjTileParams {
-    const float4* quad;
-    const uint2* quad16;        // 16-bit quads (qdt 1: BF16, 2: FP16; quad is then null)
-    int qdt;
-    int n_cells, n_ls;
+struct AdjTileParams : SlabParams {
     const DepRec* rec;          // [n_in] forward records (sorted order)
-    const float4* wu;           // [n_in] unit-mass bilinear weights (0: spectrum misses every bin)
+    const float2* wu;           // [n_in] position (ta, tz) in the SSP cell
     const Item* items;
     const int* item_off;        // [n_s + 1]
     const int* seg_off;         // [n_s * n_bands + 2]
-    int n_s, n_bands;
-    int band_cell0[kMaxBands];
+    int n_s;
     const float* G0;            // [n_s][n_lambda] dL/d(cube before PSF/LSF)
     float4* part;               // [n_tiles][n_cap]
     long long n_cap;
-    int n_lambda, tile_w, n_tiles;
-    const int* tile_klo;
-    int slab_w, ncb, box_w, n_boxes;
-    int cost_c0;
     float ls0_over;             // ls0 / dls: node index -> rest wavelength / dls
     int resample;               // 1: bin means (records hold the bins' lower edges)
-    unsigned* err;
 };
-int launch_adjoint_tiles(const AdjTileParams& P, const CUtensorMap* tmap, int n_ctas, int threads, size_t smem,
-                         cudaStream_t st);
-// Unit-mass bilinear weights per sorted particle (K7 setup).
-int launch_adjoint_setup(const AdjointParams& P, const DepRec* rec, float4* wu, cudaStream_t st);
+int launch_adjoint_tiles(const AdjTileParams& P, int n_ctas, int threads, size_t smem, cudaStream_t st);
+// Position in the SSP cell per sorted particle (K7 setup).
+int launch_adjoint_setup(const AdjointParams& P, float2* wu, cudaStream_t st);
 // Sum of the tiles' parts in FP64 (tile order) and the chain rule to
 // dL/d(mass, age, Z, v_los) in original order (+ contributions to global sums).
 int launch_adjoint_final(const AdjointParams& P, const float4* part, int n_tiles, long long n_cap, cudaStream_t st);

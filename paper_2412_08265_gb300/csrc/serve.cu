@@ -347,7 +347,7 @@ extern "C" rubix_status rubix_serve_create(const rubix_ssp_grid* ssp, const rubi
     srv->max_batch = max_batch;
     cudaGetDevice(&srv->device);
     {
-        st = ssp_state_create(ssp, wavelength_grid, &srv->S);
+        st = ssp_state_create(ssp, wavelength_grid, false, &srv->S);
         if (st != RUBIX_OK) goto done;
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;

@@ -84,7 +84,7 @@ __global__ void k_setup(SetupParams P) {
         r.w[1] = ms * (ta * (1.f - tz));
         r.w[2] = ms * ((1.f - ta) * tz);
         r.w[3] = ms * (ta * tz);
-        const int c0 = ia * max(P.ssp.n_Z - 1, 1) + iz;  // SSP cell of the four corners
+        const int c0 = ia * P.ssp.n_Z + iz;  // SSP cell: its first entry among the age pairs
         // b = v/c, q = 1 + b, g = b / q: one FP32 quotient and one correction
         // from the double-float residual b - g0 q (relative error ~2^-46)
         const DF b = df_mul_f(invc, pr.v);

@@ -33,101 +33,163 @@ __device__ __forceinline__ int node_pos(int j, int bi, float bf, float a_hi, flo
     return bi + (int)pi + (int)fl;
 }
 
+// Geometry of the rounds: a warp takes a particle's tile in rounds of kBins
+// consecutive bins, lane l owning bin j0 + kBins r + l. The kind follows from
+// the bin step in template nodes A = dt/dj (chosen once per wavelength grid):
+//   0: A near 1 (1 - A in [0, 1/31)): 31 bins, lanes on consecutive nodes;
+//   1: A in [1/2, 1): 30 bins, each lane on its bin's node, the next node's
+//      value from lane l + 1 or l + 2;
+//   2: any A: 32 bins, each lane reads both of its bin's nodes.
+constexpr int kind_bins(int kind) { return kind == 0 ? 31 : kind == 1 ? 30 : 32; }
+
 struct TileCtx {
-    int j0, klo, slab_w, ncb, cell0, n_lambda, n_ls, n_cells;
-    const uint2* q16;  // 16-bit cell quads (qdt 1: BF16, 2: FP16); null: FP32 quads
-    int qdt;
+    int j0, klo, slab_w, pitch, e0, es, n_lambda, n_ls, pad;
+    uint32_t slab;         // shared-space address of the slab
+    const void* gband;     // this band's entries in global memory (FP32 float2 or 16-bit uint32_t)
+    int qdt;               // 0: FP32, 1: BF16, 2: FP16
+    float a_max;           // largest dt/dj whose rounds stay within `need` nodes
+    int need;              // nodes the rounds of one particle can read, from its first
 #if RUBIX_DEBUG
-    unsigned* err;     // error word for the debug build's index checks
+    unsigned* err;         // error word for the debug build's index checks
 #endif
 };
 
+// Entry of a record's cell within the band's node rows (es = 2 for a grid of
+// one metallicity, whose rows repeat each age's entry).
+__device__ __forceinline__ int rec_entry(int c0_bi, const TileCtx& C) { return rec_c0(c0_bi) * C.es - C.e0; }
+
+// The two 16-bit values of an entry as FP32 (exact).
+__device__ __forceinline__ float2 unpack_pair(uint32_t v, int qdt) {
+    if (qdt == 1) return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+    return make_float2(__half2float(__ushort_as_half((unsigned short)(v & 0xffffu))),
+                       __half2float(__ushort_as_half((unsigned short)(v >> 16))));
+}
+
+// A cell's two entries (four corner templates) at one node.
+struct Quad {
+    float2 a, b;  // corners (ia, iz) (ia+1, iz); (ia, iz+1) (ia+1, iz+1)
+};
+
+// Shared-memory read of the two entries at byte address `addr`. Two 8-byte
+// loads: 32 lanes on consecutive nodes are an odd number of 8-byte entries
+// apart, so each load is conflict-free (two wavefronts).
+__device__ __forceinline__ Quad lds_quad(uint32_t addr, const TileCtx& C) {
+    Quad q;
 #if RUBIX_DEBUG
-// Debug builds: the slab nodes the fast-path rounds of one particle will
-// read, replayed with the rounds' own carry arithmetic (rounds of `step`
-// bins; node K0 + o_r + lane for r < n_rounds, the last round read by lanes
-// up to last_lanes only, plus the neighbours lo .. hi of each node) lie
-// inside the slab.
-__device__ __forceinline__ bool dbg_rounds_in_slab(int base, float f, float delta, const TileCtx& C, int lane,
-                                                   int n_rounds, int step, int last_lanes, int lo, int hi) {
-    const float d = (float)step * delta;
-    const int n = C.slab_w * C.ncb;
-    bool ok = true;
-    int o = 0;
-    for (int r = 0; r < n_rounds; ++r) {
-        if (r < n_rounds - 1 || lane <= last_lanes) {
-            ok = ok && base + (o + lane + lo) * C.ncb >= 0 && base + (o + lane + hi) * C.ncb < n;
-        }
-        f -= d;
-        const bool carry = f < 0.f;
-        f = carry ? f + 1.f : f;
-        o += carry ? step - 1 : step;
+    const uint32_t off = addr - C.slab;
+    const bool ok = off + 16u <= (uint32_t)(C.slab_w * C.pitch) * 8u && (off & 7u) == 0u;
+    dbg_check(ok, C.err);
+    if (!ok) {
+        q.a = q.b = make_float2(0.f, 0.f);
+        return q;
     }
-    return ok;
-}
 #endif
-
-// The four corner templates of a 16-bit cell quad (x = corners 0 | 1 << 16,
-// y = corners 2 | 3 << 16) as FP32 values (exact).
-__device__ __forceinline__ float4 unpack_quad(const uint2 v, int qdt) {
-    if (qdt == 1)
-        return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
-                           __uint_as_float(v.y & 0xffff0000u));
-    return make_float4(__half2float(__ushort_as_half((unsigned short)(v.x & 0xffffu))),
-                       __half2float(__ushort_as_half((unsigned short)(v.x >> 16))),
-                       __half2float(__ushort_as_half((unsigned short)(v.y & 0xffffu))),
-                       __half2float(__ushort_as_half((unsigned short)(v.y >> 16))));
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(q.a.x), "=f"(q.a.y) : "r"(addr));
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+8];" : "=f"(q.b.x), "=f"(q.b.y) : "r"(addr));
+    return q;
 }
 
-// Quad of `cell` at node k from the global quad array, FP32 or 16-bit (zero
-// outside the template range: the template's zero extension).
-__device__ __forceinline__ float4 quad_global(const float4* __restrict__ quad, const TileCtx& C, int cell, int k) {
-    if (k < 0 || k >= C.n_ls) return make_float4(0.f, 0.f, 0.f, 0.f);
-    const long long i = (long long)k * C.n_cells + cell;
-    return C.qdt ? unpack_quad(__ldg(C.q16 + i), C.qdt) : __ldg(quad + i);
+// The same from the band's global array (zero outside the template range: the
+// template's zero extension). e: the cell's entry within the band.
+__device__ __forceinline__ Quad quad_global(const TileCtx& C, int e, int k) {
+    Quad q;
+    if (k < 0 || k >= C.n_ls) {
+        q.a = q.b = make_float2(0.f, 0.f);
+        return q;
+    }
+    const long long i = (long long)(k + C.pad) * C.pitch + e;
+    if (C.qdt) {
+        const uint32_t* g = static_cast<const uint32_t*>(C.gband) + i;
+        q.a = unpack_pair(__ldg(g), C.qdt);
+        q.b = unpack_pair(__ldg(g + 1), C.qdt);
+    } else {
+        const float2* g = static_cast<const float2*>(C.gband) + i;
+        q.a = __ldg(g);
+        q.b = __ldg(g + 1);
+    }
+    return q;
 }
 
-// Slab of a (tile, band) from 16-bit quads, by all threads of the CTA: node
-// rows klo .. klo + slab_w of cells cell0 .. cell0 + ncb, converted to FP32
-// (zero outside the template range and past the last cell, as TMA's fill
-// does for FP32 quads). Thread i fills slab entries i, i + T, ... (T threads,
-// entry e = row e / ncb, cell e % ncb): consecutive threads read consecutive
-// cells of a node row and store consecutive 16-byte entries; kFill loads are
-// in flight per thread before their stores. The caller synchronises the CTA
-// afterwards.
-__device__ __forceinline__ void fill_slab16(float4* __restrict__ slab, const TileCtx& C) {
+// Node k of a cell from the slab or, with use_slab false, from global memory.
+__device__ __forceinline__ Quad quad_at(const TileCtx& C, bool use_slab, int e, int k) {
+    return use_slab ? lds_quad(C.slab + (uint32_t)((k - C.klo) * C.pitch + e) * 8u, C) : quad_global(C, e, k);
+}
+
+// Slab of a (tile, band) by bulk copies (FP32): the band's entries are stored
+// contiguously, node rows padded with zero nodes on both sides, so the slab is
+// one contiguous range, taken in pieces. Issued by one thread; `bar` gets the
+// bytes. klo is a multiple of 4: 16-byte aligned.
+__device__ __forceinline__ void load_slab(const TileCtx& C, uint64_t* bar) {
+    const uint32_t bytes = (uint32_t)(C.slab_w * C.pitch) * 8u;
+    const char* src = static_cast<const char*>(C.gband) + (long long)(C.klo + C.pad) * C.pitch * 8;
+    fence_proxy_async_smem();
+    mbar_arrive_expect_tx(bar, bytes);
+    for (uint32_t o = 0; o < bytes; o += 16384u) bulk_load(C.slab + o, src + o, min(16384u, bytes - o), bar);
+}
+
+// Slab of a (tile, band) from 16-bit entries, by all threads of the CTA: the
+// same contiguous range read in 16-byte pieces (four entries), widened to
+// FP32; kFill loads are in flight per thread before their stores. The caller
+// synchronises the CTA afterwards.
+__device__ __forceinline__ void fill_slab16(const TileCtx& C) {
     constexpr int kFill = 4;
-    const int T = blockDim.x, total = C.slab_w * C.ncb;
-    const int dr = T / C.ncb, dc = T - dr * C.ncb;
-    int r = threadIdx.x / C.ncb, c = threadIdx.x - r * C.ncb;
-    for (int e0 = threadIdx.x; e0 < total; e0 += kFill * T) {
-        uint2 v[kFill];
-        bool ok[kFill];
+    const int T = blockDim.x, total = C.slab_w * C.pitch / 4;  // slab_w is a multiple of 4
+    const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint32_t*>(C.gband) +
+                                                      (long long)(C.klo + C.pad) * C.pitch);
+    for (int i0 = threadIdx.x; i0 < total; i0 += kFill * T) {
+        uint4 v[kFill];
+#pragma unroll
+        for (int u = 0; u < kFill; ++u) v[u] = i0 + u * T < total ? __ldg(src + i0 + u * T) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int u = 0; u < kFill; ++u) {
-            const int k = C.klo + r, cell = C.cell0 + c;
-            ok[u] = e0 + u * T < total && k >= 0 && k < C.n_ls && cell < C.n_cells;
-            v[u] = ok[u] ? __ldg(C.q16 + (long long)k * C.n_cells + cell) : make_uint2(0u, 0u);
-            r += dr;
-            c += dc;
-            if (c >= C.ncb) {
-                c -= C.ncb;
-                ++r;
+            const int i = i0 + u * T;
+            if (i < total) {
+                const float2 x = unpack_pair(v[u].x, C.qdt), y = unpack_pair(v[u].y, C.qdt);
+                const float2 z = unpack_pair(v[u].z, C.qdt), w = unpack_pair(v[u].w, C.qdt);
+                sts_f4(C.slab + (uint32_t)i * 32u, x.x, x.y, y.x, y.y);
+                sts_f4(C.slab + (uint32_t)i * 32u + 16u, z.x, z.y, w.x, w.y);
             }
-        }
-#pragma unroll
-        for (int u = 0; u < kFill; ++u) {
-            const int e = e0 + u * T;
-            if (e < total) slab[e] = ok[u] ? unpack_quad(v[u], C.qdt) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
 }
 
 // Mass-weighted bilinear template value at one node: sum_c w_c q_c.
-__device__ __forceinline__ float quad_dot(const float4 w, const float4 q) {
-    float2 p = __fmul2_rn(make_float2(w.x, w.y), make_float2(q.x, q.y));
-    p = __ffma2_rn(make_float2(w.z, w.w), make_float2(q.z, q.w), p);
+__device__ __forceinline__ float quad_dot(const float4 w, const Quad& q) {
+    float2 p = __fmul2_rn(make_float2(w.x, w.y), q.a);
+    p = __ffma2_rn(make_float2(w.z, w.w), q.b, p);
     return p.x + p.y;
+}
+
+// ----------------------------------------------------------------------------
+// Node positions of a particle's rounds without a chain from round to round.
+// Adding a value x in (-2^21, 2^21) to kMagic with rounding towards minus
+// infinity gives kMagic + floor(x) exactly, whose low mantissa bits are the
+// integer: one addition floors, and the address is one integer multiply-add of
+// those bits.
+// ----------------------------------------------------------------------------
+constexpr float kMagic = 12582912.f;          // 1.5 * 2^23
+constexpr uint32_t kMagicBits = 0x4b400000u;  // its bit pattern
+
+// Per-lane position of the rounds of kBins bins: bin j0 + kBins r + lane sits
+// at node K0 + il + r ib + x_r with x_r = x0 + r fb, where il = floor(lane
+// a_hi) and ib (the same for every particle) are integers, so that x_r stays
+// below a few and keeps FP32's absolute precision however wide the tile.
+struct LanePos {
+    float x0, fb;
+    uint32_t base;  // byte address of node K0 + il of the cell, less kMagicBits nodes
+    float nf;       // K0 + il - klo
+};
+__device__ __forceinline__ LanePos lane_pos(const TileCtx& C, float bins, float ib, int kw, int e, float f, float a_hi,
+                                            float a_lo, float lanef) {
+    LanePos L;
+    const float y = __fmaf_rd(lanef, a_hi, kMagic);
+    const float il = y - kMagic;
+    L.x0 = f + fmaf(lanef, a_lo, fmaf(lanef, a_hi, -il));
+    L.fb = fmaf(bins, a_lo, fmaf(bins, a_hi, -ib));
+    const int n = kw + (int)(__float_as_uint(y) - kMagicBits);
+    L.base = C.slab + ((uint32_t)n * (uint32_t)C.pitch + (uint32_t)e) * 8u - kMagicBits * ((uint32_t)C.pitch * 8u);
+    L.nf = (float)kw + il;
+    return L;
 }
 
 // first index i in [0, n] with v[i] > x  (v non-decreasing)
