@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
     C.err = P.err;
 #endif
     uint32_t phase = 0;
-    const float4* __restrict__ rec4 = reinterpret_cast<const float4*>(P.rec);
+    const float4* __restrict__ map4 = reinterpret_cast<const float4*>(P.map);
 
     for (long long t = lo / CT; t < P.n_tiles && t * CT < hi; ++t) {
         const long long a = max(lo - t * CT, 0ll), b = min(hi - t * CT, CT);
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
                         // and its tile slice of dL/dcube0 on its way to L2
                         if (live) {
                             asm volatile("prefetch.global.L1 [%0];" ::"l"(P.wu + qb));
-                            asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * qb + 1));
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(map4 + qb));
                             const float* gs = P.G0 + (long long)sp * P.n_lambda + C.j0;
                             const int nbin = min(P.tile_w + 1, P.n_lambda - C.j0);
 #pragma unroll 1
@@ -549,9 +549,9 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
                     for (int q = q0; q < q1; ++q) {
                         if (q + 1 < q1) {
                             asm volatile("prefetch.global.L1 [%0];" ::"l"(P.wu + q + 1));
-                            asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * (q + 1) + 1));
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(map4 + q + 1));
                         }
-                        const AdjSums S = adj_particle<R, KIND, MEAN, TW, NR>(P.wu[q], rec4[2 * q + 1], C, lane, lanef,
+                        const AdjSums S = adj_particle<R, KIND, MEAN, TW, NR>(P.wu[q], map4[q], C, lane, lanef,
                                                                               G, grow, P.ls0_over);
                         // the four sums over the warp with 6 shuffles: halves of the
                         // warp trade pairs, quarters trade singles, then a butterfly

@@ -352,7 +352,7 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
     static_cast<SlabParams&>(T) = S.geo;
     T.pair = S.d_pair_adj;
     T.qdt = 0;
-    T.rec = P.d_rec;
+    T.map = P.d_map;
     T.wu = P.d_wu;
     T.items = P.d_items;
     T.item_off = P.d_item_off;

@@ -168,19 +168,39 @@ __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
 // ----------------------------------------------------------------------------
 // Work descriptors
 // ----------------------------------------------------------------------------
-// Per in-field particle, in sorted order: everything the deposit needs (32 B).
-// Spectrum value at output bin j:  sum_c w[c] * lerp(T_c, t(j)), with the
-// fractional SSP node position t(j) = bi + bf + j*(a_hi + a_lo). a_hi keeps 11
-// significant bits, so j*a_hi is exact in FP32 for j < 2^13 and only the small
-// term j*a_lo is rounded.
+// Per in-field particle, in sorted order: everything the deposit's fast rounds
+// need (32 B). With t(j) = tau(j) + s(j), tau the node position of bin j for a
+// particle at rest, s(j) = s0 + (j - jc) g is the particle's Doppler shift in
+// nodes, in fixed point: s0 in units of 2^-fb nodes, g of 2^-(fb + 13)
+// (SlabParams::fb, jc), so that a tile's first node and fraction are one
+// multiply-high and an addition to the tile's constant.
 struct __align__(16) DepRec {
     float w[4];        // mass * flux_scale * bilinear weights: (ia,iz) (ia+1,iz) (ia,iz+1) (ia+1,iz+1)
-    int c0_bi;         // (SSP cell ia * n_Z + iz) << 16 | (floor(t(0)) & 0xffff)
-    float bf;          // t(0) - floor(t(0)), in [0, 1)
-    float a_hi;        // dt/dj, high part
-    float a_lo;        // dt/dj, low part
+    int s0;            // s(jc)
+    int g;             // ds/dj
+    float d;           // kind 0: 1 - dt/dj; kinds 1, 2: dt/dj less that of a particle at rest
+    unsigned ef;       // 8 * (entry of the cell within its band) | RecPath << 30
 };
 static_assert(sizeof(DepRec) == 32, "DepRec layout");
+
+// Which rounds a particle takes in every tile: the kind's own, the two-read
+// rounds (centres) or two-read edges (means), or the per-bin path.
+enum RecPath : unsigned { kPathMain = 0u, kPathTwoRead = 1u, kPathBins = 2u };
+
+// Smallest 1 - dt/dj of the kind-1 rounds (deposit_kernel.cuh).
+constexpr float kShuffleTol = 1e-5f;
+
+// The full affine map of the same particle (16 B), for the per-bin path and the
+// adjoint: bin j at fractional SSP node position t(j) = bi + bf + j*(a_hi +
+// a_lo). a_hi keeps 11 significant bits, so j*a_hi is exact in FP32 for
+// j < 2^13 and only the small term j*a_lo is rounded.
+struct __align__(16) MapRec {
+    int c0_bi;         // (SSP cell ia * n_Z + iz) << 16 | (floor(t(0)) & 0xffff)
+    float bf;          // t(0) - floor(t(0)), in [0, 1)
+    float a_hi;        // dt/dj, high part (0: the spectrum misses every output bin)
+    float a_lo;        // dt/dj, low part
+};
+static_assert(sizeof(MapRec) == 16, "MapRec layout");
 
 __device__ __forceinline__ int rec_c0(int c0_bi) { return (int)((unsigned)c0_bi >> 16); }
 __device__ __forceinline__ int rec_bi(int c0_bi) { return (c0_bi << 16) >> 16; }

@@ -160,18 +160,17 @@ __device__ __forceinline__ void rounds_near1(const float4 w4, const TileCtx& C, 
     }
 }
 
-// Kind 1 (A in [1/2, 1 - kTol1)) and the two-read rounds (any A): lane l reads
+// Kind 1 (A in [1/2, 1 - kShuffleTol)) and the two-read rounds (any A): lane l reads
 // its bin's node n_l. In kind 1 the next node is lane l + 1's, or lane l + 2's
 // when lane l + 1 has the same node (phi_l + A < 1). Near that limit (within
-// the rounding of phi, kTol1 / 2) lane l + 2 holds node n_l + 1 in either case,
-// since 1 - A > kTol1.
-constexpr float kTol1 = 1e-5f;
+// the rounding of phi, kShuffleTol / 2) lane l + 2 holds node n_l + 1 in either case,
+// since 1 - A > kShuffleTol.
 template <int R, int B, bool SHUFFLE>
 __device__ __forceinline__ void rounds_phi(const float4 w4, const TileCtx& C, const LanePos& L, float ib, float delta,
                                            int lane, float (&acc)[R]) {
     const uint32_t p8 = (uint32_t)C.pitch * 8u;
     const uint32_t sib = (uint32_t)(int)ib * p8;
-    const float dt = -(delta + 0.5f * kTol1);
+    const float dt = -(delta + 0.5f * kShuffleTol);
     uint32_t base = L.base;
 #pragma unroll
     for (int r = 0; r < R; r += 2) {
@@ -328,33 +327,51 @@ __device__ __forceinline__ void mean_rounds_phi(const float4 w4, const TileCtx& 
     }
 }
 
+// What the rounds of a (tile, job) share: the tile's first bin at rest in the
+// records' fixed point (SlabParams::tile_ref), and the lane's constants.
+struct RoundCtx {
+    int jrel;            // (j0 - jc) << 19: times DepRec::g, high word = the shift since jc
+    uint32_t ref;
+    int fb;
+    float fscale;        // 2^-fb
+    float a0_1m;
+    float ib, fbr;       // whole nodes of a round and the rest, at rest
+    float il, fl;        // whole nodes of the lane's bins and the rest, at rest
+};
+
 // Adds one particle's spectrum to acc (setup by every lane; warp-uniform path).
 template <int R, int KIND, bool MEAN, int NR>
-__device__ __forceinline__ void deposit_particle(const float4 w4, const float4 g4, const TileCtx& C, float ib,
-                                                 int lane, float lanef, float (&acc)[NR],
-                                                 unsigned long long* slow_count) {
+__device__ __forceinline__ void deposit_particle(const float4 w4, const float4 r4, const float4* __restrict__ map4,
+                                                 const TileCtx& C, const RoundCtx& T, int lane, float lanef,
+                                                 float (&acc)[NR], unsigned long long* slow_count) {
     constexpr int B = kind_bins(KIND), BR = MEAN ? B - 1 : B;
-    const int c0_bi = __float_as_int(g4.x);
-    float f;
-    const int kw = node_pos(C.j0, rec_bi(c0_bi), g4.y, g4.z, g4.w, f) - C.klo;  // the tile's first bin
-    const float delta = (1.f - g4.z) - g4.w;                                   // 1 - dt/dj (one rounding)
-    const float A = g4.z + g4.w;
-    const int e = rec_entry(c0_bi, C);
-    const bool fits = A <= C.a_max && (unsigned)kw < (unsigned)(C.slab_w - C.need) &&
-                      (unsigned)e < (unsigned)(C.pitch - 1);
-    if (KIND == 0 && fits && delta >= 0.f && delta * 31.f < 1.f) {
-        const uint32_t base = C.slab + ((uint32_t)(kw + lane) * (uint32_t)C.pitch + (uint32_t)e) * 8u;
-        if constexpr (MEAN) mean_rounds_near1<R>(w4, C, base, f, delta, lane, lanef, acc);
-        else rounds_near1<R>(w4, C, base, f, delta, lane, lanef, acc);
-    } else if (fits && (!MEAN || (A >= 0.5f && A < 1.999f)) && A > 0.f) {
-        const LanePos L = lane_pos(C, (float)BR, ib, kw, e, f, g4.z, g4.w, lanef);
-        if constexpr (MEAN) mean_rounds_phi<R, B>(w4, C, L, ib, A, lane, acc);
-        else {
-            if (KIND == 1 && A >= 0.5f && delta > kTol1) rounds_phi<R, B, true>(w4, C, L, ib, delta, lane, acc);
-            else rounds_phi<R, B, false>(w4, C, L, ib, delta, lane, acc);
+    const unsigned ef = __float_as_uint(r4.w);
+    const uint32_t p = (uint32_t)(__mulhi(T.jrel, __float_as_int(r4.y)) + __float_as_int(r4.x)) + T.ref;
+    const uint32_t p8 = (uint32_t)C.pitch * 8u;
+    const uint32_t kw = p >> T.fb;  // first node, from the slab's
+    const float f = (float)(p & ((1u << T.fb) - 1u)) * T.fscale;
+    if ((ef >> 30) == kPathMain && KIND == 0) {
+        const uint32_t base = C.slab + (kw + (uint32_t)lane) * p8 + ef;
+        if constexpr (MEAN) mean_rounds_near1<R>(w4, C, base, f, r4.z, lane, lanef, acc);
+        else rounds_near1<R>(w4, C, base, f, r4.z, lane, lanef, acc);
+    } else if ((ef >> 30) != kPathBins) {
+        const float da = KIND == 0 ? T.a0_1m - r4.z : r4.z;  // dt/dj less that at rest
+        LanePos L;
+        L.x0 = fmaf(lanef, da, f + T.fl);
+        L.fb = fmaf((float)BR, da, T.fbr);
+        L.base = C.slab + (kw + (uint32_t)(int)T.il) * p8 + (ef & 0x3fffffffu) - kMagicBits * p8;
+        const float delta = T.a0_1m - da;
+        if constexpr (MEAN) {
+            L.nf = (float)kw + T.il;
+            mean_rounds_phi<R, B>(w4, C, L, T.ib, 1.f - delta, lane, acc);
+        } else {
+            if (KIND == 1 && (ef >> 30) == kPathMain) rounds_phi<R, B, true>(w4, C, L, T.ib, delta, lane, acc);
+            else rounds_phi<R, B, false>(w4, C, L, T.ib, delta, lane, acc);
         }
-    } else if (g4.z > 0.f) {  // a_hi = 0 marks a spectrum that misses every bin
-        general_particle<NR, BR, MEAN ? R : B, MEAN>(w4, g4, C, lane, acc, slow_count);
+    } else {
+        const float4 g4 = *map4;
+        if (g4.z > 0.f)  // a_hi = 0 marks a spectrum that misses every bin
+            general_particle<NR, BR, MEAN ? R : B, MEAN>(w4, g4, C, lane, acc, slow_count);
     }
 }
 
@@ -364,34 +381,46 @@ constexpr int kJobChunk = 32;  // jobs per shared-memory work table
 // registers in sorted order onto the item's row dst (zero for band 0, the
 // earlier bands' sum for later bands), then stored.
 template <int R, int KIND, bool MEAN>
-__device__ __forceinline__ void deposit_item(const DepositParams& P, const TileCtx& C, const float4* __restrict__ rec4,
-                                             int q0, int q1, float* dst, int band, int lane, float lanef) {
+__device__ __forceinline__ void deposit_item(const DepositParams& P, const TileCtx& C, const DepJob& J, int t, int q0,
+                                             int q1, float* dst, int band, int lane, float lanef, float2 lref) {
     constexpr int B = kind_bins(KIND), BR = MEAN ? B - 1 : B, NR = MEAN ? R + 1 : R;
+    const float4* __restrict__ rec4 = reinterpret_cast<const float4*>(J.rec);
+    // the next particle's record is pulled into L1 while the current one is
+    // deposited (no registers held across the particle)
+    if (q0 < q1) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * q0));
     float acc[NR];
     // band 0 starts the row from zero; later bands continue the row the
     // earlier bands left (loaded now, in flight while the first particle's
     // record and setup are prepared), so the row is written back with plain
     // stores and no atomics
+    const bool full = C.j0 + B * R <= P.n_lambda;
+    dst += C.j0 + lane;
+    const int left = full ? 1 << 20 : P.n_lambda - C.j0 - lane;  // bins from the lane's first to the row's end
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-        const int j = C.j0 + BR * r + lane;
         const bool owned = lane < (MEAN && r == R ? R : BR);
-        acc[r] = (band > 0 && owned && j < P.n_lambda) ? dst[j] : 0.f;
+        acc[r] = (band > 0 && owned && BR * r < left) ? dst[BR * r] : 0.f;
     }
-    const float ib = MEAN ? P.ib_mean : P.ib;
-    // the next particle's record is pulled into L1 while the current one is
-    // deposited (no registers held across the particle)
-    if (q0 < q1) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * q0));
+    RoundCtx T;
+    T.jrel = (int)((unsigned)(C.j0 - P.jc) << 19);
+    T.ref = P.tile_ref[(MEAN ? P.n_tiles : 0) + t];
+    T.fb = P.fb;
+    T.fscale = __int_as_float((127 - P.fb) << 23);
+    T.a0_1m = P.a0_1m;
+    T.ib = P.ib[MEAN];
+    T.fbr = P.fbr[MEAN];
+    T.il = lref.x;
+    T.fl = lref.y;
     for (int q = q0; q < q1; ++q) {
         if (q + 1 < q1) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * (q + 1)));
-        const float4 w4 = rec4[2 * q], g4 = rec4[2 * q + 1];
-        deposit_particle<R, KIND, MEAN, NR>(w4, g4, C, ib, lane, lanef, acc, P.slow_count);
+        const float4 w4 = rec4[2 * q], r4 = rec4[2 * q + 1];
+        deposit_particle<R, KIND, MEAN, NR>(w4, r4, reinterpret_cast<const float4*>(J.map) + q, C, T, lane, lanef, acc,
+                                            P.slow_count);
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-        const int j = C.j0 + BR * r + lane;
         const bool owned = lane < (MEAN && r == R ? R : BR);
-        if (owned && j < P.n_lambda) dst[j] = acc[r];
+        if (owned && BR * r < left) dst[BR * r] = acc[r];
     }
 }
 
@@ -444,6 +473,7 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
     C.err = P.err;
 #endif
     uint32_t phase = 0;
+    const float2 lref = P.lane_ref[lane];
 
     for (long long t = lo / CT; t < P.n_tiles && t * CT < hi; ++t) {
         const long long a = max(lo - t * CT, 0ll), b = min(hi - t * CT, CT);
@@ -539,13 +569,12 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
                     const int s = __shfl_sync(0xffffffffu, sp, src);
                     const int pr = __shfl_sync(0xffffffffu, prow, src);
                     const DepJob& J = P.jobs[s_job[k]];
-                    const float4* __restrict__ rec4 = reinterpret_cast<const float4*>(J.rec);
                     float* dst = (pr < 0) ? J.cube + (long long)s * J.pitch
                                           : J.partials + (long long)pr * P.n_lambda;
                     if (MEANS && J.resample)
-                        deposit_item<R, KIND, true>(P, C, rec4, q0, q1, dst, band, lane, lanef);
+                        deposit_item<R, KIND, true>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref);
                     else
-                        deposit_item<R, KIND, false>(P, C, rec4, q0, q1, dst, band, lane, lanef);
+                        deposit_item<R, KIND, false>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref);
                 }
             }
         }

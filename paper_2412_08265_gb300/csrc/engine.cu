@@ -209,7 +209,7 @@ void ssp_state_destroy(SspState* S) {
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(S->device);
-    void* ptrs[] = {S->d_pair, S->d_pair_adj, S->d_la, S->d_lz, S->d_tile_klo, S->d_err, S->d_slow};
+    void* ptrs[] = {S->d_pair, S->d_pair_adj, S->d_la, S->d_lz, S->d_tile_klo, S->d_tile_ref, S->d_lane_ref, S->d_err, S->d_slow};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     cudaSetDevice(prev);
@@ -290,13 +290,15 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
         if (bands > kMaxBands) break;
         if (RUBIX_DEP_BANDS > 0 && bands != std::min(RUBIX_DEP_BANDS, ca)) continue;
         const int pitch = (apb * nzc) | 1;
-        const int slab_w = (int)std::min<long long>(budget / pitch, 1 << 14) / 4 * 4;
+        const int slab_max = (int)std::min<long long>(budget / pitch, 1 << 14) / 4 * 4;
         for (int r : rounds) {
             // bins of the last lane of the last round, deposit (also a mean
             // round more) and adjoint (rounds of 32 bins, of 31 edges for means)
             const int last = std::max({B * (r - 1) + 31, (B - 1) * r + r + 1, (B * r + 31) / 32 * 32 - 1});
             const int need = (int)std::ceil((last + 1) * std::max(a_hi, 1.0)) + 3;
-            if (need + 2 * shift + 8 > slab_w) continue;
+            if (need + 2 * shift + 8 > slab_max) continue;
+            // a slab twice the halo wide at most: more would only be staged
+            const int slab_w = std::min(slab_max, (need + 4 * shift + 11) / 4 * 4);
             const int n_tiles = (tel->n_lambda + B * r - 1) / (B * r);
             const double cost = n_tiles * (40.0 + 15.0 * r + 6.0 * bands);
             if (cost < best.cost) best = Geo{apb, bands, pitch, slab_w, r, need, cost};
@@ -317,24 +319,56 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
     G.n_ls = S.n_ls;
     G.es = S.n_Z > 1 ? 1 : 2;
     G.pad = G.slab_w + 8;
-    G.ib = (float)std::floor(B * A0 + 0.5);
-    G.ib_mean = (float)std::floor((B - 1) * A0 + 0.5);
+    for (int m = 0; m < 2; ++m) {
+        G.ib[m] = (float)std::floor((B - m) * A0 + 0.5);
+        G.fbr[m] = (float)((B - m) * A0 - G.ib[m]);
+    }
+    G.a0_1m = (float)(1.0 - A0);
+    // fixed point of the Doppler shifts: fb bits after the point, such that a
+    // position anywhere in a slab's margin fits 32 bits and the shift per bin
+    // (|g| <= A0 beta / (1 - beta), times 2^(fb + 13)) 31
+    G.fb = 26;
+    while (G.fb > 0 && ((G.slab_w - G.need + 4.0) * std::ldexp(1.0, G.fb) >= 4294967296.0 ||
+                        A0 * beta / (1.0 - beta) * std::ldexp(1.0, G.fb + 13) >= 2147483648.0))
+        --G.fb;
+    G.jc = tel->n_lambda > 4096 ? 4096 : 0;
     G.cost_c0 = RUBIX_DEP_COSTC0;
     for (int b = 0; b < kMaxBands; ++b) G.band_e0[b] = std::min(b * best.apb, ca - 1) * nzc;
     std::vector<int> klo(G.n_tiles, 0);
+    std::vector<unsigned> tref(2 * (size_t)G.n_tiles, 0u);
+    std::vector<float2> lref(32);
+    G.s_min = -1e30f;
+    G.s_max = 1e30f;
     for (int t = 0; t < G.n_tiles; ++t) {
         // nodes the tile's fast path reads: K0 .. K0 + need - 1 with K0 within
-        // +-shift of the zero-velocity position t00 of its first bin; slabs
-        // that would start beyond the templates' zero rows hold none of the
-        // tile's nodes
+        // +-shift of the zero-velocity position t00 of its first bin
         const int j0 = t * G.tile_w;
         const double t00 = ((tel->lambda0 + j0 * tel->dlambda) / (1.0 + tel->z_cosmo) - S.ls0) / S.dls;
         const double k = std::floor((t00 - shift - 1.0 - 0.5 * (G.slab_w - G.need - 2 * shift - 8)) / 4.0) * 4.0;
-        const double k_last = (S.n_ls + 3) / 4 * 4;
-        klo[t] = (int)std::max((double)-G.slab_w, std::min(k, k_last));
+        klo[t] = (int)std::max(-1e6, std::min(k, 1e6));
+        for (int m = 0; m < 2; ++m) {
+            const double c = t00 - 0.5 * A0 * m - klo[t];  // at rest, from the slab's first node
+            if (G.slab_w > 0 && std::abs(t00) < 9e5)
+                tref[(size_t)m * G.n_tiles + t] = (unsigned)std::llround(std::ldexp(c, G.fb));
+            else
+                G.s_max = -1e30f;  // no slab, or bins absurdly far from the templates: per-bin path
+            // a particle's first node K0 in [0, slab_w - need) for every tile
+            G.s_min = std::max(G.s_min, (float)(0.01 - c));
+            G.s_max = std::min(G.s_max, (float)(G.slab_w - G.need - 0.01 - c));
+        }
     }
-    if (dalloc_sync(&h->d_tile_klo, G.n_tiles)) return bail(fail(RUBIX_ERR_OOM, "tile alloc"));
+    for (int l = 0; l < 32; ++l) {
+        const double w = std::floor(l * A0);
+        lref[l] = make_float2((float)w, (float)(l * A0 - w));
+    }
+    if (dalloc_sync(&h->d_tile_klo, G.n_tiles) || dalloc_sync(&h->d_tile_ref, 2 * (size_t)G.n_tiles) ||
+        dalloc_sync(&h->d_lane_ref, 32))
+        return bail(fail(RUBIX_ERR_OOM, "tile alloc"));
     cudaMemcpy(h->d_tile_klo, klo.data(), klo.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(h->d_tile_ref, tref.data(), tref.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(h->d_lane_ref, lref.data(), 32 * sizeof(float2), cudaMemcpyHostToDevice);
+    G.tile_ref = h->d_tile_ref;
+    G.lane_ref = h->d_lane_ref;
     G.tile_klo = h->d_tile_klo;
     h->dep_smem = deposit_smem_bytes(G.pitch, G.slab_w);
     h->dep_ctas = h->n_sm;
@@ -458,6 +492,7 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_perm, 4 * N}, {(void**)&P->d_pin, 16 * N},
         {(void**)&P->d_sort_scratch, 4 * sort_scratch_ints((long long)N)},
         {(void**)&P->d_items, sizeof(Item) * (size_t)item_cap}, {(void**)&P->d_rec, sizeof(DepRec) * N},
+        {(void**)&P->d_map, sizeof(MapRec) * N},
         {(void**)&P->d_prec, sizeof(PartRec) * N},
         {(void**)&P->d_partials, 4 * (size_t)part_cap * n_lambda},
         {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.geo.n_bands + 2)}, {(void**)&P->d_n_items, 4 * ((size_t)n_s + 1)},
@@ -755,6 +790,14 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     SP.n_lambda = P.tel.n_lambda;
     SP.resample = P.tel.resample;
     SP.rec = P.d_rec;
+    SP.map = P.d_map;
+    SP.fb = S.geo.fb;
+    SP.jc = S.geo.jc;
+    SP.apb = S.apb;
+    SP.kind = S.geo.kind;
+    SP.a_max = S.geo.a_max;
+    SP.s_min = S.geo.s_min;
+    SP.s_max = S.geo.s_max;
     SP.prec = P.d_prec;
     SP.n_cap = P.cap;
     P.launches += launch_setup(SP, n, st);
@@ -782,6 +825,7 @@ float* deposit_target(const Plan& P, float* out, bool noise) { return (P.need_co
 DepJob plan_job(const Plan& P, float* target) {
     DepJob J{};
     J.rec = P.d_rec;
+    J.map = P.d_map;
     J.items = P.d_items;
     J.item_off = P.d_item_off;
     J.seg_off = P.d_seg_off;

@@ -46,6 +46,8 @@ struct SspState {
     int apb = 1;                // age cells per band
     size_t dep_smem = 0;
     int* d_tile_klo = nullptr;
+    unsigned* d_tile_ref = nullptr;
+    float2* d_lane_ref = nullptr;
     int dep_ctas = 0, dep_threads = RUBIX_DEP_THREADS, chunk = RUBIX_DEP_CHUNK;
     unsigned* d_err = nullptr;              // device error word (kernel bit flags)
     unsigned long long* d_slow = nullptr;   // (particle, tile) pairs on the global-memory path
@@ -103,6 +105,7 @@ struct Plan {
     int *d_part_off = nullptr, *d_scan_scratch = nullptr;
     Item* d_items = nullptr;
     DepRec* d_rec = nullptr;
+    MapRec* d_map = nullptr;
     PartRec* d_prec = nullptr;
     float* d_partials = nullptr;
     float *d_cube0 = nullptr, *d_tmp = nullptr, *d_out = nullptr;

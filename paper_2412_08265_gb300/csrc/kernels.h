@@ -9,6 +9,7 @@
 namespace rubix {
 
 struct DepRec;
+struct MapRec;
 struct PartRec;
 struct Item;
 
@@ -111,6 +112,10 @@ struct SetupParams {
     int n_lambda;
     int resample;            // 0: records map bin centres, 1: bin lower edges (bin means)
     DepRec* rec;             // [n_in]
+    MapRec* map;             // [n_in]
+    // the deposit's geometry: fixed-point shifts, band entries, path limits
+    int fb, jc, apb, kind;
+    float a_max, s_min, s_max;
     PartRec* prec;           // [n_in]
     long long n_cap;         // capacity of rec / prec
 };
@@ -137,6 +142,7 @@ constexpr int kMaxJobs = 64;
 constexpr int kDepHeader = 1024;  // deposit shared-memory header (barrier, counters, job table)
 struct DepJob {
     const DepRec* rec;
+    const MapRec* map;
     const Item* items;
     const int* item_off;     // [n_s + 1]: total items at [n_s]
     const int* seg_off;      // [n_s * n_bands + 2]: in-field particles at [n_s * n_bands]
@@ -165,10 +171,20 @@ struct SlabParams {
     int tile_w;                 // output bins per tile = rounds x kind_bins(kind)
     int n_tiles;
     const int* tile_klo;        // [n_tiles] first SSP node of each tile's slab (a multiple of 4)
+    // [2][n_tiles] node position of each tile's first bin (bin centres, then
+    // lower edges) for a particle at rest, from the slab's first node, in units
+    // of 2^-fb nodes
+    const unsigned* tile_ref;
+    int fb, jc;                 // fixed point of the records' shifts (DepRec)
+    float a0_1m;                // 1 - dt/dj of a particle at rest
+    float s_min, s_max;         // shifts (nodes) whose rounds stay in every tile's slab
     int slab_w;                 // nodes per slab (0 = no slab: global path only)
     float a_max;                // largest dt/dj of the fast rounds, and
     int need;                   // the nodes they read from a particle's first
-    float ib, ib_mean;  // whole nodes per round (LanePos::base steps)
+    // per round of centres and of means: whole nodes, and the rest, for a
+    // particle at rest
+    float ib[2], fbr[2];
+    const float2* lane_ref;     // [32] lane * dt/dj at rest: whole nodes, rest
     int cost_c0;                // per-item cost in particle units
     unsigned* err;
 };
@@ -239,7 +255,7 @@ struct AdjointParams {
 //   part = (sum_j G S, sum_j G dS/dta', sum_j G dS/dtz', sum_j G dS/dt * t_abs)
 // over the tile's bins (unit mass), from the same shared-memory quad slabs.
 struct AdjTileParams : SlabParams {
-    const DepRec* rec;          // [n_in] forward records (sorted order)
+    const MapRec* map;          // [n_in] the forward's maps (sorted order)
     const float2* wu;           // [n_in] position (ta, tz) in the SSP cell
     const Item* items;
     const int* item_off;        // [n_s + 1]

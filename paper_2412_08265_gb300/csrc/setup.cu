@@ -53,6 +53,13 @@ __device__ __forceinline__ DF df_mul_f(DF a, float b) {
     return df_norm(p, fmaf(a.lo, b, e));
 }
 
+// x * scale (a power of two) rounded to an integer; saturates.
+__device__ __forceinline__ int df_fixed(DF x, float scale) {
+    const float v = x.hi * scale;  // exact
+    const int i = __float2int_rn(v);
+    return i + __float2int_rn(__fadd_rn(v - (float)i, x.lo * scale));
+}
+
 // ----------------------------------------------------------------------------
 // K3: per-particle setup (sorted order).
 // ----------------------------------------------------------------------------
@@ -69,6 +76,11 @@ __global__ void k_setup(SetupParams P) {
     // double-float from the FP64 constants below (converted once per thread).
     const DF Az = df_of(P.dl * P.alpha_z), L = df_of(P.l0 * P.alpha_z);
     const DF Bz = df_of(fma(P.l0, P.alpha_z, -P.ls0_dls)), invc = df_of(P.inv_c);
+    // the shift s(j) = -g (L' + j A_z) of DepRec at j = jc, L' = L (bin centres)
+    // or L - A_z / 2 (edges), and its step -g A_z
+    const DF Ls = df_of(P.l0 * P.alpha_z + ((double)P.jc - (P.resample ? 0.5 : 0.0)) * (P.dl * P.alpha_z));
+    const float sc = __int_as_float((127 + P.fb) << 23), scg = __int_as_float((127 + P.fb + 13) << 23);
+    const int nzc = max(P.ssp.n_Z, 2);
     const float t_lastj = (float)(P.resample ? P.n_lambda : P.n_lambda - 1);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_in;
          i += (long long)gridDim.x * blockDim.x) {
@@ -80,6 +92,7 @@ __global__ void k_setup(SetupParams P) {
         ssp_cell(log10f(Z), P.ssp.lz_nodes, P.ssp.n_Z, iz, tz, dtz);
         const float ms = (float)P.flux_scale * m;
         DepRec r;
+        MapRec mr;
         r.w[0] = ms * ((1.f - ta) * (1.f - tz));
         r.w[1] = ms * (ta * (1.f - tz));
         r.w[2] = ms * ((1.f - ta) * tz);
@@ -114,10 +127,26 @@ __global__ void k_setup(SetupParams P) {
             a_hi = __uint_as_float(__float_as_uint(A.hi) & ~((1u << 13) - 1u));
             a_lo = __fadd_rn(__fsub_rn(A.hi, a_hi), A.lo);
         }
-        r.c0_bi = (c0 << 16) | (bi & 0xffff);
-        r.bf = bf;
-        r.a_hi = a_hi;
-        r.a_lo = a_lo;
+        mr.c0_bi = (c0 << 16) | (bi & 0xffff);
+        mr.bf = bf;
+        mr.a_hi = a_hi;
+        mr.a_lo = a_lo;
+        // Doppler shift in fixed point, and which rounds the particle takes
+        const DF S = df_neg(df_mul(Ls, g)), D = df_neg(df_mul(Az, g));
+        r.s0 = df_fixed(S, sc);
+        r.g = df_fixed(D, scg);
+        const float Af = a_hi + a_lo, delta = (1.f - a_hi) - a_lo;
+        r.d = P.kind == 0 ? delta : D.hi;
+        const float s_a = fmaf(-(float)P.jc, D.hi, S.hi), s_b = fmaf((float)(P.n_lambda - P.jc), D.hi, S.hi);
+        const bool fits = Af > 0.f && Af <= P.a_max && fabsf(D.hi * scg) < 2147483000.f && fminf(s_a, s_b) >= P.s_min && fmaxf(s_a, s_b) <= P.s_max;
+        const bool edges = Af >= 0.5f && Af < 1.999f;  // two-read edges (bin means)
+        unsigned path = kPathBins;
+        if (fits && P.kind == 0 && delta >= 0.f && delta * 31.f < 1.f) path = kPathMain;
+        else if (fits && P.resample) path = !edges ? kPathBins : (P.kind == 0 ? kPathTwoRead : kPathMain);
+        else if (fits) path = P.kind == 2 || (P.kind == 1 && Af >= 0.5f && delta > kShuffleTol) ? kPathMain : kPathTwoRead;
+        const int e = path == kPathBins ? 0 : (ia - age_band(ia, P.apb, P.n_bands) * P.apb) * nzc + iz;
+        r.ef = (unsigned)(8 * e) | (path << 30);
+        P.map[i] = mr;
         P.rec[i] = r;
         P.prec[i] = pr;
     }

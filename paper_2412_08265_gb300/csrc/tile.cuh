@@ -47,8 +47,8 @@ struct TileCtx {
     uint32_t slab;         // shared-space address of the slab
     const void* gband;     // this band's entries in global memory (FP32 float2 or 16-bit uint32_t)
     int qdt;               // 0: FP32, 1: BF16, 2: FP16
-    float a_max;           // largest dt/dj whose rounds stay within `need` nodes
-    int need;              // nodes the rounds of one particle can read, from its first
+    float a_max;           // largest dt/dj whose rounds stay within `need` nodes (adjoint)
+    int need;              // nodes the rounds of one particle can read, from its first (adjoint)
 #if RUBIX_DEBUG
     unsigned* err;         // error word for the debug build's index checks
 #endif
@@ -115,13 +115,19 @@ __device__ __forceinline__ Quad quad_at(const TileCtx& C, bool use_slab, int e, 
     return use_slab ? lds_quad(C.slab + (uint32_t)((k - C.klo) * C.pitch + e) * 8u, C) : quad_global(C, e, k);
 }
 
+// First row of a slab in the band's padded array. A slab that lies outside the
+// templates altogether is zero wherever it is read from.
+__device__ __forceinline__ int slab_row(const TileCtx& C) {
+    return max(-C.slab_w, min(C.klo, (C.n_ls + 3) / 4 * 4)) + C.pad;
+}
+
 // Slab of a (tile, band) by bulk copies (FP32): the band's entries are stored
 // contiguously, node rows padded with zero nodes on both sides, so the slab is
 // one contiguous range, taken in pieces. Issued by one thread; `bar` gets the
 // bytes. klo is a multiple of 4: 16-byte aligned.
 __device__ __forceinline__ void load_slab(const TileCtx& C, uint64_t* bar) {
     const uint32_t bytes = (uint32_t)(C.slab_w * C.pitch) * 8u;
-    const char* src = static_cast<const char*>(C.gband) + (long long)(C.klo + C.pad) * C.pitch * 8;
+    const char* src = static_cast<const char*>(C.gband) + (long long)slab_row(C) * C.pitch * 8;
     fence_proxy_async_smem();
     mbar_arrive_expect_tx(bar, bytes);
     for (uint32_t o = 0; o < bytes; o += 16384u) bulk_load(C.slab + o, src + o, min(16384u, bytes - o), bar);
@@ -135,7 +141,7 @@ __device__ __forceinline__ void fill_slab16(const TileCtx& C) {
     constexpr int kFill = 4;
     const int T = blockDim.x, total = C.slab_w * C.pitch / 4;  // slab_w is a multiple of 4
     const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint32_t*>(C.gband) +
-                                                      (long long)(C.klo + C.pad) * C.pitch);
+                                                      (long long)slab_row(C) * C.pitch);
     for (int i0 = threadIdx.x; i0 < total; i0 += kFill * T) {
         uint4 v[kFill];
 #pragma unroll
@@ -171,26 +177,15 @@ constexpr float kMagic = 12582912.f;          // 1.5 * 2^23
 constexpr uint32_t kMagicBits = 0x4b400000u;  // its bit pattern
 
 // Per-lane position of the rounds of kBins bins: bin j0 + kBins r + lane sits
-// at node K0 + il + r ib + x_r with x_r = x0 + r fb, where il = floor(lane
-// a_hi) and ib (the same for every particle) are integers, so that x_r stays
-// below a few and keeps FP32's absolute precision however wide the tile.
+// at node K0 + il + r ib + x_r with x_r = x0 + r fb, where il and ib are the
+// whole nodes of lane (kBins) bins at rest, the same for every particle, so
+// that x_r stays below a few and keeps FP32's absolute precision however wide
+// the tile.
 struct LanePos {
     float x0, fb;
     uint32_t base;  // byte address of node K0 + il of the cell, less kMagicBits nodes
     float nf;       // K0 + il - klo
 };
-__device__ __forceinline__ LanePos lane_pos(const TileCtx& C, float bins, float ib, int kw, int e, float f, float a_hi,
-                                            float a_lo, float lanef) {
-    LanePos L;
-    const float y = __fmaf_rd(lanef, a_hi, kMagic);
-    const float il = y - kMagic;
-    L.x0 = f + fmaf(lanef, a_lo, fmaf(lanef, a_hi, -il));
-    L.fb = fmaf(bins, a_lo, fmaf(bins, a_hi, -ib));
-    const int n = kw + (int)(__float_as_uint(y) - kMagicBits);
-    L.base = C.slab + ((uint32_t)n * (uint32_t)C.pitch + (uint32_t)e) * 8u - kMagicBits * ((uint32_t)C.pitch * 8u);
-    L.nf = (float)kw + il;
-    return L;
-}
 
 // first index i in [0, n] with v[i] > x  (v non-decreasing)
 __device__ __forceinline__ int upper_bound_ll(const long long* __restrict__ v, int n, long long x) {
