@@ -261,21 +261,15 @@ extern "C" rubix_status rubix_convolve(const rubix_telescope* tel, const float* 
         CK(cudaMemcpyAsync(cube_out, cube_in, bytes, cudaMemcpyDeviceToDevice, st));
         return RUBIX_OK;
     }
-    unsigned* d_err = nullptr;
     float* tmp = nullptr;
-    CK(cudaMallocAsync(reinterpret_cast<void**>(&d_err), 16, st));
-    CK(cudaMemsetAsync(d_err, 0, 16, st));
-    C.err = d_err;
     if (psf_lsf_needs_tmp(C.rp, C.rl)) {
         const cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), bytes, st);
         if (e != cudaSuccess) {
-            cudaFreeAsync(d_err, st);
             return fail(RUBIX_ERR_OOM, "rubix_convolve scratch: %s", cudaGetErrorString(e));
         }
     }
     const int l = launch_psf_lsf(C, cube_in, tel->n_lambda, nullptr, tmp, cube_out, st);
     if (tmp) cudaFreeAsync(tmp, st);
-    cudaFreeAsync(d_err, st);
     if (l < 0) return fail(RUBIX_ERR_CUDA, "PSF/LSF launch failed");
     CK(cudaGetLastError());
     return RUBIX_OK;
@@ -311,16 +305,7 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
         // the PSF and LSF kernels are symmetric: their adjoint is the same convolution
         ConvParams C = P.conv;
         C.noise_inv_s2n = 0.f;
-        int lc;
-        if (P.has_grad_map) {
-            // the gradient into pitched rows, then the TMA kernel, as in the forward
-            CK(cudaMemcpy2DAsync(P.d_tmp, (size_t)P.pitch0 * sizeof(float), dL_dcube,
-                                 (size_t)P.tel.n_lambda * sizeof(float), (size_t)P.tel.n_lambda * sizeof(float),
-                                 (size_t)P.n_s, cudaMemcpyDeviceToDevice, st));
-            lc = launch_psf_lsf(C, P.d_tmp, P.pitch0, &P.grad_map, nullptr, P.d_cube0, st);
-        } else {
-            lc = launch_psf_lsf(C, dL_dcube, P.tel.n_lambda, nullptr, P.d_tmp, P.d_cube0, st);
-        }
+        const int lc = launch_psf_lsf(C, dL_dcube, P.tel.n_lambda, nullptr, P.d_tmp, P.d_cube0, st);
         if (lc < 0) return fail(RUBIX_ERR_CUDA, "PSF/LSF transpose launch failed");
         G0 = P.d_cube0;
     }

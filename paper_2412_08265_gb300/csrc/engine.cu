@@ -503,10 +503,8 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_job_cost, 8 * (size_t)(kMaxJobs + 1)},
     };
     v.insert(v.end(), rest.begin(), rest.end());
-    // with gradients d_tmp also holds the loss gradient in pitched rows, so that
-    // the transposed PSF/LSF reads it through a TMA map like the forward
-    if (need_tmp || with_grad)
-        v.push_back({(void**)&P->d_tmp, with_grad ? (size_t)n_s * std::max(pitch0, n_lambda) * sizeof(float) : cube});
+    if (need_tmp) v.push_back({(void**)&P->d_tmp, cube});
+    v.push_back({(void**)&P->d_occ, (size_t)n_s});
     if (with_out) v.push_back({(void**)&P->d_out, cube});
     if (with_grad) {
         v.push_back({(void**)&P->d_contrib, 8 * kGlobal * N});
@@ -608,7 +606,6 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
     C.err = S->d_err;
     P->pitch0 = cube0_pitch(C.rp, C.rl, tel->n_lambda);
     P->has_conv_map = false;
-    P->has_grad_map = false;
     P->cap = std::max(n, 1ll);
     P->item_cap = (long long)P->n_s + P->cap / S->chunk + 2;
     P->part_cap = 2 * (P->cap / S->chunk) + 2;
@@ -632,7 +629,7 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
         P->bytes += round256(b.bytes);
     }
     unsigned box[2];
-    if (P->pitch0 != tel->n_lambda && conv_tma_box(C.rp, C.rl, box)) {
+    if (P->need_conv && conv_tma_box(C.rp, C.rl, box)) {
         // 3-D view of the pre-convolution cube: x = bin (n_lambda of each
         // pitched row), y = spaxel x, z = spaxel y; zero fill outside
         PFN_encodeTiled_t enc = get_encode_tiled();
@@ -652,17 +649,6 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
             return fail(RUBIX_ERR_CUDA, "cuTensorMapEncodeTiled (PSF/LSF) failed (%d)", (int)r);
         }
         P->has_conv_map = true;
-        if (with_grad && P->d_tmp) {
-            // the same view of d_tmp: the loss gradient, copied into pitched rows by the backward
-            r = enc(&P->grad_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, P->d_tmp, gdim, gstr, bx, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) {
-                plan_release(P);
-                return fail(RUBIX_ERR_CUDA, "cuTensorMapEncodeTiled (PSF/LSF gradient) failed (%d)", (int)r);
-            }
-            P->has_grad_map = true;
-        }
     }
     return RUBIX_OK;
 }
@@ -854,14 +840,18 @@ int enqueue_post(Plan& P, float* target, float* out, uint64_t noise_seed, float 
                  cudaEvent_t* ev) {
     NvtxRange nvtx("rubix: rows, PSF/LSF, noise");
     const int pitch = target == P.d_cube0 ? P.pitch0 : P.tel.n_lambda;
-    int l = launch_zero_empty(P.d_seg_off, P.n_s, P.S->geo.n_bands, target, pitch, P.tel.n_lambda, st);
+    const bool noise = noise_s2n > 0.f;
+    // the fused convolution does not read rows out of every particle's reach
+    unsigned char* occ = target == P.d_cube0 && P.has_conv_map ? P.d_occ : nullptr;
+    int l = launch_zero_empty(P.d_seg_off, P.tel.nx, P.rows, P.S->geo.n_bands, target, pitch, P.tel.n_lambda, occ,
+                              P.conv.rp, st);
     // d_n_parts (scanned into d_part_off by the item stage) is free here: the
     // combine's list of split spaxels
     l += launch_combine(P.d_part_off, P.n_s, P.tel.n_lambda, P.d_partials, target, pitch, P.d_n_parts, st);
     if (ev) cudaEventRecord(ev[4], st);
-    const bool noise = noise_s2n > 0.f;
     if (P.need_conv || noise) {
         ConvParams C = P.conv;
+        C.occ = occ;
         C.noise_inv_s2n = noise ? 1.0f / noise_s2n : 0.f;
         C.seed_lo = (uint32_t)noise_seed;
         C.seed_hi = (uint32_t)(noise_seed >> 32);

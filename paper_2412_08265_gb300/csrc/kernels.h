@@ -201,8 +201,11 @@ struct DepositParams : SlabParams {
 int launch_deposit(const DepositParams& P, int n_ctas, int threads, size_t smem, cudaStream_t st);
 size_t deposit_smem_bytes(int pitch, int slab_w);
 
-// Zero rows of the spaxels without particles (no work item covers them).
-int launch_zero_empty(const int* seg_off, int n_s, int nb, float* cube, int pitch, int n_lambda, cudaStream_t st);
+// Zero rows of the spaxels without particles (no work item covers them). With
+// occ ([ny][ceil(nx / kConvX)], written first: ConvParams::occ for radius rp),
+// only of those that an occupied block's columns reach.
+int launch_zero_empty(const int* seg_off, int nx, int ny, int nb, float* cube, int pitch, int n_lambda,
+                      unsigned char* occ, int rp, cudaStream_t st);
 
 // K5: combine partial rows of split spaxels in a fixed order: FP32 for at most
 // kCombineF32Rows rows, a compensated FP32 sum (two-sum) above. list: n_s + 1
@@ -220,16 +223,21 @@ struct ConvParams {
     float gl[2 * kMaxRadius + 1];
     float noise_inv_s2n;         // 0 = no noise
     uint32_t seed_lo, seed_hi;
-    unsigned* err;               // device error word (bounded waits of the TMA kernel)
+    unsigned* err;               // device error word (bounded waits of the fused kernel; nullable)
+    int ty;                      // output rows per CTA (set at launch)
+    // [ny][ceil(nx / kConvX)] (nullable): does row y hold anything within rp of
+    // block b's columns? Rows of blocks that do not are taken as zero, unread.
+    const unsigned char* occ;
 };
+constexpr int kConvX = 8;        // spaxels along x per fused CTA
 // `in` rows have stride in_pitch floats; `out` is dense ([ny][nx][n_lambda]).
 // in_map (nullable): a 3-D TMA map of `in` (x = wavelength over n_lambda, y = x
-// spaxel, z = y spaxel; zero fill outside) from conv_tma_map; with it the
-// instrument radii take the TMA kernel.
+// spaxel, z = y spaxel; zero fill outside) over a box of conv_tma_box; without
+// it `in` is dense, at any alignment.
 int launch_psf_lsf(const ConvParams& P, const float* in, int in_pitch, const CUtensorMap* in_map, float* tmp,
                    float* out, cudaStream_t st);
-// Box the TMA kernel loads for these radii: {wavelength, x}; false if the
-// radii have no TMA instantiation.
+// Box the fused kernel loads for these radii: {wavelength, x}; false if the
+// radii have no fused instantiation.
 bool conv_tma_box(int rp, int rl, unsigned box[2]);
 // True if launch_psf_lsf needs the intermediate cube `tmp` for these radii.
 bool psf_lsf_needs_tmp(int rp, int rl);

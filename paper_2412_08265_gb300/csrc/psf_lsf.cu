@@ -4,7 +4,7 @@
 //
 // The 3-D kernel is separable, g(dy) g(dx) h(dj), with zero padding on every
 // axis. For the radii of the instruments used here a single fused pass
-// (k_psf_lsf_fused, below) reads the cube once and writes it once. Other radii
+// (k_psf_lsf, below) reads the cube once and writes it once. Other radii
 // take two passes through an intermediate cube:
 //   pass 1 (k_lsf_psfx): one CTA per (wavelength chunk, x chunk, row y) loads
 //     the row segment with its halos into shared memory, applies the LSF along
@@ -58,6 +58,27 @@ __global__ void __launch_bounds__(256) k_lsf_psfx(const ConvParams P, const floa
     }
 }
 
+__device__ __forceinline__ float add_noise(float v, long long idx, float inv_s2n, uint32_t seed_lo, uint32_t seed_hi) {
+    U4 c;
+    c.x = (uint32_t)idx;
+    c.y = (uint32_t)((unsigned long long)idx >> 32);
+    c.z = 0u;
+    c.w = 0u;
+    const U4 r = philox4x32_10(c, seed_lo, seed_hi);
+    const float u1 = (float)((r.x >> 8) + 1u) * (1.0f / 16777216.0f);  // (0, 1]
+    const float u2 = (float)(r.y >> 8) * (1.0f / 16777216.0f);         // [0, 1)
+    const float z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+    return fmaf(fabsf(v) * inv_s2n, z, v);
+}
+
+// The same for 4 voxels, out of line: the fused kernel's unrolled rows would
+// hold 28 copies, and their length costs instruction fetches.
+__device__ __noinline__ float4 add_noise4(float4 v, long long idx, float inv_s2n, uint32_t seed_lo, uint32_t seed_hi) {
+    return make_float4(add_noise(v.x, idx, inv_s2n, seed_lo, seed_hi), add_noise(v.y, idx + 1, inv_s2n, seed_lo, seed_hi),
+                       add_noise(v.z, idx + 2, inv_s2n, seed_lo, seed_hi),
+                       add_noise(v.w, idx + 3, inv_s2n, seed_lo, seed_hi));
+}
+
 constexpr int kYC = 32;  // rows per thread in pass 2
 
 __global__ void __launch_bounds__(256) k_psfy_noise(const ConvParams P, const float* __restrict__ in,
@@ -76,244 +97,79 @@ __global__ void __launch_bounds__(256) k_psfy_noise(const ConvParams P, const fl
             acc = fmaf(P.gp[d + rp], in[(long long)yy * plane + col], acc);
         }
         const long long idx = (long long)y * plane + col;
-        if (P.noise_inv_s2n > 0.f) {
-            U4 c;
-            c.x = (uint32_t)idx;
-            c.y = (uint32_t)((unsigned long long)idx >> 32);
-            c.z = 0u;
-            c.w = 0u;
-            const U4 r = philox4x32_10(c, P.seed_lo, P.seed_hi);
-            const float u1 = (float)((r.x >> 8) + 1u) * (1.0f / 16777216.0f);   // (0, 1]
-            const float u2 = (float)(r.y >> 8) * (1.0f / 16777216.0f);          // [0, 1)
-            const float z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
-            acc = fmaf(fabsf(acc) * P.noise_inv_s2n, z, acc);
-        }
+        if (P.noise_inv_s2n > 0.f) acc = add_noise(acc, idx, P.noise_inv_s2n, P.seed_lo, P.seed_hi);
         out[idx] = acc;
     }
 }
 
 
 // ----------------------------------------------------------------------------
-// Fused single pass for the common radii (compile-time rp, rl): one CTA owns an
-// (x block of kFX spaxels, wavelength chunk of kFL = 32 bins, y band of kFY
-// rows) and streams the input rows of its band, plus rp halo rows, through a
-// cp.async pipeline (zero fill outside the cube). For each input row: PSF along
-// x into shared memory (each warp its own output columns, over the tile's
-// bins and the LSF halo; lanes run along wavelength), then LSF along
-// wavelength; the value of input row y_in is added, with weight
-// gp[m], to the register accumulator of output row y_in - rp + m (the 2 rp + 1
-// accumulators of each owned (x, wavelength) rotate with the row, the loop
-// being unrolled by 2 rp + 1 so their indices are static). After row y_in the
-// accumulator of output row y_in - rp is complete: noise is added and it is
-// written once. The cube is read once (plus halos) and written once.
-// ----------------------------------------------------------------------------
-#ifndef RUBIX_PSF_STAGES
-#define RUBIX_PSF_STAGES 3      // input rows in flight (cp.async pipeline depth)
-#endif
-#ifndef RUBIX_PSF_FX
-#define RUBIX_PSF_FX 32         // spaxels along x per CTA (a multiple of 8)
-#endif
-#ifndef RUBIX_PSF_FY
-#define RUBIX_PSF_FY 50         // output rows along y per CTA
-#endif
-constexpr int kFX = RUBIX_PSF_FX, kFL = 32, kFY = RUBIX_PSF_FY;  // kFL must equal the warp width
-constexpr int kFThreads = 256;
-constexpr int kFWarps = kFThreads / 32;
-constexpr int kFXW = kFX / kFWarps;          // output x rows owned by each warp
-constexpr int kFStages = RUBIX_PSF_STAGES;
-
-template <int RP, int RL>
-constexpr size_t fused_smem_bytes() {
-    return sizeof(float) * ((size_t)kFStages * (kFX + 2 * RP) * (kFL + 2 * RL) + (size_t)kFX * (kFL + 2 * RL));
-}
-
-__device__ __forceinline__ float add_noise(float v, long long idx, const ConvParams& P) {
-    U4 c;
-    c.x = (uint32_t)idx;
-    c.y = (uint32_t)((unsigned long long)idx >> 32);
-    c.z = 0u;
-    c.w = 0u;
-    const U4 r = philox4x32_10(c, P.seed_lo, P.seed_hi);
-    const float u1 = (float)((r.x >> 8) + 1u) * (1.0f / 16777216.0f);  // (0, 1]
-    const float u2 = (float)(r.y >> 8) * (1.0f / 16777216.0f);         // [0, 1)
-    const float z = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
-    return fmaf(fabsf(v) * P.noise_inv_s2n, z, v);
-}
-
-template <int RP, int RL>
-__global__ void __launch_bounds__(kFThreads) k_psf_lsf_fused(const ConvParams P, const float* __restrict__ in,
-                                                             float* __restrict__ out) {
-    constexpr int XW = kFX + 2 * RP, LW = kFL + 2 * RL, NR = 2 * RP + 1;
-    extern __shared__ float sm[];
-    float* s_in = sm;                        // [kFStages][XW][LW]
-    float* s_x = s_in + kFStages * XW * LW;  // [kFX][LW]   PSF-x output (row xo written and read by its warp)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j0 = blockIdx.x * kFL;
-    const int x0 = blockIdx.y * kFX;
-    const int y0 = blockIdx.z * kFY;
-    const int y1 = min(y0 + kFY, P.ny);
-    const int nx = P.nx, ny = P.ny, nl = P.n_lambda;
-    const int n_rows = (y1 - y0) + 2 * RP;   // input rows y0 - RP .. y1 + RP - 1
-    float gl[2 * RL + 1], gp[NR];
-#pragma unroll
-    for (int d = 0; d <= 2 * RL; ++d) gl[d] = P.gl[d];
-#pragma unroll
-    for (int d = 0; d < NR; ++d) gp[d] = P.gp[d];
-
-    auto load_row = [&](int i, int buf) {
-        const int y = y0 - RP + i;
-        float* dst = s_in + buf * XW * LW;
-        const bool yok = (y >= 0 && y < ny);
-        for (int xi = warp; xi < XW; xi += kFWarps) {
-            const int x = x0 - RP + xi;
-            const bool xok = yok && x >= 0 && x < nx;
-            const float* row = in + ((long long)(xok ? y : 0) * nx + (xok ? x : 0)) * nl;
-#pragma unroll
-            for (int l = lane; l < LW; l += 32) {
-                const int j = j0 - RL + l;
-                const bool ok = xok && j >= 0 && j < nl;
-                cp_async4(dst + xi * LW + l, ok ? row + j : in, ok);
-            }
-        }
-        cp_async_commit();
-    };
-
-    float acc[kFXW][NR];
-#pragma unroll
-    for (int k = 0; k < kFXW; ++k)
-#pragma unroll
-        for (int m = 0; m < NR; ++m) acc[k][m] = 0.f;
-
-    for (int k = 0; k < kFStages - 1; ++k) {
-        if (k < n_rows) load_row(k, k);
-        else cp_async_commit();
-    }
-    int buf = 0;
-    const int j = j0 + lane;
-    for (int ib = 0; ib < n_rows; ib += NR) {
-#pragma unroll
-        for (int ph = 0; ph < NR; ++ph) {   // input row i = ib + ph; accumulator of row y_in - RP + m is (ph + m) % NR
-            const int i = ib + ph;
-            if (i < n_rows) {
-                const int ahead = i + kFStages - 1;
-                int abuf = buf + kFStages - 1;
-                if (abuf >= kFStages) abuf -= kFStages;
-                if (ahead < n_rows) load_row(ahead, abuf);  // that buffer was read in iteration i - 1
-                else cp_async_commit();
-                cp_async_wait<kFStages - 1>();
-                __syncthreads();  // row i landed
-                const float* src = s_in + buf * XW * LW;
-                if (++buf == kFStages) buf = 0;
-#pragma unroll
-                for (int k = 0; k < kFXW; ++k) {
-                    const int xo = warp + k * kFWarps;
-                    for (int l = lane; l < LW; l += 32) {
-                        const float* c = src + xo * LW + l;
-                        float a = 0.f;
-#pragma unroll
-                        for (int d = 0; d < NR; ++d) a = fmaf(gp[d], c[d * LW], a);
-                        s_x[xo * LW + l] = a;
-                    }
-                }
-                __syncthreads();  // every warp is done with row i's input buffer
-                const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
-#pragma unroll
-                for (int k = 0; k < kFXW; ++k) {
-                    const int xi = warp + k * kFWarps;
-                    const float* r = s_x + xi * LW + lane;
-                    float v = 0.f;
-#pragma unroll
-                    for (int d = 0; d <= 2 * RL; ++d) v = fmaf(gl[d], r[d], v);
-#pragma unroll
-                    for (int m = 0; m < NR; ++m) acc[k][(ph + m) % NR] = fmaf(gp[m], v, acc[k][(ph + m) % NR]);
-                    // accumulator (ph + 0) % NR holds output row y_in - RP = y_done: complete
-                    float& done = acc[k][ph % NR];
-                    const int x = x0 + xi;
-                    if (y_done >= y0 && x < nx && j < nl) {
-                        const long long idx = ((long long)y_done * nx + x) * nl + j;
-                        out[idx] = (P.noise_inv_s2n > 0.f) ? add_noise(done, idx, P) : done;
-                    }
-                    done = 0.f;
-                }
-            }
-        }
-    }
-}
-
-template <int RP, int RL>
-static bool launch_fused(const ConvParams& P, const float* in, float* out, cudaStream_t st) {
-    constexpr size_t smem = fused_smem_bytes<RP, RL>();
-    static_assert(smem <= 200 * 1024, "fused PSF/LSF tile does not fit shared memory");
-    // per launch: the attribute belongs to the current device
-    if (cudaFuncSetAttribute(k_psf_lsf_fused<RP, RL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return false;
-    dim3 g((P.n_lambda + kFL - 1) / kFL, (P.nx + kFX - 1) / kFX, (P.ny + kFY - 1) / kFY);
-    k_psf_lsf_fused<RP, RL><<<g, kFThreads, smem, st>>>(P, in, out);
-    return true;
-}
-
-// Radii with a fused instantiation: the PSF of FWHM 1.5 spaxels (rp = 3) and
-// LSFs of sigma 1.2 A on 1.25 A or 3 A bins (rl = 4, 2), plus neighbours.
-#define RUBIX_FUSED_RADII(X) X(3, 4) X(3, 2) X(3, 0) X(0, 4) X(0, 2) X(2, 4) X(4, 4) X(3, 3) X(3, 5)
-
-static bool try_fused(const ConvParams& P, const float* in, float* out, cudaStream_t st) {
-#define RUBIX_FUSED_CASE(RP_, RL_) \
-    if (P.rp == RP_ && P.rl == RL_) return launch_fused<RP_, RL_>(P, in, out, st);
-    RUBIX_FUSED_RADII(RUBIX_FUSED_CASE)
-#undef RUBIX_FUSED_CASE
-    return false;
-}
-
-
-// ----------------------------------------------------------------------------
-// TMA variant of the fused pass for a cube whose rows are 16-byte aligned (the
-// deposit's own pitched cube). One CTA owns kTX = 8 spaxels along x (one per
-// warp) x kTY rows along y x kTL = kTB - 2 RLa bins. Each input row arrives
-// as one 3-D TMA box (kTB = 128 bins from j0 - RLa, spaxels x0 - rp ..
-// x0 + kTX + rp; zero fill outside the cube is the zero padding) in a
-// kTS-stage mbarrier ring. Warp w owns output column x0 + w and lane q the
-// box's bins 4q .. 4q + 3:
-//   PSF along x: the lane's 4 bins of column w from the box's columns
+// Fused single pass for the common radii (compile-time rp, rl): the cube is
+// read once (plus halos) and written once. One CTA owns kTX = 8 spaxels along
+// x (one per warp) x ty rows along y x kTL = kTB - 2 RLa bins. Each input row
+// (kTB = 128 bins from j0 - RLa, spaxels x0 - rp .. x0 + kTX + rp) arrives by
+// asynchronous copies in a kTS-stage mbarrier ring:
+//   pitched rows (the deposit's own cube, 16-byte rows): one 3-D TMA box, whose
+//     zero fill outside the cube is the zero padding;
+//   dense rows of any alignment (a caller's cube): one bulk copy per spaxel of
+//     the 16-byte granules that hold its bins (DenseRows).
+// Warp w owns output column x0 + w:
+//   PSF along x: the 4 bins per lane of column w from the box's columns
 //     w .. w + 2 rp, into the warp's own row of px (so every bin the LSF
 //     needs, halo included, is computed once, by the warp that reads it);
 //   LSF along wavelength from the warp's px row (lanes RLa/4 .. 31 - RLa/4,
-//     whose bins are the tile's), then the rotating PSF-y register
-//     accumulators.
+//     bins 4q .. 4q + 3 of lane q, which are the tile's), then the rotating
+//     PSF-y register accumulators: the value of input row y_in is added, with
+//     weight gp[m], to the accumulator of output row y_in - rp + m (2 rp + 1
+//     per owned bin, static indices by unrolling the rows), and the output row
+//     y_in - rp is then complete: noise is added and it is written once.
 // One CTA barrier per input row (every warp is done with the stage before it
-// is refilled); px is private to its warp. The terms of each output are
-// summed in the order of the cp.async kernel (PSF x, LSF, PSF y; each over
-// its taps in order), so the cube is bitwise the same.
+// is refilled); px is private to its warp. The terms of each output are summed
+// in the same order for both forms (PSF x, LSF, PSF y; each over its taps in
+// order), so they give the same bits.
+//
+// Bound by shared-memory loads and the barrier per row, at about half of the
+// copy bandwidth. The dense form replaced a kernel of 4-byte cp.async copies
+// (81 x 150 spaxels x 3721 bins: 0.32 ms).
 // ----------------------------------------------------------------------------
-#ifndef RUBIX_PSF_TY
-#define RUBIX_PSF_TY 150
-#endif
 #ifndef RUBIX_PSF_TSTAGES
 #define RUBIX_PSF_TSTAGES 4
 #endif
 #ifndef RUBIX_PSF_TMINB
 #define RUBIX_PSF_TMINB 4       // CTAs per SM the register budget is sized for
 #endif
-constexpr int kTB = 128, kTX = 8, kTThreads = 256, kTWarps = kTThreads / 32;
-constexpr int kTY = RUBIX_PSF_TY, kTS = RUBIX_PSF_TSTAGES;
+constexpr int kTB = 128, kTX = kConvX, kTThreads = 256, kTWarps = kTThreads / 32;
+constexpr int kTS = RUBIX_PSF_TSTAGES;
 static_assert(kTX == kTWarps, "one output column per warp");
+static_assert(kTS * 8 <= 32, "mbarriers before the row bits");
 
-template <int RP, int RL>
+template <int RP, int RL, bool DENSE = false>
 struct TmaGeo {
     static constexpr int RLa = (RL + 3) / 4 * 4;  // wavelength halo rounded up to 16 bytes
     static constexpr int LW = kTB;                // box: bins
     static constexpr int TL = kTB - 2 * RLa;      // output bins per tile
     static constexpr int XW = kTX + 2 * RP;       // box: spaxels along x
     static constexpr int NV = 1 + RLa / 2;        // 16-byte loads per lane for 4 LSF outputs
-    static constexpr int stage_floats = LW * XW;  // 512-byte rows: stages stay 128-byte aligned
+    static constexpr int row = LW + (DENSE ? 4 : 0);  // stage row: dense rows start anywhere in a 16-byte granule
+    static constexpr int stage_floats = (row * XW + 31) / 32 * 32;  // stages stay 128-byte aligned
     static constexpr size_t smem = 128 + (size_t)kTS * stage_floats * 4 + (size_t)kTX * kTB * 4;
 };
 
-template <int RP, int RL>
-__global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf_tma(const __grid_constant__ ConvParams P,
-                                                           const __grid_constant__ CUtensorMap in_map,
-                                                           float* __restrict__ out) {
-    using G = TmaGeo<RP, RL>;
+// Dense input rows: float cube [ny][nx][nl] at any 4-byte aligned address.
+// `al` is that address rounded down to 16 bytes, `off` (0..3) the floats
+// between; positions count floats from `al`. Copies take whole 16-byte granules
+// that hold at least one float of the cube, except the last, partial one (its
+// end may lie past the buffer): those floats are read and stored singly.
+struct DenseRows {
+    const float* al;
+    long long off, full;  // first position of the cube; end of its whole granules
+};
+
+template <int RP, int RL, bool DENSE, bool NOISE>
+__global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __grid_constant__ ConvParams P,
+                                                                       const __grid_constant__ CUtensorMap in_map,
+                                                                       const DenseRows D, float* __restrict__ out) {
+    using G = TmaGeo<RP, RL, DENSE>;
     constexpr int NR = 2 * RP + 1;
     constexpr int Q0 = G::RLa / 4, Q1 = 32 - G::RLa / 4;  // lanes whose bins are the tile's
     extern __shared__ __align__(1024) float smt[];
@@ -321,8 +177,8 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf_tma(cons
     float* stages = smt + 32;  // 128 bytes in
     float* px = stages + kTS * G::stage_floats;  // [kTX][kTB] PSF-x output, one row per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j0 = blockIdx.x * G::TL, x0 = blockIdx.y * kTX, y0 = blockIdx.z * kTY;
-    const int y1 = min(y0 + kTY, P.ny);
+    const int j0 = blockIdx.x * G::TL, x0 = blockIdx.y * kTX, y0 = blockIdx.z * P.ty;
+    const int y1 = min(y0 + P.ty, P.ny);
     const int nx = P.nx, nl = P.n_lambda;
     const int n_rows = (y1 - y0) + 2 * RP;  // input rows y0 - RP .. y1 + RP - 1
     float gl[2 * RL + 1], gp[NR];
@@ -331,18 +187,73 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf_tma(cons
 #pragma unroll
     for (int d = 0; d < NR; ++d) gp[d] = P.gp[d];
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kTS; ++s) mbar_init(&bars[s], 1);
+        // arrivals per phase: the one box, or each copied column's lane
+        const int n = DENSE ? min(x0 + kTX + RP, nx) - max(x0 - RP, 0) : 1;
+        for (int s = 0; s < kTS; ++s) mbar_init(&bars[s], n);
         fence_mbar_init();
     }
+    // which input rows hold anything for this CTA: rows outside the cube, or
+    // without a particle within reach of these columns, are zero
+    unsigned* s_live = reinterpret_cast<unsigned*>(smt) + 8;
+    for (int i0 = warp * 32; i0 < n_rows; i0 += kTThreads) {
+        const int y = y0 - RP + i0 + lane;
+        const bool on = i0 + lane < n_rows && y >= 0 && y < P.ny &&
+                        (!P.occ || P.occ[(long long)y * gridDim.y + blockIdx.y]);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (lane == 0) s_live[i0 >> 5] = m;
+    }
+    if constexpr (DENSE) {
+        // columns outside the cube are zero in every stage and never copied
+        for (int c = warp; c < G::XW; c += kTWarps)
+            if (x0 - RP + c < 0 || x0 - RP + c >= nx)
+                for (int k = lane; k < kTS * G::row; k += 32)
+                    stages[k / G::row * G::stage_floats + c * G::row + k % G::row] = 0.f;
+    }
     __syncthreads();
-    auto issue = [&](int i) {  // input row i into stage i % kTS (thread 0)
-        const int s = i % kTS;
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(&bars[s], (uint32_t)(G::LW * G::XW * 4));
-        tma_load_3d(stages + s * G::stage_floats, &in_map, &bars[s], j0 - G::RLa, x0 - RP, y0 - RP + i);
+    auto live = [&](int i) { return (s_live[i >> 5] >> (i & 31)) & 1u; };
+    // dense rows: the lane's spaxel column (warp 0), whose granules of bins
+    // [j_a, j_b) it copies
+    const bool copies = lane < G::XW && x0 - RP + lane >= 0 && x0 - RP + lane < nx;
+    const int j_a = max(j0 - G::RLa, 0), j_b = min(j0 - G::RLa + G::LW, nl);
+    const long long row_len = (long long)nx * nl;
+    const long long row0 = D.off + (long long)(y0 - RP) * row_len + (long long)(x0 - RP + lane) * nl;
+    auto issue = [&](int i, int s) {  // input row i into stage s (warp 0)
+        if constexpr (!DENSE) {
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                mbar_arrive_expect_tx(&bars[s], (uint32_t)(G::LW * G::XW * 4));
+                tma_load_3d(stages + s * G::stage_floats, &in_map, &bars[s], j0 - G::RLa, x0 - RP, y0 - RP + i);
+            }
+        } else {
+            // lane xi copies the granules of spaxel x0 - RP + xi's bins
+            if (copies) {
+                const long long row = row0 + i * row_len;
+                const long long a4 = (row + j_a) & ~3ll;
+                const uint32_t bytes = (uint32_t)max(min((row + j_b + 3) & ~3ll, D.full) - a4, 0ll) * 4u;
+                float* dst = stages + s * G::stage_floats + lane * G::row;
+                // position of the stage row's first float: (row + j0 - RLa) & ~3
+                const int at = (int)(a4 - ((row + j0 - G::RLa) & ~3ll));
+                // the cube's last, partial granule
+                for (long long e = max(a4, D.full); e < row + j_b; ++e) dst[at + (int)(e - a4)] = D.al[e];
+                fence_proxy_async_smem();
+                mbar_arrive_expect_tx(&bars[s], bytes);
+                if (bytes) bulk_load(smem_addr(dst + at), D.al + a4, bytes, &bars[s]);
+            }
+        }
     };
-    if (threadIdx.x == 0)
-        for (int i = 0; i < min(kTS, n_rows); ++i) issue(i);
+    // rows that hold nothing take no stage; live rows take the stages in turn
+    int next = 0, issued = 0;  // warp 0: next input row to look at, live rows issued
+    auto issue_next = [&]() {
+        while (next < n_rows && !live(next)) ++next;
+        if (next < n_rows) {
+            issue(next, issued % kTS);
+            ++next;
+            ++issued;
+        }
+    };
+    if (warp == 0)
+        for (int k = 0; k < kTS; ++k) issue_next();
+    int turn = 0;  // live rows taken
 
     float acc[NR][4];
 #pragma unroll
@@ -353,76 +264,105 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf_tma(cons
     const bool owns = lane >= Q0 && lane < Q1;
     const int x = x0 + warp;
     const int jl = j0 - G::RLa + 4 * lane;  // cube bin of the lane's first box bin
+    // dense rows: position (modulo 2^32) of tap 0's first bin in input row 0
+    const unsigned row_step = (unsigned)nx * (unsigned)nl;
+    const unsigned col0 = (unsigned)D.off + (unsigned)(y0 - RP) * row_step + (unsigned)((x - RP) * nl + j0 - G::RLa);
 
     for (int ib = 0; ib < n_rows; ib += NR) {
 #pragma unroll
         for (int ph = 0; ph < NR; ++ph) {  // accumulator of output row y_in - RP + m is (ph + m) % NR
             const int i = ib + ph;
             if (i < n_rows) {
-                const int s = i % kTS;
-                const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((i / kTS) & 1), 2000000000ll);
-                if (ok) {
-                    // PSF along x: box columns warp .. warp + 2 RP, bins 4 lane .. 4 lane + 3
-                    const float* src = stages + s * G::stage_floats + warp * G::LW + 4 * lane;
-                    float a[4] = {0.f, 0.f, 0.f, 0.f};
+                const bool has = live(i);  // uniform over the CTA
+                if (has) {
+                    const int s = turn % kTS;
+                    const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((turn / kTS) & 1), 2000000000ll);
+                    if (ok) {
+                        float a[4] = {0.f, 0.f, 0.f, 0.f};
+                        if constexpr (!DENSE) {
+                            // PSF along x: box columns warp .. warp + 2 RP, bins 4 lane .. 4 lane + 3
+                            const float* src = stages + s * G::stage_floats + warp * G::row + 4 * lane;
 #pragma unroll
-                    for (int d = 0; d < NR; ++d) {
-                        const float4 c = *reinterpret_cast<const float4*>(src + d * G::LW);
-                        a[0] = fmaf(gp[d], c.x, a[0]);
-                        a[1] = fmaf(gp[d], c.y, a[1]);
-                        a[2] = fmaf(gp[d], c.z, a[2]);
-                        a[3] = fmaf(gp[d], c.w, a[3]);
-                    }
-                    *reinterpret_cast<float4*>(prow + 4 * lane) = make_float4(a[0], a[1], a[2], a[3]);
-                }
-                if (__syncthreads_or(!ok)) {
-                    // a load did not complete in time: record it, let the copies in
-                    // flight land (bounded), and stop
-                    if (threadIdx.x == 0) {
-                        if (P.err) atomicOr(P.err, kErrTmaTimeout);
-                        for (int r = i; r < min(i + kTS, n_rows); ++r)
-                            mbar_wait_bounded(&bars[r % kTS], (uint32_t)((r / kTS) & 1), 200000000ll);
-                    }
-                    return;
-                }
-                // every warp is done with stage s (and the barrier made this
-                // warp's px row visible to its lanes): refill it
-                if (threadIdx.x == 0 && i + kTS < n_rows) issue(i + kTS);
-                const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
-                if (owns) {
-                    // LSF along wavelength from px: bins 4 lane - RLa .. 4 lane + 3 + RLa
-                    const float4* r4 = reinterpret_cast<const float4*>(prow + 4 * lane - G::RLa);
-                    float v[4 * G::NV];
+                            for (int d = 0; d < NR; ++d) {
+                                const float4 c = *reinterpret_cast<const float4*>(src + d * G::row);
+                                a[0] = fmaf(gp[d], c.x, a[0]);
+                                a[1] = fmaf(gp[d], c.y, a[1]);
+                                a[2] = fmaf(gp[d], c.z, a[2]);
+                                a[3] = fmaf(gp[d], c.w, a[3]);
+                            }
+                            *reinterpret_cast<float4*>(prow + 4 * lane) = make_float4(a[0], a[1], a[2], a[3]);
+                        } else {
+                            // bins lane + 32 u: a row starts anywhere in its first granule
+                            const unsigned p = col0 + (unsigned)i * row_step;  // its position, modulo 2^32
+                            const float* stage = stages + s * G::stage_floats + lane;
 #pragma unroll
-                    for (int c = 0; c < G::NV; ++c) {
-                        const float4 t = r4[c];
-                        v[4 * c] = t.x;
-                        v[4 * c + 1] = t.y;
-                        v[4 * c + 2] = t.z;
-                        v[4 * c + 3] = t.w;
-                    }
-                    float o[4];
+                            for (int d = 0; d < NR; ++d) {
+                                const float* src = stage + (warp + d) * G::row + ((p + (unsigned)(d * nl)) & 3u);
+                                float c[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        float b = 0.f;
+                                for (int u = 0; u < 4; ++u) c[u] = src[32 * u];
 #pragma unroll
-                        for (int d = 0; d <= 2 * RL; ++d) b = fmaf(gl[d], v[u + d + G::RLa - RL], b);
-                        o[u] = b;
-                    }
+                                for (int u = 0; u < 4; ++u) a[u] = fmaf(gp[d], c[u], a[u]);
+                            }
 #pragma unroll
-                    for (int m = 0; m < NR; ++m)
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) acc[(ph + m) % NR][u] = fmaf(gp[m], o[u], acc[(ph + m) % NR][u]);
-                    float* done = acc[ph % NR];
-                    if (y_done >= y0 && x < nx) {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int j = jl + u;
-                            if (j < nl) {
-                                const long long idx = ((long long)y_done * nx + x) * nl + j;
-                                out[idx] = (P.noise_inv_s2n > 0.f) ? add_noise(done[u], idx, P) : done[u];
+                            for (int u = 0; u < 4; ++u) {
+                                const int j = j0 - G::RLa + lane + 32 * u;
+                                prow[lane + 32 * u] = (j >= 0 && j < nl) ? a[u] : 0.f;
                             }
                         }
+                    }
+                    if (__syncthreads_or(!ok)) {
+                        // a load did not complete in time: record it, let the copies in
+                        // flight land (bounded), and stop
+                        if (threadIdx.x == 0) {
+                            if (P.err) atomicOr(P.err, kErrTmaTimeout);
+                            for (int r = turn; r < issued; ++r)
+                                mbar_wait_bounded(&bars[r % kTS], (uint32_t)((r / kTS) & 1), 200000000ll);
+                        }
+                        return;
+                    }
+                    // every warp is done with stage s (and the barrier made this
+                    // warp's px row visible to its lanes): refill it
+                    ++turn;
+                    if (warp == 0) issue_next();
+                }
+                const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
+                if (owns) {
+                    if (has) {
+                        // LSF along wavelength from px: bins 4 lane - RLa .. 4 lane + 3 + RLa
+                        const float4* r4 = reinterpret_cast<const float4*>(prow + 4 * lane - G::RLa);
+                        float v[4 * G::NV];
+#pragma unroll
+                        for (int c = 0; c < G::NV; ++c) {
+                            const float4 t = r4[c];
+                            v[4 * c] = t.x;
+                            v[4 * c + 1] = t.y;
+                            v[4 * c + 2] = t.z;
+                            v[4 * c + 3] = t.w;
+                        }
+                        float o[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            float b = 0.f;
+#pragma unroll
+                            for (int d = 0; d <= 2 * RL; ++d) b = fmaf(gl[d], v[u + d + G::RLa - RL], b);
+                            o[u] = b;
+                        }
+#pragma unroll
+                        for (int m = 0; m < NR; ++m)
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) acc[(ph + m) % NR][u] = fmaf(gp[m], o[u], acc[(ph + m) % NR][u]);
+                    }
+                    float* done = acc[ph % NR];
+                    if (y_done >= y0 && x < nx) {
+                        const long long idx = ((long long)y_done * nx + x) * nl + jl;
+                        float4 v = make_float4(done[0], done[1], done[2], done[3]);
+                        if constexpr (NOISE) v = add_noise4(v, idx, P.noise_inv_s2n, P.seed_lo, P.seed_hi);
+                        float* o = out + idx;
+                        if (jl < nl) o[0] = v.x;
+                        if (jl + 1 < nl) o[1] = v.y;
+                        if (jl + 2 < nl) o[2] = v.z;
+                        if (jl + 3 < nl) o[3] = v.w;
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) done[u] = 0.f;
@@ -433,7 +373,9 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf_tma(cons
     }
 }
 
-// Radii with a TMA instantiation (the wavelength halo of at most 8 bins).
+// Radii with a fused instantiation: the PSF of FWHM 1.5 spaxels (rp = 3) and
+// LSFs of sigma 1.2 A on 1.25 A or 3 A bins (rl = 4, 2), plus neighbours (the
+// wavelength halo of at most 8 bins).
 #define RUBIX_TMA_RADII(X) X(3, 4) X(3, 2) X(3, 0) X(0, 4) X(0, 2) X(2, 4) X(4, 4) X(3, 3) X(3, 5)
 
 bool conv_tma_box(int rp, int rl, unsigned box[2]) {
@@ -448,40 +390,73 @@ bool conv_tma_box(int rp, int rl, unsigned box[2]) {
     return false;
 }
 
-template <int RP, int RL>
-static bool launch_tma(const ConvParams& P, const CUtensorMap* map, float* out, cudaStream_t st) {
-    constexpr size_t smem = TmaGeo<RP, RL>::smem;
-    static_assert(smem <= 200 * 1024, "TMA PSF/LSF tile does not fit shared memory");
-    if (cudaFuncSetAttribute(k_psf_lsf_tma<RP, RL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+// Output rows per CTA: the split of the rows that fills whole waves of the
+// resident CTAs with the fewest input rows (each CTA reads 2 rp rows more than it
+// writes). One wave of 150-row CTAs is best for 150 x 150 spaxels x 3721 bins; a
+// 25 x 25 x 1000 cube runs 36 CTAs unsplit.
+constexpr int kMaxTY = 600;  // input rows (ty + 2 rp) have a bit each in the kernel's 96-byte header
+static int rows_per_cta(int ny, int rp, long long columns) {
+    const long long slots = (long long)RUBIX_PSF_TMINB * sm_count();
+    int best = ny;
+    double cost = 1e300;
+    for (int k = 1; k <= ny; ++k) {
+        const int ty = (ny + k - 1) / k;
+        if (ty > kMaxTY) continue;
+        if (ty < 2 * rp && best <= kMaxTY) break;
+        const long long ctas = columns * ((ny + ty - 1) / ty);
+        // the rows of the CTAs one slot takes, and a pipeline start for each
+        const double c = (double)((ctas + slots - 1) / slots) * (ty + 2 * rp + 4);
+        if (c < cost * 0.999) {
+            cost = c;
+            best = ty;
+        }
+    }
+    return best;
+}
+
+template <int RP, int RL, bool DENSE, bool NOISE>
+static bool launch_conv(ConvParams P, const CUtensorMap* map, const DenseRows& D, float* out, cudaStream_t st) {
+    using G = TmaGeo<RP, RL, DENSE>;
+    static_assert(G::smem <= 200 * 1024, "PSF/LSF tile does not fit shared memory");
+    // per launch: the attribute belongs to the current device
+    if (cudaFuncSetAttribute(k_psf_lsf<RP, RL, DENSE, NOISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem) !=
         cudaSuccess)
         return false;
-    constexpr int TL = TmaGeo<RP, RL>::TL;
-    dim3 g((P.n_lambda + TL - 1) / TL, (P.nx + kTX - 1) / kTX, (P.ny + kTY - 1) / kTY);
-    k_psf_lsf_tma<RP, RL><<<g, kTThreads, smem, st>>>(P, *map, out);
+    dim3 g((P.n_lambda + G::TL - 1) / G::TL, (P.nx + kTX - 1) / kTX, 1);
+    P.ty = rows_per_cta(P.ny, RP, (long long)g.x * g.y);
+    g.z = (P.ny + P.ty - 1) / P.ty;
+    k_psf_lsf<RP, RL, DENSE, NOISE><<<g, kTThreads, G::smem, st>>>(P, *map, D, out);
     return true;
 }
 
-static bool try_tma(const ConvParams& P, const CUtensorMap* map, float* out, cudaStream_t st) {
-#define RUBIX_TMA_CASE(RP_, RL_) \
-    if (P.rp == RP_ && P.rl == RL_) return launch_tma<RP_, RL_>(P, map, out, st);
-    RUBIX_TMA_RADII(RUBIX_TMA_CASE)
-#undef RUBIX_TMA_CASE
+static bool try_conv(const ConvParams& P, const CUtensorMap* map, const float* in, float* out, cudaStream_t st) {
+    DenseRows D{};
+    const uintptr_t a = reinterpret_cast<uintptr_t>(in);
+    D.al = reinterpret_cast<const float*>(a & ~(uintptr_t)15);
+    D.off = (long long)((a & 15) / sizeof(float));
+    D.full = (D.off + (long long)P.ny * P.nx * P.n_lambda) & ~3ll;
+    const CUtensorMap none{};
+    const bool noise = P.noise_inv_s2n > 0.f;
+    if (noise && !map) return false;  // (no caller asks for it)
+#define RUBIX_CONV_CASE(RP_, RL_)                                                                       \
+    if (P.rp == RP_ && P.rl == RL_)                                                                      \
+        return !map ? launch_conv<RP_, RL_, true, false>(P, &none, D, out, st)                           \
+                    : (noise ? launch_conv<RP_, RL_, false, true>(P, map, D, out, st)                    \
+                             : launch_conv<RP_, RL_, false, false>(P, map, D, out, st));
+    RUBIX_TMA_RADII(RUBIX_CONV_CASE)
+#undef RUBIX_CONV_CASE
     return false;
 }
 
 bool psf_lsf_needs_tmp(int rp, int rl) {
-#define RUBIX_FUSED_HAS(RP_, RL_) \
-    if (rp == RP_ && rl == RL_) return false;
-    RUBIX_FUSED_RADII(RUBIX_FUSED_HAS)
-#undef RUBIX_FUSED_HAS
-    return true;
+    unsigned box[2];
+    return !conv_tma_box(rp, rl, box);
 }
 
 int launch_psf_lsf(const ConvParams& P, const float* in, int in_pitch, const CUtensorMap* in_map, float* tmp,
                    float* out, cudaStream_t st) {
-    if (in_map && try_tma(P, in_map, out, st)) return 1;
-    if (in_pitch != P.n_lambda) return -1;  // the cp.async kernels read dense rows
-    if (try_fused(P, in, out, st)) return 1;
+    if (!in_map && in_pitch != P.n_lambda) return -1;  // without a map: dense rows
+    if (try_conv(P, in_map, in, out, st)) return 1;
     // generic radii: two passes through an intermediate cube
     const int XW = kXC + 2 * P.rp;
     const size_t smem = (size_t)XW * (kLC + 2 * P.rl + kLC) * sizeof(float);

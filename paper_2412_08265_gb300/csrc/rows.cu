@@ -11,15 +11,39 @@ namespace rubix {
 // Rows of spaxels without particles: zeros (one warp per row, 16-byte stores
 // when the rows are 16-byte aligned). The deposit has no work item for them,
 // so a small galaxy in a large field costs the deposit only its own spaxels.
+// Before a convolution, rows out of reach of any particle are left alone: the
+// fused PSF/LSF kernel takes (row, block of columns) pairs without a particle
+// in reach as zero without reading them (1e4 particles in 300 x 300 x 3721:
+// zero rows 0.21 ms and PSF/LSF 0.75 ms when all are written and read).
 // ----------------------------------------------------------------------------
-__global__ void k_zero_empty(const int* __restrict__ seg_off, int n_s, int nb, float* __restrict__ cube, int pitch,
-                             int n_lambda) {
+__global__ void k_occupied(const int* __restrict__ seg_off, int nx, int ny, int nb, int rp, unsigned char* __restrict__ occ) {
+    const int nxb = (nx + kConvX - 1) / kConvX;
+    const long long n = (long long)ny * nxb;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const int y = (int)(i / nxb), b = (int)(i % nxb);
+        const long long row = (long long)y * nx;
+        const int lo = max(b * kConvX - rp, 0), hi = min((b + 1) * kConvX + rp, nx);
+        occ[i] = seg_off[(row + hi) * nb] != seg_off[(row + lo) * nb];
+    }
+}
+
+__global__ void k_zero_empty(const int* __restrict__ seg_off, int nx, int n_s, int nb, float* __restrict__ cube,
+                             int pitch, int n_lambda, const unsigned char* __restrict__ occ, int rp) {
     const int lane = threadIdx.x & 31;
     const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     const bool vec = (pitch % 4) == 0 && (reinterpret_cast<uintptr_t>(cube) & 15) == 0;
+    const int nxb = (nx + kConvX - 1) / kConvX;
     for (long long s = w0; s < n_s; s += nw) {
         if (seg_off[(s + 1) * nb] != seg_off[s * nb]) continue;
+        if (occ) {
+            // blocks whose columns and reach include this spaxel
+            const int y = (int)(s / nx), x = (int)(s - (long long)y * nx);
+            bool read = false;
+            for (int b = max(x - rp, 0) / kConvX; b <= min((x + rp) / kConvX, nxb - 1); ++b)
+                read = read || occ[(long long)y * nxb + b];
+            if (!read) continue;
+        }
         float* row = cube + s * pitch;
         int j0 = 0;
         if (vec) {
@@ -32,13 +56,19 @@ __global__ void k_zero_empty(const int* __restrict__ seg_off, int n_s, int nb, f
     }
 }
 
-int launch_zero_empty(const int* seg_off, int n_s, int nb, float* cube, int pitch, int n_lambda, cudaStream_t st) {
+int launch_zero_empty(const int* seg_off, int nx, int ny, int nb, float* cube, int pitch, int n_lambda,
+                      unsigned char* occ, int rp, cudaStream_t st) {
+    const long long n_s = (long long)nx * ny;
     if (n_s <= 0) return 0;
-    long long nb_blocks = ((long long)n_s * 32 + 255) / 256;
+    if (occ) {
+        const long long n = (long long)ny * ((nx + kConvX - 1) / kConvX);
+        k_occupied<<<(int)((n + 255) / 256), 256, 0, st>>>(seg_off, nx, ny, nb, rp, occ);
+    }
+    long long nb_blocks = (n_s * 32 + 255) / 256;
     const long long cap = 16ll * sm_count();
     if (nb_blocks > cap) nb_blocks = cap;
-    k_zero_empty<<<(int)nb_blocks, 256, 0, st>>>(seg_off, n_s, nb, cube, pitch, n_lambda);
-    return 1;
+    k_zero_empty<<<(int)nb_blocks, 256, 0, st>>>(seg_off, nx, (int)n_s, nb, cube, pitch, n_lambda, occ, rp);
+    return occ ? 2 : 1;
 }
 
 // ----------------------------------------------------------------------------
