@@ -110,13 +110,12 @@ extern "C" rubix_status rubix_cube_forward(rubix_cube_t* h, const rubix_particle
         h->ring_count = std::min(h->ring_count + 1, rubix_cube::kRing);
     }
     rec_ev(h, 0, st);
-    CK(cudaMemsetAsync(S.d_slow, 0, 8, st));
     s = enqueue_pre(P, p, st, h->prof ? h->ev : nullptr);
     if (s != RUBIX_OK) return s;
     rec_ev(h, 2, st);
     float* target = deposit_target(P, out, noise);
     const DepJob job = plan_job(P, target);
-    const int l = enqueue_deposit(S, &job, 1, P.d_job_cost, st);
+    const int l = enqueue_deposit(S, &job, 1, st);
     if (l < 0) return fail(RUBIX_ERR_CUDA, "deposit launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     P.launches += l;
     P.dep_launches = 1;

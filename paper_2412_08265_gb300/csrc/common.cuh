@@ -13,7 +13,7 @@ constexpr double kC_kms = 299792.458;
 
 // Error word written by kernels (bit flags), read by the host after a forward.
 enum DeviceError : unsigned {
-    kErrTmaTimeout = 1u,      // a bounded mbarrier wait on a TMA slab load expired
+    kErrTmaTimeout = 1u,      // a bounded wait expired (an mbarrier of a slab load, a chained scan)
     kErrBadItem = 2u,         // a work item pointed outside its buffers
     kErrBounds = 4u,          // debug builds: a computed index fell outside its buffer
 };
@@ -152,6 +152,80 @@ __device__ __forceinline__ void ssp_cell(float q, const float* __restrict__ node
 __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
     const int b = (apb > 0) ? ia / apb : 0;
     return b < n_bands - 1 ? b : n_bands - 1;
+}
+
+// ----------------------------------------------------------------------------
+// Scans in one launch. Blocks take tiles in order from a ticket, publish their
+// tile's sum, and add up the sums published before theirs: a block waits only
+// for blocks that hold an earlier ticket, which are running and publish without
+// waiting for anyone. chain[0] is the ticket, chain[1 + tile] the tile's sum
+// with its top bit set; all are cleared beforehand. The wait has a limit, after
+// which the block takes what it has (a sum too small, never too large) and sets
+// the error word.
+// ----------------------------------------------------------------------------
+inline __host__ __device__ size_t chain_words(long long tiles) { return (size_t)tiles + 1; }
+
+struct ChainShared {
+    unsigned ticket;
+    unsigned long long warp[32];
+    unsigned long long total;
+};
+
+__device__ __forceinline__ unsigned chain_ticket(unsigned long long* chain, ChainShared& sh) {
+    if (threadIdx.x == 0) sh.ticket = (unsigned)atomicAdd(chain, 1ull);
+    __syncthreads();
+    return sh.ticket;
+}
+
+// Sum over the block (all threads take part; up to 1024 threads).
+__device__ __forceinline__ unsigned long long block_exclusive(unsigned long long v, ChainShared& sh,
+                                                              unsigned long long& total) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sh.warp[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        const unsigned long long t = (lane < (int)((blockDim.x + 31) >> 5)) ? sh.warp[lane] : 0ull;
+        unsigned long long s = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        sh.warp[lane] = s - t;
+        if (lane == 31) sh.total = s;
+    }
+    __syncthreads();
+    const unsigned long long r = x - v + sh.warp[wid];
+    total = sh.total;
+    __syncthreads();
+    return r;
+}
+
+// Exclusive prefix of v over all threads of all tiles before this one (values
+// and sums below 2^63).
+__device__ __forceinline__ unsigned long long chain_exclusive(unsigned long long v, unsigned tile,
+                                                              unsigned long long* chain, ChainShared& sh, unsigned* err) {
+    unsigned long long total;
+    const unsigned long long e = block_exclusive(v, sh, total);
+    volatile unsigned long long* pub = chain + 1;
+    if (threadIdx.x == 0) pub[tile] = total | (1ull << 63);
+    unsigned long long before = 0;
+    const long long t0 = clock64();
+    for (unsigned i = threadIdx.x; i < tile; i += blockDim.x) {
+        unsigned long long w = pub[i];
+        while (!(w >> 63) && clock64() - t0 < 4000000000ll) w = pub[i];
+        if (w >> 63) before += w & ~(1ull << 63);
+        else if (err) atomicOr(err, kErrTmaTimeout);
+    }
+    unsigned long long sum;
+    block_exclusive(before, sh, sum);
+    return sum + e;
 }
 
 // ----------------------------------------------------------------------------

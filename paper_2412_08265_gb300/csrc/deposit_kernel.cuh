@@ -439,12 +439,38 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
     int* s_job = reinterpret_cast<int*>(smem + 64);        // [kJobChunk] job of table row k
     int* s_ia = s_job + kJobChunk;                         // [kJobChunk] its first item
     int* s_pre = s_ia + kJobChunk;                         // [kJobChunk + 1] prefix of item counts
+    // [kMaxJobs + 1] exclusive prefix of the jobs' per-tile costs
+    long long* jc = reinterpret_cast<long long*>(smem + 64 + 4 * (3 * kJobChunk + 2));
+    static_assert(64 + 4 * (3 * kJobChunk + 2) + 8 * (kMaxJobs + 1) <= kDepHeader, "header");
+    static_assert(kMaxJobs <= 64, "two jobs per lane");
 
     const int lane = threadIdx.x & 31;
     const float lanef = (float)lane;
     const int nb = P.n_bands;
-    const long long* __restrict__ jc = P.job_cost;
     const long long C0 = P.cost_c0;
+    // per-tile cost of each job (in-field particles + cost_c0 per work item),
+    // from the device-side counts, lane l taking jobs 2l and 2l + 1
+    if (threadIdx.x < 32) {
+        long long c[2] = {0, 0};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = 2 * lane + h;
+            if (j < P.n_jobs) {
+                const DepJob& J = P.jobs[j];
+                c[h] = J.seg_off[(long long)J.n_s * nb] + C0 * J.item_off[J.n_s];
+            }
+        }
+        long long x = c[0] + c[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (2 * lane <= P.n_jobs) jc[2 * lane] = x - c[0] - c[1];
+        if (2 * lane + 1 <= P.n_jobs) jc[2 * lane + 1] = x - c[1];
+        if (lane == 31 && P.n_jobs == kMaxJobs) jc[kMaxJobs] = x;
+    }
+    __syncthreads();
     const long long CT = jc[P.n_jobs];
     if (CT <= 0) return;
     const long long total = CT * P.n_tiles;
@@ -548,10 +574,8 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
                     if (prow >= J.part_cap || sp < 0 || sp >= J.n_s) {
                         atomicOr(P.err, kErrBadItem);
                     } else {
-                        if (nb > 1) {
-                            qb = max(qb, J.seg_off[(long long)sp * nb + band]);
-                            qe = min(qe, J.seg_off[(long long)sp * nb + band + 1]);
-                        }
+                        qb = max(qb, J.seg_off[(long long)sp * nb + band]);
+                        qe = min(qe, J.seg_off[(long long)sp * nb + band + 1]);
                         // band 0 visits every item: it writes the row, zeros included
                         live = band == 0 || qb < qe;
                         // the item's first record, on its way to L1 before the warp reaches it

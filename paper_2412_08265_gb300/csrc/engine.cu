@@ -495,16 +495,13 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_map, sizeof(MapRec) * N},
         {(void**)&P->d_prec, sizeof(PartRec) * N},
         {(void**)&P->d_partials, 4 * (size_t)part_cap * n_lambda},
-        {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.geo.n_bands + 2)}, {(void**)&P->d_n_items, 4 * ((size_t)n_s + 1)},
-        {(void**)&P->d_n_parts, 4 * ((size_t)n_s + 1)}, {(void**)&P->d_item_off, 4 * ((size_t)n_s + 1)},
-        {(void**)&P->d_part_off, 4 * ((size_t)n_s + 1)},
-        {(void**)&P->d_scan_scratch, 4 * (scan_scratch_ints(n_s + 1) + 16)},
+        {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.geo.n_bands + 2)},
+        {(void**)&P->d_item_off, 4 * ((size_t)n_s + 1)}, {(void**)&P->d_part_off, 4 * ((size_t)n_s + 1)},
+        {(void**)&P->d_split, 4 * (size_t)n_s}, {(void**)&P->d_chain, 8 * item_chain_words(n_s)},
         {(void**)&P->d_cube0, (size_t)n_s * std::max(pitch0, n_lambda) * sizeof(float)},
-        {(void**)&P->d_job_cost, 8 * (size_t)(kMaxJobs + 1)},
     };
     v.insert(v.end(), rest.begin(), rest.end());
     if (need_tmp) v.push_back({(void**)&P->d_tmp, cube});
-    v.push_back({(void**)&P->d_occ, (size_t)n_s});
     if (with_out) v.push_back({(void**)&P->d_out, cube});
     if (with_grad) {
         v.push_back({(void**)&P->d_contrib, 8 * kGlobal * N});
@@ -754,8 +751,10 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         A.n_bands = S.geo.n_bands;
         P.launches += launch_assign(A, st);
         P.launches += launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
-                                         P.d_perm, P.d_seg_off, P.d_sort_scratch, st);
+                                         P.d_perm, P.d_seg_off, P.d_sort_scratch, false, P.d_chain,
+                                         (int)item_chain_words(P.n_s), S.d_err, st);
     } else {
+        CK(cudaMemsetAsync(P.d_chain, 0, 8 * item_chain_words(P.n_s), st));
         CK(cudaMemsetAsync(P.d_seg_off, 0, ((size_t)P.n_s * S.geo.n_bands + 2) * sizeof(int), st));
     }
     if (ev) cudaEventRecord(ev[1], st);
@@ -785,6 +784,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     SP.s_min = S.geo.s_min;
     SP.s_max = S.geo.s_max;
     SP.prec = P.d_prec;
+    SP.n_total = n;
     SP.n_cap = P.cap;
     P.launches += launch_setup(SP, n, st);
     ItemParams IP{};
@@ -792,13 +792,13 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     IP.n_s = P.n_s;
     IP.n_bands = S.geo.n_bands;
     IP.chunk = S.chunk;
-    IP.n_items = P.d_n_items;
-    IP.n_parts = P.d_n_parts;
     IP.item_off = P.d_item_off;
     IP.part_off = P.d_part_off;
     IP.items = P.d_items;
     IP.item_cap = P.item_cap;
-    IP.scan_scratch = P.d_scan_scratch;
+    IP.split = P.d_split;
+    IP.chain = P.d_chain;
+    IP.slow_count = P.alloc.async ? nullptr : S.d_slow;  // one forward at a time on a handle
     IP.err = S.d_err;
     P.launches += launch_items(IP, st);
     P.last_n = n;
@@ -824,14 +824,13 @@ DepJob plan_job(const Plan& P, float* target) {
     return J;
 }
 
-int enqueue_deposit(const SspState& S, const DepJob* jobs, int n_jobs, long long* d_job_cost, cudaStream_t st) {
+int enqueue_deposit(const SspState& S, const DepJob* jobs, int n_jobs, cudaStream_t st) {
     NvtxRange nvtx("rubix: deposit");
     if (n_jobs < 1 || n_jobs > kMaxJobs) return -1;
     DepositParams DP{};
     static_cast<SlabParams&>(DP) = S.geo;
     for (int j = 0; j < n_jobs; ++j) DP.jobs[j] = jobs[j];
     DP.n_jobs = n_jobs;
-    DP.job_cost = d_job_cost;
     DP.slow_count = S.d_slow;
     return launch_deposit(DP, S.dep_ctas, S.dep_threads, S.dep_smem, st);
 }
@@ -842,16 +841,26 @@ int enqueue_post(Plan& P, float* target, float* out, uint64_t noise_seed, float 
     const int pitch = target == P.d_cube0 ? P.pitch0 : P.tel.n_lambda;
     const bool noise = noise_s2n > 0.f;
     // the fused convolution does not read rows out of every particle's reach
-    unsigned char* occ = target == P.d_cube0 && P.has_conv_map ? P.d_occ : nullptr;
-    int l = launch_zero_empty(P.d_seg_off, P.tel.nx, P.rows, P.S->geo.n_bands, target, pitch, P.tel.n_lambda, occ,
-                              P.conv.rp, st);
-    // d_n_parts (scanned into d_part_off by the item stage) is free here: the
-    // combine's list of split spaxels
-    l += launch_combine(P.d_part_off, P.n_s, P.tel.n_lambda, P.d_partials, target, pitch, P.d_n_parts, st);
+    const bool skip = target == P.d_cube0 && P.has_conv_map;
+    RowParams RP{};
+    RP.seg_off = P.d_seg_off;
+    RP.nx = P.tel.nx;
+    RP.ny = P.rows;
+    RP.n_bands = P.S->geo.n_bands;
+    RP.n_lambda = P.tel.n_lambda;
+    RP.pitch = pitch;
+    RP.skip_rp = skip ? P.conv.rp : -1;
+    RP.part_off = P.d_part_off;
+    RP.split = P.d_split;
+    RP.n_split = P.d_chain + item_chain_words(P.n_s) - 1;
+    RP.partials = P.d_partials;
+    RP.cube = target;
+    int l = launch_rows(RP, st);
     if (ev) cudaEventRecord(ev[4], st);
     if (P.need_conv || noise) {
         ConvParams C = P.conv;
-        C.occ = occ;
+        C.seg_off = skip ? P.d_seg_off : nullptr;
+        C.seg_bands = P.S->geo.n_bands;
         C.noise_inv_s2n = noise ? 1.0f / noise_s2n : 0.f;
         C.seed_lo = (uint32_t)noise_seed;
         C.seed_hi = (uint32_t)(noise_seed >> 32);

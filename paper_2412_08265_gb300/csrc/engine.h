@@ -101,8 +101,8 @@ struct Plan {
     int *d_key = nullptr, *d_keys_tmp = nullptr, *d_vals_tmp = nullptr, *d_skeys = nullptr, *d_perm = nullptr;
     PartRec* d_pin = nullptr;  // [cap] (mass, age, Z, v_los) in original order, written by the assign
     int* d_sort_scratch = nullptr;
-    int *d_seg_off = nullptr, *d_n_items = nullptr, *d_n_parts = nullptr, *d_item_off = nullptr;
-    int *d_part_off = nullptr, *d_scan_scratch = nullptr;
+    int *d_seg_off = nullptr, *d_item_off = nullptr, *d_part_off = nullptr, *d_split = nullptr;
+    unsigned long long* d_chain = nullptr;  // scan of the work items (ItemParams::chain)
     Item* d_items = nullptr;
     DepRec* d_rec = nullptr;
     MapRec* d_map = nullptr;
@@ -112,8 +112,6 @@ struct Plan {
     int pitch0 = 0;                         // row stride of d_cube0 (16-byte rows for the TMA PSF/LSF)
     CUtensorMap conv_map{};                 // 3-D TMA map of d_cube0 for the PSF/LSF kernel
     bool has_conv_map = false;
-    unsigned char* d_occ = nullptr;         // ConvParams::occ of the last forward
-    long long* d_job_cost = nullptr;        // deposit launch scratch [kMaxJobs + 1]
     double *d_contrib = nullptr, *d_red = nullptr;
     float2* d_dvda = nullptr;               // backward: dv_los/d(inclination, azimuth) per particle [cap]
     float2* d_wu = nullptr;                 // backward: (ta, tz) in the SSP cell [cap]
@@ -146,7 +144,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
 rubix_status enqueue_keys(Plan& P, const rubix_particles* p, int* keys_out, cudaStream_t st);
 float* deposit_target(const Plan& P, float* out, bool noise);
 DepJob plan_job(const Plan& P, float* target);
-int enqueue_deposit(const SspState& S, const DepJob* jobs, int n_jobs, long long* d_job_cost, cudaStream_t st);
+int enqueue_deposit(const SspState& S, const DepJob* jobs, int n_jobs, cudaStream_t st);
 int enqueue_post(Plan& P, float* target, float* out, uint64_t noise_seed, float noise_s2n, cudaStream_t st,
                  cudaEvent_t* ev = nullptr);
 const char* last_error();

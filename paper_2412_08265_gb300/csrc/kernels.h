@@ -82,12 +82,14 @@ struct AssignParams {
 };
 
 int launch_assign(const AssignParams& P, cudaStream_t st);
-size_t scan_scratch_ints(long long n);
-int launch_exclusive_scan(const int* in, int* out, long long n, int* scratch, cudaStream_t st);
-size_t sort_scratch_ints(long long n);
-// Stable sort of keys in [0, n_keys); seg_off gets n_keys + 1 entries.
+// Scratch of a sort of n keys (long_tiles: with the large tiles whatever n is,
+// for less scratch).
+size_t sort_scratch_ints(long long n, bool long_tiles = false);
+// Stable sort of keys in [0, n_keys); seg_off gets n_keys + 1 entries. Also
+// clears next_chain (nullable), the chain of a scan that follows.
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
-                       int* perm_out, int* seg_off, int* scratch, cudaStream_t st);
+                       int* perm_out, int* seg_off, int* scratch, bool long_tiles, unsigned long long* next_chain,
+                       int n_next_chain, unsigned* err, cudaStream_t st);
 
 // SSP grid as seen by the kernels (the templates themselves as cell quads).
 struct SspDev {
@@ -117,6 +119,7 @@ struct SetupParams {
     int fb, jc, apb, kind;
     float a_max, s_min, s_max;
     PartRec* prec;           // [n_in]
+    long long n_total;       // particles (perm holds indices below it)
     long long n_cap;         // capacity of rec / prec
 };
 int launch_setup(const SetupParams& P, long long n_total, cudaStream_t st);
@@ -125,15 +128,18 @@ struct ItemParams {
     const int* seg_off;      // [n_s * n_bands + 2]
     int n_s, n_bands;
     int chunk;               // max particles per item
-    int* n_items;            // [n_s + 1] scratch
-    int* n_parts;            // [n_s + 1] scratch
     int* item_off;           // [n_s + 1]
     int* part_off;           // [n_s + 1]
+    int* split;              // [n_s] the split spaxels, in any order
     Item* items;             // capacity item_cap
     long long item_cap;
-    int* scan_scratch;
+    // item_chain_words(n_s) words, cleared (common.cuh); the last counts the
+    // split spaxels
+    unsigned long long* chain;
+    unsigned long long* slow_count;  // nullable: the forward's count of per-bin visits, reset here
     unsigned* err;
 };
+size_t item_chain_words(int n_s);
 int launch_items(const ItemParams& P, cudaStream_t st);
 
 // K4: deposit. One launch deposits up to kMaxJobs galaxies (jobs) that share
@@ -195,24 +201,27 @@ inline __host__ __device__ const void* band_ptr(const void* pair, int qdt, long 
 struct DepositParams : SlabParams {
     DepJob jobs[kMaxJobs];
     int n_jobs;
-    long long* job_cost;     // [n_jobs + 1] device scratch: exclusive prefix of the jobs' per-tile cost
     unsigned long long* slow_count;
 };
 int launch_deposit(const DepositParams& P, int n_ctas, int threads, size_t smem, cudaStream_t st);
 size_t deposit_smem_bytes(int pitch, int slab_w);
 
-// Zero rows of the spaxels without particles (no work item covers them). With
-// occ ([ny][ceil(nx / kConvX)], written first: ConvParams::occ for radius rp),
-// only of those that an occupied block's columns reach.
-int launch_zero_empty(const int* seg_off, int nx, int ny, int nb, float* cube, int pitch, int n_lambda,
-                      unsigned char* occ, int rp, cudaStream_t st);
-
-// K5: combine partial rows of split spaxels in a fixed order: FP32 for at most
-// kCombineF32Rows rows, a compensated FP32 sum (two-sum) above. list: n_s + 1
-// ints of scratch (the split spaxels and their count).
+// Rows the deposit leaves: zeros for the spaxels without particles (no work
+// item covers them; with skip_rp >= 0 only those within the fused convolution's
+// reach of a particle: ConvParams::seg_off with rp = skip_rp), and the partial
+// rows of split spaxels summed in a fixed order (K5): FP32 for at most
+// kCombineF32Rows rows, a compensated FP32 sum (two-sum) above.
 constexpr int kCombineF32Rows = 4;
-int launch_combine(const int* part_off, int n_s, int n_lambda, const float* partials, float* cube, int pitch,
-                   int* list, cudaStream_t st);
+struct RowParams {
+    const int* seg_off;
+    int nx, ny, n_bands, n_lambda, pitch, skip_rp;
+    const int* part_off;
+    const int* split;                    // the split spaxels
+    const unsigned long long* n_split;   // their number
+    const float* partials;
+    float* cube;
+};
+int launch_rows(const RowParams& P, cudaStream_t st);
 
 // K6: PSF + LSF (+ noise).
 constexpr int kMaxRadius = 64;
@@ -225,9 +234,11 @@ struct ConvParams {
     uint32_t seed_lo, seed_hi;
     unsigned* err;               // device error word (bounded waits of the fused kernel; nullable)
     int ty;                      // output rows per CTA (set at launch)
-    // [ny][ceil(nx / kConvX)] (nullable): does row y hold anything within rp of
-    // block b's columns? Rows of blocks that do not are taken as zero, unread.
-    const unsigned char* occ;
+    // segment offsets of the cube's spaxels, seg_bands per spaxel (nullable): a
+    // (row, block of kConvX columns) without a particle within rp columns is
+    // taken as zero, unread
+    const int* seg_off;
+    int seg_bands;
 };
 constexpr int kConvX = 8;        // spaxels along x per fused CTA
 // `in` rows have stride in_pitch floats; `out` is dense ([ny][nx][n_lambda]).

@@ -35,7 +35,7 @@ constexpr long long kNoallocMaxParticles = 1ll << 18;   // 262144
 constexpr int kNoallocMaxKeys = 1 << 18;                // keys in [0, nx*ny]
 constexpr long long kNoallocTiles = (kNoallocMaxParticles + 4095) / 4096;
 // keys, keys_tmp, vals_tmp, sorted keys, then the sort's digit counts/offsets/scan scratch
-constexpr long long kNoallocSortInts = 2 * kNoallocTiles * 512 + (kNoallocTiles * 512 + 4095) / 4096 + 1 + 16;
+constexpr long long kNoallocSortInts = 2 * kNoallocTiles * 512 + 2 * ((kNoallocTiles * 512 + 4095) / 4096 + 1) + 16;
 constexpr long long kNoallocInts = 4 * kNoallocMaxParticles + kNoallocSortInts;
 
 static __device__ __align__(256) int g_noalloc_scratch[kNoallocInts];
@@ -96,7 +96,7 @@ extern "C" rubix_status rubix_spaxel_sort_noalloc(const rubix_particles* p, cons
     // the sort's scratch layout (tiles, digit buckets, scan tiles) must fit
     // the fixed array; a change of those constants shows up here, not as an
     // overrun
-    if ((long long)sort_scratch_ints(n_or_1(p->n)) > kNoallocSortInts) {
+    if ((long long)sort_scratch_ints(n_or_1(p->n), true) > kNoallocSortInts) {
         set_last_error("internal: the sort needs more scratch than the no-allocation array holds");
         return RUBIX_ERR_UNSUPPORTED;
     }
@@ -135,7 +135,8 @@ extern "C" rubix_status rubix_spaxel_sort_noalloc(const rubix_particles* p, cons
     A.key = keys;
     A.pin_out = nullptr;
     launch_assign(A, st);
-    launch_sort_by_key(keys, n, n_keys, keys_tmp, vals_tmp, skeys, perm_out, seg_off_out, sort_scratch, st);
+    launch_sort_by_key(keys, n, n_keys, keys_tmp, vals_tmp, skeys, perm_out, seg_off_out, sort_scratch, true,
+                       nullptr, 0, nullptr, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         char m[160];

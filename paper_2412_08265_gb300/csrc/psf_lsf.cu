@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     for (int i0 = warp * 32; i0 < n_rows; i0 += kTThreads) {
         const int y = y0 - RP + i0 + lane;
         const bool on = i0 + lane < n_rows && y >= 0 && y < P.ny &&
-                        (!P.occ || P.occ[(long long)y * gridDim.y + blockIdx.y]);
+                        (!P.seg_off || P.seg_off[((long long)y * nx + min(x0 + kTX + RP, nx)) * P.seg_bands] !=
+                                           P.seg_off[((long long)y * nx + max(x0 - RP, 0)) * P.seg_bands]);
         const unsigned m = __ballot_sync(0xffffffffu, on);
         if (lane == 0) s_live[i0 >> 5] = m;
     }

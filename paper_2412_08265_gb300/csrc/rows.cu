@@ -16,59 +16,33 @@ namespace rubix {
 // in reach as zero without reading them (1e4 particles in 300 x 300 x 3721:
 // zero rows 0.21 ms and PSF/LSF 0.75 ms when all are written and read).
 // ----------------------------------------------------------------------------
-__global__ void k_occupied(const int* __restrict__ seg_off, int nx, int ny, int nb, int rp, unsigned char* __restrict__ occ) {
-    const int nxb = (nx + kConvX - 1) / kConvX;
-    const long long n = (long long)ny * nxb;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(i / nxb), b = (int)(i % nxb);
-        const long long row = (long long)y * nx;
-        const int lo = max(b * kConvX - rp, 0), hi = min((b + 1) * kConvX + rp, nx);
-        occ[i] = seg_off[(row + hi) * nb] != seg_off[(row + lo) * nb];
-    }
-}
-
-__global__ void k_zero_empty(const int* __restrict__ seg_off, int nx, int n_s, int nb, float* __restrict__ cube,
-                             int pitch, int n_lambda, const unsigned char* __restrict__ occ, int rp) {
-    const int lane = threadIdx.x & 31;
-    const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const bool vec = (pitch % 4) == 0 && (reinterpret_cast<uintptr_t>(cube) & 15) == 0;
-    const int nxb = (nx + kConvX - 1) / kConvX;
+__device__ __forceinline__ void zero_rows(const RowParams& P, long long w0, long long nw, int lane) {
+    const int nb = P.n_bands, nx = P.nx;
+    const long long n_s = (long long)nx * P.ny;
+    const bool vec = (P.pitch % 4) == 0 && (reinterpret_cast<uintptr_t>(P.cube) & 15) == 0;
     for (long long s = w0; s < n_s; s += nw) {
-        if (seg_off[(s + 1) * nb] != seg_off[s * nb]) continue;
-        if (occ) {
-            // blocks whose columns and reach include this spaxel
-            const int y = (int)(s / nx), x = (int)(s - (long long)y * nx);
+        if (P.seg_off[(s + 1) * nb] != P.seg_off[s * nb]) continue;
+        if (P.skip_rp >= 0) {
+            // is it read: by a block whose columns, widened by rp, hold both the
+            // spaxel and a particle of its row
+            const long long y = s / nx;
+            const int x = (int)(s - y * nx), rp = P.skip_rp;
+            const int* row = P.seg_off + y * nx * nb;
             bool read = false;
-            for (int b = max(x - rp, 0) / kConvX; b <= min((x + rp) / kConvX, nxb - 1); ++b)
-                read = read || occ[(long long)y * nxb + b];
+            for (int b = max(x - rp, 0) / kConvX; b <= (x + rp) / kConvX && b * kConvX < nx; ++b)
+                read = read || row[min((b + 1) * kConvX + rp, nx) * nb] != row[max(b * kConvX - rp, 0) * nb];
             if (!read) continue;
         }
-        float* row = cube + s * pitch;
+        float* row = P.cube + s * P.pitch;
         int j0 = 0;
         if (vec) {
             float4* r4 = reinterpret_cast<float4*>(row);
-            const int n4 = n_lambda >> 2;
+            const int n4 = P.n_lambda >> 2;
             for (int j = lane; j < n4; j += 32) r4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             j0 = n4 << 2;
         }
-        for (int j = j0 + lane; j < n_lambda; j += 32) row[j] = 0.f;
+        for (int j = j0 + lane; j < P.n_lambda; j += 32) row[j] = 0.f;
     }
-}
-
-int launch_zero_empty(const int* seg_off, int nx, int ny, int nb, float* cube, int pitch, int n_lambda,
-                      unsigned char* occ, int rp, cudaStream_t st) {
-    const long long n_s = (long long)nx * ny;
-    if (n_s <= 0) return 0;
-    if (occ) {
-        const long long n = (long long)ny * ((nx + kConvX - 1) / kConvX);
-        k_occupied<<<(int)((n + 255) / 256), 256, 0, st>>>(seg_off, nx, ny, nb, rp, occ);
-    }
-    long long nb_blocks = (n_s * 32 + 255) / 256;
-    const long long cap = 16ll * sm_count();
-    if (nb_blocks > cap) nb_blocks = cap;
-    k_zero_empty<<<(int)nb_blocks, 256, 0, st>>>(seg_off, nx, (int)n_s, nb, cube, pitch, n_lambda, occ, rp);
-    return occ ? 2 : 1;
 }
 
 // ----------------------------------------------------------------------------
@@ -82,21 +56,6 @@ int launch_zero_empty(const int* seg_off, int nx, int ny, int nb, float* cube, i
 // which on this GPU runs at 1/64 of the FP32 rate.
 // ----------------------------------------------------------------------------
 
-// The split spaxels, compacted (in any order: each row's sum is in item order,
-// so the result does not depend on it); list[n_s] counts them.
-__global__ void k_split_list(const int* __restrict__ part_off, int n_s, int* __restrict__ list) {
-    const int lane = threadIdx.x & 31;
-    for (int s0 = blockIdx.x * blockDim.x; s0 < n_s; s0 += gridDim.x * blockDim.x) {
-        const int s = s0 + threadIdx.x;
-        const bool split = s < n_s && part_off[s + 1] > part_off[s];
-        const unsigned m = __ballot_sync(0xffffffffu, split);
-        int at = 0;
-        if (lane == 0 && m) at = atomicAdd(list + n_s, __popc(m));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (split) list[at + __popc(m & ((1u << lane) - 1u))] = s;
-    }
-}
-
 constexpr int kCombineBins = 128;  // bins of one row per combine unit: 4 per lane of one warp
 
 // One unit = kCombineBins bins of one split spaxel's row, taken by one warp
@@ -104,20 +63,15 @@ constexpr int kCombineBins = 128;  // bins of one row per combine unit: 4 per la
 // loads per partial row in flight), so that the rows of a very high-count
 // spaxel are summed by many warps at once and each warp has several loads
 // in flight while it waits on the next unit's row offsets.
-__global__ void __launch_bounds__(256) k_combine(const int* __restrict__ part_off, int n_s, int n_lambda,
-                                                 const int* __restrict__ list, const float* __restrict__ partials,
-                                                 float* __restrict__ cube, int pitch) {
-    const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const int n_split = list[n_s];
+__device__ __forceinline__ void combine_rows(const RowParams& P, long long warp, long long n_warps, int lane) {
+    const int n_split = (int)*P.n_split, n_lambda = P.n_lambda;
     const int n_chunks = (n_lambda + kCombineBins - 1) / kCombineBins;
     const long long n_units = (long long)n_split * n_chunks;
     for (long long u = warp; u < n_units; u += n_warps) {
-        const int s = list[u / n_chunks];
+        const int s = P.split[u / n_chunks];
         const int j0 = (int)(u % n_chunks) * kCombineBins + lane;
-        const int p0 = part_off[s], nr = part_off[s + 1] - p0;
-        const float* __restrict__ col = partials + (long long)p0 * n_lambda;
+        const int p0 = P.part_off[s], nr = P.part_off[s + 1] - p0;
+        const float* __restrict__ col = P.partials + (long long)p0 * n_lambda;
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, err[4] = {0.f, 0.f, 0.f, 0.f};
         bool in[4];
 #pragma unroll
@@ -140,19 +94,27 @@ __global__ void __launch_bounds__(256) k_combine(const int* __restrict__ part_of
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (in[k]) cube[(long long)s * pitch + j0 + 32 * k] = acc[k];
+            if (in[k]) P.cube[(long long)s * P.pitch + j0 + 32 * k] = acc[k];
     }
 }
 
-int launch_combine(const int* part_off, int n_s, int n_lambda, const float* partials, float* cube, int pitch,
-                   int* list, cudaStream_t st) {
+// The split spaxels' rows first: they take longest.
+__global__ void __launch_bounds__(256) k_rows(const __grid_constant__ RowParams P) {
+    const int lane = threadIdx.x & 31;
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
+    combine_rows(P, warp, n_warps, lane);
+    zero_rows(P, warp, n_warps, lane);
+}
+
+int launch_rows(const RowParams& P, cudaStream_t st) {
+    const long long n_s = (long long)P.nx * P.ny;
     if (n_s < 1) return 0;
-    cudaMemsetAsync(list + n_s, 0, sizeof(int), st);  // an error here is the caller's next cudaGetLastError
-    long long nb = ((long long)n_s + 255) / 256;
-    if (nb > 4ll * sm_count()) nb = 4ll * sm_count();
-    k_split_list<<<(int)nb, 256, 0, st>>>(part_off, n_s, list);
-    k_combine<<<8 * sm_count(), 256, 0, st>>>(part_off, n_s, n_lambda, list, partials, cube, pitch);
-    return 2;
+    long long nb = (n_s * 32 + 255) / 256;
+    const long long cap = 8ll * sm_count();
+    if (nb > cap) nb = cap;
+    k_rows<<<(int)nb, 256, 0, st>>>(P);
+    return 1;
 }
 
 }  // namespace rubix

@@ -90,7 +90,6 @@ struct rubix_server {
     int max_slots = 1, max_batch = 1;
     cudaMemPool_t pool = nullptr;
     cudaStream_t dep_stream = nullptr;
-    long long* d_job_cost = nullptr;
     std::vector<Slot> slots;
     std::vector<Batch> batch_ev;  // deposit launches in flight (at most 2 used)
 
@@ -195,7 +194,7 @@ bool launch_batch(rubix_server* srv) {
         cudaStreamWaitEvent(srv->dep_stream, srv->slots[batch[j]->slot].ev_pre, 0);
         jobs[j] = plan_job(batch[j]->plan, batch[j]->target);
     }
-    const int l = enqueue_deposit(*srv->S, jobs, n, srv->d_job_cost, srv->dep_stream);
+    const int l = enqueue_deposit(*srv->S, jobs, n, srv->dep_stream);
     if (l < 0 || cudaEventRecord(B->ev, srv->dep_stream) != cudaSuccess) {
         const char* m = cudaGetErrorString(cudaGetLastError());
         for (const ReqPtr& r : batch) {
@@ -324,7 +323,6 @@ static void free_server(rubix_server* srv) {
     }
     for (Batch& b : srv->batch_ev)
         if (b.ev) cudaEventDestroy(b.ev);
-    if (srv->d_job_cost) cudaFree(srv->d_job_cost);
     if (srv->dep_stream) cudaStreamDestroy(srv->dep_stream);
     if (srv->pool) cudaMemPoolDestroy(srv->pool);
     ssp_state_destroy(srv->S);
@@ -358,7 +356,6 @@ extern "C" rubix_status rubix_serve_create(const rubix_ssp_grid* ssp, const rubi
         cuuint64_t keep = hbm_budget_bytes;
         SCK(cudaMemPoolSetAttribute(srv->pool, cudaMemPoolAttrReleaseThreshold, &keep));
         SCK(cudaStreamCreateWithFlags(&srv->dep_stream, cudaStreamNonBlocking));
-        SCK(cudaMalloc(&srv->d_job_cost, sizeof(long long) * (kMaxJobs + 1)));
         srv->slots.resize(max_slots);
         for (int i = 0; i < max_slots; ++i) {
             Slot& sl = srv->slots[i];

@@ -84,7 +84,11 @@ __global__ void k_setup(SetupParams P) {
     const float t_lastj = (float)(P.resample ? P.n_lambda : P.n_lambda - 1);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_in;
          i += (long long)gridDim.x * blockDim.x) {
-        const PartRec pr = P.pin[P.perm[i]];
+        // (an index out of range: only after an expired wait in the sort, which
+        // the error word reports)
+        const int pi = P.perm[i];
+        PartRec pr{0.f, 1.f, 1.f, 0.f};
+        if ((unsigned)pi < (unsigned)P.n_total) pr = P.pin[pi];
         const float m = pr.mass, age = pr.age, Z = pr.Z;
         int ia, iz;
         float ta, tz, dta, dtz;
@@ -161,47 +165,52 @@ int launch_setup(const SetupParams& P, long long n_total, cudaStream_t st) {
 }
 
 // ----------------------------------------------------------------------------
-// Work items: one per <= chunk particles of a spaxel (all age bands). Empty
-// spaxels get no item: k_zero_empty writes their rows.
+// Work items: one per <= chunk particles of a spaxel (all age bands), in one
+// launch over a chained scan (common.cuh) of the spaxels' items and partial
+// rows. Empty spaxels get no item: k_rows writes their rows. (Counts, two scans
+// of three launches and the fill were eight launches.)
 // ----------------------------------------------------------------------------
-__global__ void k_item_counts(ItemParams P) {
-    const int nb = P.n_bands;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s <= P.n_s; s += gridDim.x * blockDim.x) {
-        if (s == P.n_s) { P.n_items[s] = 0; P.n_parts[s] = 0; continue; }
-        const int cnt = P.seg_off[(long long)(s + 1) * nb] - P.seg_off[(long long)s * nb];
-        const int ni = (cnt + P.chunk - 1) / P.chunk;
-        P.n_items[s] = ni;
-        P.n_parts[s] = ni > 1 ? ni : 0;
-    }
-}
+constexpr int kItemTile = 1024;  // spaxels per block, one per thread
 
-__global__ void k_item_fill(ItemParams P) {
+size_t item_chain_words(int n_s) { return chain_words(((long long)n_s + kItemTile) / kItemTile) + 1; }
+
+__global__ void __launch_bounds__(kItemTile) k_items(const ItemParams P, int n_tiles) {
+    __shared__ ChainShared sh;
+    const unsigned tile = chain_ticket(P.chain, sh);
+    if (tile == 0 && threadIdx.x == 0 && P.slow_count) *P.slow_count = 0ull;
     const int nb = P.n_bands;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < P.n_s; s += gridDim.x * blockDim.x) {
-        const int base = P.item_off[s], ni = P.item_off[s + 1] - base;
-        const bool split = P.part_off[s + 1] > P.part_off[s];
-        const int b0 = P.seg_off[(long long)s * nb], e0 = P.seg_off[(long long)(s + 1) * nb];
-        for (int i = 0; i < ni; ++i) {
-            if ((long long)base + i >= P.item_cap) { atomicOr(P.err, kErrBadItem); return; }
-            Item it;
-            it.spaxel = s;
-            it.begin = b0 + i * P.chunk;
-            it.end = min(b0 + (i + 1) * P.chunk, e0);
-            it.part_row = split ? P.part_off[s] + i : -1;
-            P.items[base + i] = it;
+    const long long s = (long long)tile * kItemTile + threadIdx.x;  // entry n_s closes the offsets
+    int b0 = 0, e0 = 0;
+    if (s < P.n_s) {
+        b0 = P.seg_off[s * nb];
+        e0 = P.seg_off[(s + 1) * nb];
+    }
+    const int ni = (e0 - b0 + P.chunk - 1) / P.chunk;
+    const int np = ni > 1 ? ni : 0;  // partial rows
+    const unsigned long long pre = chain_exclusive(((unsigned long long)np << 32) | (unsigned)ni, tile, P.chain, sh, P.err);
+    if (s > P.n_s) return;
+    const int base = (int)(pre & 0xffffffffu), part = (int)(pre >> 32);
+    P.item_off[s] = base;
+    P.part_off[s] = part;
+    if (np) P.split[atomicAdd(P.chain + n_tiles + 1, 1ull)] = (int)s;
+    for (int i = 0; i < ni; ++i) {
+        if ((long long)base + i >= P.item_cap) {
+            atomicOr(P.err, kErrBadItem);
+            return;
         }
+        Item it;
+        it.spaxel = (int)s;
+        it.begin = b0 + i * P.chunk;
+        it.end = min(b0 + (i + 1) * P.chunk, e0);
+        it.part_row = np ? part + i : -1;
+        P.items[base + i] = it;
     }
 }
 
 int launch_items(const ItemParams& P, cudaStream_t st) {
-    int nb = (P.n_s + 1 + 255) / 256;
-    if (nb > 4096) nb = 4096;
-    k_item_counts<<<nb, 256, 0, st>>>(P);
-    int l = 1;
-    l += launch_exclusive_scan(P.n_items, P.item_off, P.n_s + 1, P.scan_scratch, st);
-    l += launch_exclusive_scan(P.n_parts, P.part_off, P.n_s + 1, P.scan_scratch, st);
-    k_item_fill<<<nb, 256, 0, st>>>(P);
-    return l + 1;
+    const int n_tiles = (int)(((long long)P.n_s + kItemTile) / kItemTile);  // covers entry n_s
+    k_items<<<n_tiles, kItemTile, 0, st>>>(P, n_tiles);
+    return 1;
 }
 
 }  // namespace rubix

@@ -131,98 +131,34 @@ __global__ void k_assign(AssignParams P) {
 }
 
 // ----------------------------------------------------------------------------
-// Exclusive scan of int32 (3 phases: block sums, scan of sums, block scans).
+// Exclusive scan of int32 in one launch (ChainedTiles, common.cuh): a tile's
+// blocks publish their sums as soon as they have them and add up those before
+// theirs, so that no block waits for more than another block's loads. (Three
+// launches -- block sums, scan of the sums, block scans -- took 8 us of a small
+// galaxy's pass each time.)
 // ----------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_tot[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int t = (lane < (int)(blockDim.x >> 5)) ? warp_tot[lane] : 0;
-        int s = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        warp_tot[lane] = s - t;
-        if (lane == 31) *total = s;
-    }
-    __syncthreads();
-    int r = x - v + warp_tot[wid];
-    __syncthreads();
-    return r;
-}
-
-__global__ void k_scan_reduce(const int* __restrict__ in, long long n, int* __restrict__ sums) {
-    __shared__ int wt[32];
-    __shared__ int tot;
-    long long base = (long long)blockIdx.x * kScanTile;
-    int s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        long long idx = base + (long long)i * kScanThreads + threadIdx.x;
-        if (idx < n) s += in[idx];
-    }
-    block_exclusive_scan(s, wt, &tot);
-    if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-__global__ void k_scan_sums(int* sums, int nb) {
-    __shared__ int wt[32];
-    __shared__ int tot;
-    int carry = 0;
-    for (int base = 0; base < nb; base += blockDim.x) {
-        int i = base + threadIdx.x;
-        int v = (i < nb) ? sums[i] : 0;
-        int e = block_exclusive_scan(v, wt, &tot);
-        if (i < nb) sums[i] = carry + e;
-        carry += tot;
-        __syncthreads();
-    }
-}
-
-__global__ void k_scan_apply(const int* __restrict__ in, long long n, const int* __restrict__ sums,
-                             int* __restrict__ out) {
-    __shared__ int wt[32];
-    __shared__ int tot;
-    long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
+__global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, long long n, int* __restrict__ out,
+                                                       unsigned long long* __restrict__ chain, unsigned* err) {
+    __shared__ ChainShared sh;
+    const unsigned tile = chain_ticket(chain, sh);
+    const long long base = (long long)tile * kScanTile + (long long)threadIdx.x * kScanItems;
     int v[kScanItems];
     int s = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        long long idx = base + i;
-        v[i] = (idx < n) ? in[idx] : 0;
+        v[i] = (base + i < n) ? in[base + i] : 0;
         s += v[i];
     }
-    int e = block_exclusive_scan(s, wt, &tot) + sums[blockIdx.x];
+    unsigned long long e = chain_exclusive((unsigned long long)s, tile, chain, sh, err);
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        long long idx = base + i;
-        if (idx < n) out[idx] = e;
-        e += v[i];
+        if (base + i < n) out[base + i] = (int)e;
+        e += (unsigned)v[i];
     }
-}
-
-size_t scan_scratch_ints(long long n) { return (size_t)((n + kScanTile - 1) / kScanTile) + 1; }
-
-int launch_exclusive_scan(const int* in, int* out, long long n, int* scratch, cudaStream_t st) {
-    if (n <= 0) return 0;
-    int nb = (int)((n + kScanTile - 1) / kScanTile);
-    k_scan_reduce<<<nb, kScanThreads, 0, st>>>(in, n, scratch);
-    k_scan_sums<<<1, kScanThreads, 0, st>>>(scratch, nb);
-    k_scan_apply<<<nb, kScanThreads, 0, st>>>(in, n, scratch, out);
-    return 3;
 }
 
 // ----------------------------------------------------------------------------
@@ -232,21 +168,39 @@ int launch_exclusive_scan(const int* in, int* out, long long n, int* scratch, cu
 // ----------------------------------------------------------------------------
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortRounds = 16;
-constexpr int kSortTile = kSortThreads * kSortRounds;  // 4096 keys
 constexpr int kMaxBuckets = 512;
+// Keys per tile: 16 per thread, or 4 while that leaves the tiles fewer than two
+// per SM (each round of a tile is a dependent step: 1e4 keys took 10 us for the
+// counts and 14 us for the scatter in 3 tiles of 4096).
+constexpr int kRoundsLong = 16, kRoundsShort = 4;
+static int sort_rounds(long long n) {
+    return n > 2ll * sm_count() * kSortThreads * kRoundsLong ? kRoundsLong : kRoundsShort;
+}
+static long long sort_tiles(long long n, int rounds) {
+    return (n + (long long)kSortThreads * rounds - 1) / ((long long)kSortThreads * rounds);
+}
 
+// Also clears the chain of the scan that follows.
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int* __restrict__ keys, long long n, int shift,
-                                                             int nbits, int n_tiles, int* __restrict__ counts) {
+                                                             int nbits, int n_tiles, int* __restrict__ counts,
+                                                             unsigned long long* __restrict__ chain, int n_chain) {
+    constexpr int kSortTile = kSortThreads * ROUNDS;
+    for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < n_chain; i += gridDim.x * kSortThreads) chain[i] = 0ull;
     __shared__ int hist[kMaxBuckets];
     const int nb = 1 << nbits, mask = nb - 1;
     for (int d = threadIdx.x; d < nb; d += blockDim.x) hist[d] = 0;
     __syncthreads();
     long long base = (long long)blockIdx.x * kSortTile;
-    for (int i = threadIdx.x; i < kSortTile; i += blockDim.x) {
-        long long idx = base + i;
-        if (idx < n) atomicAdd(&hist[(keys[idx] >> shift) & mask], 1);
+    int key[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const long long idx = base + r * kSortThreads + threadIdx.x;
+        key[r] = idx < n ? keys[idx] : -1;
     }
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r)
+        if (key[r] >= 0) atomicAdd(&hist[(key[r] >> shift) & mask], 1);
     __syncthreads();
     for (int d = threadIdx.x; d < nb; d += blockDim.x) counts[(long long)d * n_tiles + blockIdx.x] = hist[d];
 }
@@ -259,12 +213,14 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int* __restri
 // per-key scatter (tile offset of the digit + keys of that digit before it in
 // the tile): the sort is stable and its result does not depend on this
 // staging.
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const int* __restrict__ keys_in,
                                                                 const int* __restrict__ vals_in, long long n,
                                                                 int shift, int nbits, int n_tiles,
                                                                 const int* __restrict__ offsets,
                                                                 int* __restrict__ keys_out,
                                                                 int* __restrict__ vals_out) {
+    constexpr int kSortRounds = ROUNDS, kSortTile = kSortThreads * ROUNDS;
     // wcnt is dead once the local positions are known: the staged keys reuse it
     __shared__ int wcnt[kSortWarps][kMaxBuckets];  // 16 KB = kSortTile ints
     __shared__ int s_val[kSortTile];
@@ -283,9 +239,14 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const int* __res
     int key[kSortRounds], rank[kSortRounds];
 #pragma unroll
     for (int r = 0; r < kSortRounds; ++r) {
+        const long long idx = base + r * 32 + lane;
+        key[r] = idx < n ? keys_in[idx] : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < kSortRounds; ++r) {
         long long idx = base + r * 32 + lane;
         bool valid = idx < n;
-        int k = valid ? keys_in[idx] : 0;
+        int k = key[r];
         int d = valid ? ((k >> shift) & mask) : (nb + 1);
         unsigned peers = __match_any_sync(0xffffffffu, d);
         int before = valid ? wcnt[w][d] : 0;
@@ -293,7 +254,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const int* __res
         int leader = 31 - __clz(peers);
         if (valid && lane == leader) wcnt[w][d] = before + __popc(peers);
         __syncwarp();
-        key[r] = k;
         rank[r] = before + __popc(peers & lt);
     }
     __syncthreads();
@@ -365,7 +325,10 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const int* __res
 // however the particles are spread (a small galaxy in a large field leaves
 // runs of hundreds of thousands of empty segments, which one thread per
 // particle would write one after another).
-__global__ void k_seg_bounds(const int* __restrict__ skeys, long long n, int n_keys, int* __restrict__ seg_off) {
+// Also clears the chain of the work items' scan.
+__global__ void k_seg_bounds(const int* __restrict__ skeys, long long n, int n_keys, int* __restrict__ seg_off,
+                             unsigned long long* __restrict__ chain, int n_chain) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_chain; i += gridDim.x * blockDim.x) chain[i] = 0ull;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s <= n_keys;
          s += (long long)gridDim.x * blockDim.x) {
         long long lo = 0, hi = n;
@@ -377,46 +340,57 @@ __global__ void k_seg_bounds(const int* __restrict__ skeys, long long n, int n_k
     }
 }
 
-size_t sort_scratch_ints(long long n) {
-    long long n_tiles = (n + kSortTile - 1) / kSortTile;
-    long long counts = n_tiles * kMaxBuckets;
-    return (size_t)(2 * counts) + scan_scratch_ints(counts) + 16;
+size_t sort_scratch_ints(long long n, bool long_tiles) {
+    const long long counts = sort_tiles(n, long_tiles ? kRoundsLong : sort_rounds(n)) * kMaxBuckets;
+    return (size_t)(2 * counts) + 2 * chain_words((counts + kScanTile - 1) / kScanTile) + 2;
 }
 
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
-                       int* perm_out, int* seg_off, int* scratch, cudaStream_t st) {
+                       int* perm_out, int* seg_off, int* scratch, bool long_tiles, unsigned long long* next_chain,
+                       int n_next_chain, unsigned* err, cudaStream_t st) {
     int launches = 0;
     if (n > 0) {
         int bits = 1;
         while ((1ll << bits) < (long long)n_keys) ++bits;   // keys lie in [0, n_keys)
-        int passes = (bits + 8) / 9;
-        int per = (bits + passes - 1) / passes;
-        int n_tiles = (int)((n + kSortTile - 1) / kSortTile);
-        long long n_counts = (long long)n_tiles << per;
-        int* counts = scratch;
-        int* offs = scratch + n_counts;
-        int* sscr = offs + n_counts;
+        const int passes = (bits + 8) / 9;
+        const int per = (bits + passes - 1) / passes;
+        const bool short_tiles = !long_tiles && sort_rounds(n) == kRoundsShort;
+        const int n_tiles = (int)sort_tiles(n, short_tiles ? kRoundsShort : kRoundsLong);
+        const long long n_counts = (long long)n_tiles << per;
+        // the chain first, on an 8-byte boundary
+        unsigned long long* chain =
+            reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(scratch) + 7) & ~(uintptr_t)7);
+        int* counts = reinterpret_cast<int*>(chain + chain_words((n_counts + kScanTile - 1) / kScanTile));
+        int* offs = counts + n_counts;
         const int* kin = keys;
         const int* vin = nullptr;
         for (int ps = 0; ps < passes; ++ps) {
-            int shift = ps * per;
-            int nb = (ps == passes - 1) ? (bits - shift) : per;
+            const int shift = ps * per;
+            const int nb = (ps == passes - 1) ? (bits - shift) : per;
             // ping-pong so that the last pass lands in keys_out / perm_out
-            bool to_final = ((passes - 1 - ps) % 2) == 0;
+            const bool to_final = ((passes - 1 - ps) % 2) == 0;
             int* kout = to_final ? keys_out : keys_tmp;
             int* vout = to_final ? perm_out : vals_tmp;
-            long long cnt = (long long)n_tiles << nb;
-            k_radix_hist<<<n_tiles, kSortThreads, 0, st>>>(kin, n, shift, nb, n_tiles, counts);
-            launches += 1 + launch_exclusive_scan(counts, offs, cnt, sscr, st);
-            k_radix_scatter<<<n_tiles, kSortThreads, 0, st>>>(kin, vin, n, shift, nb, n_tiles, offs, kout, vout);
-            ++launches;
+            const long long cnt = (long long)n_tiles << nb;
+            const int n_scan = (int)((cnt + kScanTile - 1) / kScanTile);
+            const int n_chain = (int)chain_words(n_scan);
+            if (short_tiles)
+                k_radix_hist<kRoundsShort><<<n_tiles, kSortThreads, 0, st>>>(kin, n, shift, nb, n_tiles, counts, chain, n_chain);
+            else
+                k_radix_hist<kRoundsLong><<<n_tiles, kSortThreads, 0, st>>>(kin, n, shift, nb, n_tiles, counts, chain, n_chain);
+            k_scan<<<n_scan, kScanThreads, 0, st>>>(counts, cnt, offs, chain, err);
+            if (short_tiles)
+                k_radix_scatter<kRoundsShort><<<n_tiles, kSortThreads, 0, st>>>(kin, vin, n, shift, nb, n_tiles, offs, kout, vout);
+            else
+                k_radix_scatter<kRoundsLong><<<n_tiles, kSortThreads, 0, st>>>(kin, vin, n, shift, nb, n_tiles, offs, kout, vout);
+            launches += 3;
             kin = kout;
             vin = vout;
         }
     }
     long long nt = ((long long)n_keys + 1 + 255) / 256;
     if (nt > 16ll * sm_count()) nt = 16ll * sm_count();
-    k_seg_bounds<<<(int)nt, 256, 0, st>>>(keys_out, n, n_keys, seg_off);
+    k_seg_bounds<<<(int)nt, 256, 0, st>>>(keys_out, n, n_keys, seg_off, next_chain, n_next_chain);
     return launches + 1;
 }
 
