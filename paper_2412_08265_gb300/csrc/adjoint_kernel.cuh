@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
                 if (threadIdx.x == 0) atomicOr(P.err, kErrTmaTimeout);
                 return;
             }
-            constexpr int GR = RUBIX_ADJ_GRAB;
+            const int GR = claim_size(nv, RUBIX_ADJ_GRAB);
             while (true) {
                 int v0 = 0;
                 if (lane == 0) v0 = atomicAdd(s_next, GR);

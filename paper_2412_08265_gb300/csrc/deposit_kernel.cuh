@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
             }
 
             const int nv = *s_nv;
-            constexpr int G = RUBIX_DEP_GRAB;
+            const int G = claim_size(nv, RUBIX_DEP_GRAB);
             while (true) {
                 int v0 = 0;
                 if (lane == 0) v0 = atomicAdd(s_next, G);
