@@ -497,9 +497,9 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
                 if (threadIdx.x == 0) atomicOr(P.err, kErrTmaTimeout);
                 return;
             }
-            const int GR = claim_size(nv, RUBIX_ADJ_GRAB);
+            int v0 = 0;
             while (true) {
-                int v0 = 0;
+                const int GR = claim_size(nv - v0, RUBIX_ADJ_GRAB);
                 if (lane == 0) v0 = atomicAdd(s_next, GR);
                 v0 = __shfl_sync(0xffffffffu, v0, 0);
                 if (v0 >= nv) break;

@@ -211,6 +211,48 @@ __device__ __forceinline__ void rounds_phi(const float4 w4, const TileCtx& C, co
     }
 }
 
+// A in (1, kGatherMax): a round's 32 bins lie on up to 64 nodes. Lanes on their
+// own bins' nodes would collide on the banks (nodes 16 apart share one: the two
+// reads per bin took 16 wavefronts, half of them conflicts), so lane l reads
+// nodes n_0 + l and, as far as the round reaches, n_0 + 32 + l, conflict-free,
+// and each bin takes its two nodes' M from those lanes: 7 to 8 wavefronts and
+// four shuffles. Survey grid (dt/dj 1.58, 5e5 particles): 1003 -> 961 us per
+// forward; the chain of a round is longer, so CTAs of few items (1e4 particles:
+// 112 us, 120 with it) read twice.
+constexpr float kGatherMax = 1.95f;
+template <int R, int B>
+__device__ __forceinline__ void rounds_gather(const float4 w4, const TileCtx& C, const LanePos& L, uint32_t base0,
+                                              float f, float ib, int il, int hi, int lane, float (&acc)[R]) {
+    const uint32_t p8 = (uint32_t)C.pitch * 8u;
+    const uint32_t sib = (uint32_t)(int)ib * p8;
+#pragma unroll
+    for (int r = 0; r < R; r += 2) {
+        const int r1 = r + 1 < R ? r + 1 : r;
+        const float2 rr = make_float2((float)r, (float)r1), fb2 = make_float2(L.fb, L.fb);
+        const float2 mg = make_float2(kMagic, kMagic);
+        const float2 x = __ffma2_rn(rr, fb2, make_float2(L.x0, L.x0));
+        const float2 y = __fadd2_rd(x, mg);
+        const float2 fl = __fadd2_rn(y, make_float2(-kMagic, -kMagic));
+        const float2 phi = __fadd2_rn(x, make_float2(-fl.x, -fl.y));
+        const float2 y0 = __fadd2_rd(__ffma2_rn(rr, fb2, make_float2(f, f)), mg);  // lane 0's
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (r + h >= R) break;
+            const int b0 = __float_as_int(h ? y0.y : y0.x);
+            const uint32_t a = base0 + (uint32_t)b0 * p8;
+            base0 += sib;
+            const int k = il + __float_as_int(h ? y.y : y.x) - b0;  // the bin's node, from lane 0's
+            const float Ma = quad_dot(w4, lds_quad(a, C));
+            float Mb = 0.f;
+            if (lane <= hi) Mb = quad_dot(w4, lds_quad(a + 32u * p8, C));
+            const float sa = __shfl_sync(0xffffffffu, Ma, k), sb = __shfl_sync(0xffffffffu, Mb, k);
+            const float ta = __shfl_sync(0xffffffffu, Ma, k + 1), tb = __shfl_sync(0xffffffffu, Mb, k + 1);
+            const float m0 = k < 32 ? sa : sb, m1 = k < 31 ? ta : tb;
+            acc[r + h] += fmaf(h ? phi.y : phi.x, m1 - m0, m0);
+        }
+    }
+}
+
 // ----------------------------------------------------------------------------
 // Rounds of bin means (flux-conserving resampling). The record maps j to bin
 // j's lower edge e_j = t(j) - A/2 (node units); bin j's value is the mean of
@@ -337,6 +379,7 @@ struct RoundCtx {
     float a0_1m;
     float ib, fbr;       // whole nodes of a round and the rest, at rest
     float il, fl;        // whole nodes of the lane's bins and the rest, at rest
+    bool gather;         // enough work in the CTA for rounds_gather
 };
 
 // Adds one particle's spectrum to acc (setup by every lane; warp-uniform path).
@@ -366,7 +409,11 @@ __device__ __forceinline__ void deposit_particle(const float4 w4, const float4 r
             mean_rounds_phi<R, B>(w4, C, L, T.ib, 1.f - delta, lane, acc);
         } else {
             if (KIND == 1 && (ef >> 30) == kPathMain) rounds_phi<R, B, true>(w4, C, L, T.ib, delta, lane, acc);
-            else rounds_phi<R, B, false>(w4, C, L, T.ib, delta, lane, acc);
+            else if (KIND == 2 && T.gather && delta < -0.03f && delta > 1.f - kGatherMax) {
+                // lanes of the second read: up to node floor(31 dt/dj) + 2 of the round's
+                const uint32_t base0 = C.slab + (kw + (uint32_t)lane) * p8 + (ef & 0x3fffffffu) - kMagicBits * p8;
+                rounds_gather<R, B>(w4, C, L, base0, f, T.ib, (int)T.il, (int)(31.f * (1.f - delta)) + 2 - 32, lane, acc);
+            } else rounds_phi<R, B, false>(w4, C, L, T.ib, delta, lane, acc);
         }
     } else {
         const float4 g4 = *map4;
@@ -382,7 +429,7 @@ constexpr int kJobChunk = 32;  // jobs per shared-memory work table
 // earlier bands' sum for later bands), then stored.
 template <int R, int KIND, bool MEAN>
 __device__ __forceinline__ void deposit_item(const DepositParams& P, const TileCtx& C, const DepJob& J, int t, int q0,
-                                             int q1, float* dst, int band, int lane, float lanef, float2 lref) {
+                                             int q1, float* dst, int band, int lane, float lanef, float2 lref, bool gather) {
     constexpr int B = kind_bins(KIND), BR = MEAN ? B - 1 : B, NR = MEAN ? R + 1 : R;
     const float4* __restrict__ rec4 = reinterpret_cast<const float4*>(J.rec);
     // the next particle's record is pulled into L1 while the current one is
@@ -411,6 +458,7 @@ __device__ __forceinline__ void deposit_item(const DepositParams& P, const TileC
     T.fbr = P.fbr[MEAN];
     T.il = lref.x;
     T.fl = lref.y;
+    T.gather = gather;
     for (int q = q0; q < q1; ++q) {
         if (q + 1 < q1) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec4 + 2 * (q + 1)));
         const float4 w4 = rec4[2 * q], r4 = rec4[2 * q + 1];
@@ -553,9 +601,10 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
             }
 
             const int nv = *s_nv;
-            const int G = claim_size(nv, RUBIX_DEP_GRAB);
+            const bool many = nv >= 2 * (int)(blockDim.x >> 5);
+            int v0 = 0;
             while (true) {
-                int v0 = 0;
+                const int G = claim_size(nv - v0, RUBIX_DEP_GRAB);
                 if (lane == 0) v0 = atomicAdd(s_next, G);
                 v0 = __shfl_sync(0xffffffffu, v0, 0);
                 if (v0 >= nv) break;
@@ -596,9 +645,9 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
                     float* dst = (pr < 0) ? J.cube + (long long)s * J.pitch
                                           : J.partials + (long long)pr * P.n_lambda;
                     if (MEANS && J.resample)
-                        deposit_item<R, KIND, true>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref);
+                        deposit_item<R, KIND, true>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref, many);
                     else
-                        deposit_item<R, KIND, false>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref);
+                        deposit_item<R, KIND, false>(P, C, J, (int)t, q0, q1, dst, band, lane, lanef, lref, many);
                 }
             }
         }

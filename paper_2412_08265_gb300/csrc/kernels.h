@@ -20,9 +20,10 @@ constexpr int kMaxBands = 32;
 int sm_count();
 
 // Deposit launch shape: threads per CTA (one CTA per SM: the SSP slab fills
-// shared memory; 896 threads leave 72 registers per thread).
+// shared memory; 1024 threads leave 64 registers per thread. Mid-size and large
+// galaxy, ms: 1024 threads 3.41 / 53.9, 896 3.49 / 55.9, 768 3.39 / 55.1).
 #ifndef RUBIX_DEP_THREADS
-#define RUBIX_DEP_THREADS 896
+#define RUBIX_DEP_THREADS 1024
 #endif
 // Deposit geometry: particles per work item, the line-of-sight speed (km/s)
 // the shared-memory slab's Doppler halo covers, and a fixed number of age
@@ -43,10 +44,10 @@ int sm_count();
 #ifndef RUBIX_DEP_COSTC0
 #define RUBIX_DEP_COSTC0 4
 #endif
-// Work items a warp claims at once (its first lanes look them up together),
-// in the deposit and in the adjoint.
+// Most work items a warp claims at once (its first lanes look them up together;
+// claim_size in tile.cuh), in the deposit and in the adjoint.
 #ifndef RUBIX_DEP_GRAB
-#define RUBIX_DEP_GRAB 4
+#define RUBIX_DEP_GRAB 3
 #endif
 #ifndef RUBIX_ADJ_GRAB
 #define RUBIX_ADJ_GRAB 2

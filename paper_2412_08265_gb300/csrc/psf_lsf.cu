@@ -113,18 +113,20 @@ __global__ void __launch_bounds__(256) k_psfy_noise(const ConvParams P, const fl
 //     zero fill outside the cube is the zero padding;
 //   dense rows of any alignment (a caller's cube): one bulk copy per spaxel of
 //     the 16-byte granules that hold its bins (DenseRows).
-// Warp w owns output column x0 + w:
-//   PSF along x: the 4 bins per lane of column w from the box's columns
-//     w .. w + 2 rp, into the warp's own row of px (so every bin the LSF
-//     needs, halo included, is computed once, by the warp that reads it);
-//   LSF along wavelength from the warp's px row (lanes RLa/4 .. 31 - RLa/4,
-//     bins 4q .. 4q + 3 of lane q, which are the tile's), then the rotating
-//     PSF-y register accumulators: the value of input row y_in is added, with
-//     weight gp[m], to the accumulator of output row y_in - rp + m (2 rp + 1
-//     per owned bin, static indices by unrolling the rows), and the output row
-//     y_in - rp is then complete: noise is added and it is written once.
+//   PSF along x: each warp takes four output columns over 32 bins, one bin per
+//     lane: 4 + 2 rp conflict-free 4-byte loads (at any row alignment) for four
+//     outputs; with one column and four bins per lane it was 2 rp + 1 16-byte
+//     loads, nearly three times the shared-memory wavefronts, which bound the
+//     kernel. Into px, every bin the LSF needs, halo included.
+//   LSF along wavelength: warp w owns output column x0 + w, lane q bins 4q ..
+//     4q + 3 of its px row (lanes RLa/4 .. 31 - RLa/4, the tile's). Then the PSF-y
+//     register accumulators: the value of input row y_in is added, with weight
+//     gp[m], to the accumulator of output row y_in - rp + m (2 rp + 1 per owned
+//     bin, each moved down one place by the same multiply-add), and the output
+//     row y_in - rp is then complete: noise is added and it is written once.
 // One CTA barrier per input row (every warp is done with the stage before it
-// is refilled); px is private to its warp. The terms of each output are summed
+// is refilled, and px is complete; a barrier per two or three rows measured no
+// faster). The terms of each output are summed
 // in the same order for both forms (PSF x, LSF, PSF y; each over its taps in
 // order), so they give the same bits.
 //
@@ -140,8 +142,9 @@ __global__ void __launch_bounds__(256) k_psfy_noise(const ConvParams P, const fl
 #endif
 constexpr int kTB = 128, kTX = kConvX, kTThreads = 256, kTWarps = kTThreads / 32;
 constexpr int kTS = RUBIX_PSF_TSTAGES;
+constexpr int kHead = 64;              // header, in floats: mbarriers, then the row bits
 static_assert(kTX == kTWarps, "one output column per warp");
-static_assert(kTS * 8 <= 32, "mbarriers before the row bits");
+static_assert(kTS * 8 <= 128, "mbarriers before the row bits");
 
 template <int RP, int RL, bool DENSE = false>
 struct TmaGeo {
@@ -152,7 +155,7 @@ struct TmaGeo {
     static constexpr int NV = 1 + RLa / 2;        // 16-byte loads per lane for 4 LSF outputs
     static constexpr int row = LW + (DENSE ? 4 : 0);  // stage row: dense rows start anywhere in a 16-byte granule
     static constexpr int stage_floats = (row * XW + 31) / 32 * 32;  // stages stay 128-byte aligned
-    static constexpr size_t smem = 128 + (size_t)kTS * stage_floats * 4 + (size_t)kTX * kTB * 4;
+    static constexpr size_t smem = 4 * kHead + (size_t)kTS * stage_floats * 4 + (size_t)2 * kTX * kTB * 4;
 };
 
 // Dense input rows: float cube [ny][nx][nl] at any 4-byte aligned address.
@@ -174,8 +177,8 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     constexpr int Q0 = G::RLa / 4, Q1 = 32 - G::RLa / 4;  // lanes whose bins are the tile's
     extern __shared__ __align__(1024) float smt[];
     uint64_t* bars = reinterpret_cast<uint64_t*>(smt);
-    float* stages = smt + 32;  // 128 bytes in
-    float* px = stages + kTS * G::stage_floats;  // [kTX][kTB] PSF-x output, one row per warp
+    float* stages = smt + kHead;
+    float* px = stages + kTS * G::stage_floats;  // [2][kTX][kTB] PSF-x output, alternating by row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int j0 = blockIdx.x * G::TL, x0 = blockIdx.y * kTX, y0 = blockIdx.z * P.ty;
     const int y1 = min(y0 + P.ty, P.ny);
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     }
     // which input rows hold anything for this CTA: rows outside the cube, or
     // without a particle within reach of these columns, are zero
-    unsigned* s_live = reinterpret_cast<unsigned*>(smt) + 8;
+    unsigned* s_live = reinterpret_cast<unsigned*>(smt) + 32;
     for (int i0 = warp * 32; i0 < n_rows; i0 += kTThreads) {
         const int y = y0 - RP + i0 + lane;
         const bool on = i0 + lane < n_rows && y >= 0 && y < P.ny &&
@@ -261,114 +264,105 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     for (int m = 0; m < NR; ++m)
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc[m][u] = 0.f;
-    float* prow = px + warp * kTB;
+    const float* prow = px;  // column warp's row of the current px buffer
+    // PSF-x: the warp's first column of the tile and the lane's bin of the box
+    const int c0 = (warp & 1) * 4, xb = (warp >> 1) * 32 + lane;
     const bool owns = lane >= Q0 && lane < Q1;
     const int x = x0 + warp;
     const int jl = j0 - G::RLa + 4 * lane;  // cube bin of the lane's first box bin
-    // dense rows: position (modulo 2^32) of tap 0's first bin in input row 0
+    // dense rows: position (modulo 2^32) of input column c0's first bin in input row 0
     const unsigned row_step = (unsigned)nx * (unsigned)nl;
-    const unsigned col0 = (unsigned)D.off + (unsigned)(y0 - RP) * row_step + (unsigned)((x - RP) * nl + j0 - G::RLa);
+    const unsigned col0 = (unsigned)D.off + (unsigned)(y0 - RP) * row_step + (unsigned)((x0 - RP + c0) * nl + j0 - G::RLa);
 
-    for (int ib = 0; ib < n_rows; ib += NR) {
+    // rows of `out` that are 16-byte aligned take 16-byte stores (others four
+    // 4-byte ones: bringing them into order through shared memory first cost more
+    // than it saved)
+    const bool vec = (nl & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+
+    for (int i = 0; i < n_rows; ++i) {
+        const bool has = live(i);  // uniform over the CTA
+        if (has) {
+            const int s = turn % kTS;
+            const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((turn / kTS) & 1), 2000000000ll);
+            float* pbuf = px + (turn & 1) * kTX * kTB;
+            if (ok) {
+                // PSF along x: 4 output columns from 4 + 2 RP input columns, one bin per lane
+                const float* src = stages + s * G::stage_floats + c0 * G::row + xb;
+                float c[4 + 2 * RP];
+                const unsigned p = col0 + (unsigned)i * row_step;  // DENSE: position of column c0's row
 #pragma unroll
-        for (int ph = 0; ph < NR; ++ph) {  // accumulator of output row y_in - RP + m is (ph + m) % NR
-            const int i = ib + ph;
-            if (i < n_rows) {
-                const bool has = live(i);  // uniform over the CTA
-                if (has) {
-                    const int s = turn % kTS;
-                    const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((turn / kTS) & 1), 2000000000ll);
-                    if (ok) {
-                        float a[4] = {0.f, 0.f, 0.f, 0.f};
-                        if constexpr (!DENSE) {
-                            // PSF along x: box columns warp .. warp + 2 RP, bins 4 lane .. 4 lane + 3
-                            const float* src = stages + s * G::stage_floats + warp * G::row + 4 * lane;
+                for (int d = 0; d < 4 + 2 * RP; ++d)
+                    c[d] = src[d * G::row + (DENSE ? (int)((p + (unsigned)(d * nl)) & 3u) : 0)];
+                const bool in = !DENSE || (j0 - G::RLa + xb >= 0 && j0 - G::RLa + xb < nl);
 #pragma unroll
-                            for (int d = 0; d < NR; ++d) {
-                                const float4 c = *reinterpret_cast<const float4*>(src + d * G::row);
-                                a[0] = fmaf(gp[d], c.x, a[0]);
-                                a[1] = fmaf(gp[d], c.y, a[1]);
-                                a[2] = fmaf(gp[d], c.z, a[2]);
-                                a[3] = fmaf(gp[d], c.w, a[3]);
-                            }
-                            *reinterpret_cast<float4*>(prow + 4 * lane) = make_float4(a[0], a[1], a[2], a[3]);
-                        } else {
-                            // bins lane + 32 u: a row starts anywhere in its first granule
-                            const unsigned p = col0 + (unsigned)i * row_step;  // its position, modulo 2^32
-                            const float* stage = stages + s * G::stage_floats + lane;
+                for (int q = 0; q < 4; ++q) {
+                    float a = 0.f;
 #pragma unroll
-                            for (int d = 0; d < NR; ++d) {
-                                const float* src = stage + (warp + d) * G::row + ((p + (unsigned)(d * nl)) & 3u);
-                                float c[4];
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) c[u] = src[32 * u];
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) a[u] = fmaf(gp[d], c[u], a[u]);
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const int j = j0 - G::RLa + lane + 32 * u;
-                                prow[lane + 32 * u] = (j >= 0 && j < nl) ? a[u] : 0.f;
-                            }
-                        }
-                    }
-                    if (__syncthreads_or(!ok)) {
-                        // a load did not complete in time: record it, let the copies in
-                        // flight land (bounded), and stop
-                        if (threadIdx.x == 0) {
-                            if (P.err) atomicOr(P.err, kErrTmaTimeout);
-                            for (int r = turn; r < issued; ++r)
-                                mbar_wait_bounded(&bars[r % kTS], (uint32_t)((r / kTS) & 1), 200000000ll);
-                        }
-                        return;
-                    }
-                    // every warp is done with stage s (and the barrier made this
-                    // warp's px row visible to its lanes): refill it
-                    ++turn;
-                    if (warp == 0) issue_next();
+                    for (int d = 0; d < NR; ++d) a = fmaf(gp[d], c[q + d], a);
+                    pbuf[(c0 + q) * kTB + xb] = in ? a : 0.f;
                 }
-                const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
-                if (owns) {
-                    if (has) {
-                        // LSF along wavelength from px: bins 4 lane - RLa .. 4 lane + 3 + RLa
-                        const float4* r4 = reinterpret_cast<const float4*>(prow + 4 * lane - G::RLa);
-                        float v[4 * G::NV];
-#pragma unroll
-                        for (int c = 0; c < G::NV; ++c) {
-                            const float4 t = r4[c];
-                            v[4 * c] = t.x;
-                            v[4 * c + 1] = t.y;
-                            v[4 * c + 2] = t.z;
-                            v[4 * c + 3] = t.w;
-                        }
-                        float o[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            float b = 0.f;
-#pragma unroll
-                            for (int d = 0; d <= 2 * RL; ++d) b = fmaf(gl[d], v[u + d + G::RLa - RL], b);
-                            o[u] = b;
-                        }
-#pragma unroll
-                        for (int m = 0; m < NR; ++m)
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) acc[(ph + m) % NR][u] = fmaf(gp[m], o[u], acc[(ph + m) % NR][u]);
-                    }
-                    float* done = acc[ph % NR];
-                    if (y_done >= y0 && x < nx) {
-                        const long long idx = ((long long)y_done * nx + x) * nl + jl;
-                        float4 v = make_float4(done[0], done[1], done[2], done[3]);
-                        if constexpr (NOISE) v = add_noise4(v, idx, P.noise_inv_s2n, P.seed_lo, P.seed_hi);
-                        float* o = out + idx;
-                        if (jl < nl) o[0] = v.x;
-                        if (jl + 1 < nl) o[1] = v.y;
-                        if (jl + 2 < nl) o[2] = v.z;
-                        if (jl + 3 < nl) o[3] = v.w;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) done[u] = 0.f;
+            }
+            if (__syncthreads_or(!ok)) {
+                // a load did not complete in time: record it, let the copies in
+                // flight land (bounded), and stop
+                if (threadIdx.x == 0) {
+                    if (P.err) atomicOr(P.err, kErrTmaTimeout);
+                    for (int r = turn; r < issued; ++r)
+                        mbar_wait_bounded(&bars[r % kTS], (uint32_t)((r / kTS) & 1), 200000000ll);
                 }
-                __syncwarp();  // the warp's px row is rewritten by the next input row
+                return;
+            }
+            // every warp is done with stage s: refill it. The barrier also made
+            // the px rows visible; they alternate, so that the next row's are not
+            // written before every warp has read these
+            prow = pbuf + warp * kTB;
+            ++turn;
+            if (warp == 0) issue_next();
+        }
+        float o[4] = {0.f, 0.f, 0.f, 0.f};
+        if (has && owns) {
+            // LSF along wavelength from px: bins 4 lane - RLa .. 4 lane + 3 + RLa
+            const float4* r4 = reinterpret_cast<const float4*>(prow + 4 * lane - G::RLa);
+            float v[4 * G::NV];
+#pragma unroll
+            for (int c = 0; c < G::NV; ++c) {
+                const float4 t = r4[c];
+                v[4 * c] = t.x;
+                v[4 * c + 1] = t.y;
+                v[4 * c + 2] = t.z;
+                v[4 * c + 3] = t.w;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float b = 0.f;
+#pragma unroll
+                for (int d = 0; d <= 2 * RL; ++d) b = fmaf(gl[d], v[u + d + G::RLa - RL], b);
+                o[u] = b;
+            }
+        }
+        // acc[m] holds output row y_in - RP + m - 1 until this row's share moves it
+        // down by one: no rotation, so the loop stays short (unrolled by 2 rp + 1
+        // rows it waited on instruction fetches)
+#pragma unroll
+        for (int m = 0; m < NR; ++m)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[m][u] = fmaf(gp[m], o[u], m + 1 < NR ? acc[m + 1][u] : 0.f);
+        const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
+        const bool write = y_done >= y0 && x < nx;
+        float* orow = out + ((long long)y_done * nx + x) * nl + j0 - G::RLa;
+        float4 v = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+        if constexpr (NOISE) {
+            if (write && owns)
+                v = add_noise4(v, ((long long)y_done * nx + x) * nl + jl, P.noise_inv_s2n, P.seed_lo, P.seed_hi);
+        }
+        if (write && owns) {
+            if (vec) {
+                if (jl < nl) *reinterpret_cast<float4*>(orow + 4 * lane) = v;
+            } else {
+                if (jl < nl) orow[4 * lane] = v.x;
+                if (jl + 1 < nl) orow[4 * lane + 1] = v.y;
+                if (jl + 2 < nl) orow[4 * lane + 2] = v.z;
+                if (jl + 3 < nl) orow[4 * lane + 3] = v.w;
             }
         }
     }
@@ -395,7 +389,7 @@ bool conv_tma_box(int rp, int rl, unsigned box[2]) {
 // resident CTAs with the fewest input rows (each CTA reads 2 rp rows more than it
 // writes). One wave of 150-row CTAs is best for 150 x 150 spaxels x 3721 bins; a
 // 25 x 25 x 1000 cube runs 36 CTAs unsplit.
-constexpr int kMaxTY = 600;  // input rows (ty + 2 rp) have a bit each in the kernel's 96-byte header
+constexpr int kMaxTY = 600;  // input rows (ty + 2 rp) have a bit each in the kernel's header
 static int rows_per_cta(int ny, int rp, long long columns) {
     const long long slots = (long long)RUBIX_PSF_TMINB * sm_count();
     int best = ny;

@@ -159,11 +159,15 @@ __device__ __forceinline__ void fill_slab16(const TileCtx& C) {
     }
 }
 
-// Work items a warp claims at once out of nv: one where claims of `most` would
-// leave a warp fewer than two (a small galaxy's CTA holds a dozen items: claims
-// of four kept three of its 28 warps busy; deposit of 1e4 particles 98 -> 42 us).
-__device__ __forceinline__ int claim_size(int nv, int most) {
-    return nv < 2 * most * (int)(blockDim.x >> 5) ? 1 : most;
+// Work items a warp claims at once with `left` of the band's still to claim:
+// `most` while every warp has plenty, then two, one at a time at the end, where
+// the band's barrier waits for the last warp (claims of four throughout: 3.41 ms
+// on the mid-size galaxy against 3.27, and 25 of a CTA's warps idle on a galaxy
+// of 1e4 particles; of two throughout: 53.96 ms on the large galaxy against 53.6,
+// where each claim's look-up chain counts).
+__device__ __forceinline__ int claim_size(int left, int most) {
+    const int nw = (int)(blockDim.x >> 5);
+    return left > 40 * nw ? most : (left > 2 * nw ? 2 : 1);
 }
 
 // Mass-weighted bilinear template value at one node: sum_c w_c q_c.
