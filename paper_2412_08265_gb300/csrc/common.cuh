@@ -63,17 +63,20 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 // stops using the buffer instead of spinning forever).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long max_cycles) {
     const uint32_t a = smem_addr(bar);
-    const long long t0 = clock64();
-    while (true) {
-        uint32_t done;
+    auto done = [&]() {
+        uint32_t d;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
+            : "=r"(d)
             : "r"(a), "r"(parity)
             : "memory");
-        if (done) return true;
+        return d != 0;
+    };
+    if (done()) return true;  // (no clock read when the data is there)
+    const long long t0 = clock64();
+    while (!done())
         if (clock64() - t0 > max_cycles) return false;
-    }
+    return true;
 }
 
 // Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) from

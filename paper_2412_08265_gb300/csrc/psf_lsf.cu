@@ -259,11 +259,9 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
         for (int k = 0; k < kTS; ++k) issue_next();
     int turn = 0;  // live rows taken
 
-    float acc[NR][4];
+    float2 acc[NR][2];
 #pragma unroll
-    for (int m = 0; m < NR; ++m)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[m][u] = 0.f;
+    for (int m = 0; m < NR; ++m) acc[m][0] = acc[m][1] = make_float2(0.f, 0.f);
     const float* prow = px;  // column warp's row of the current px buffer
     // PSF-x: the warp's first column of the tile and the lane's bin of the box
     const int c0 = (warp & 1) * 4, xb = (warp >> 1) * 32 + lane;
@@ -279,8 +277,12 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     // than it saved)
     const bool vec = (nl & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
 
-    for (int i = 0; i < n_rows; ++i) {
-        const bool has = live(i);  // uniform over the CTA
+    float* orow = out + ((long long)(y0 - 2 * RP) * nx + x) * nl + j0 - G::RLa;  // of the row input row i completes
+    const long long ostep = (long long)nx * nl;
+    unsigned bits = 0;
+    for (int i = 0; i < n_rows; ++i, orow += ostep, bits >>= 1) {
+        if ((i & 31) == 0) bits = s_live[i >> 5];
+        const bool has = bits & 1u;  // uniform over the CTA
         if (has) {
             const int s = turn % kTS;
             const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((turn / kTS) & 1), 2000000000ll);
@@ -343,14 +345,16 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
         // acc[m] holds output row y_in - RP + m - 1 until this row's share moves it
         // down by one: no rotation, so the loop stays short (unrolled by 2 rp + 1
         // rows it waited on instruction fetches)
+        const float2 o01 = make_float2(o[0], o[1]), o23 = make_float2(o[2], o[3]);
 #pragma unroll
-        for (int m = 0; m < NR; ++m)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[m][u] = fmaf(gp[m], o[u], m + 1 < NR ? acc[m + 1][u] : 0.f);
+        for (int m = 0; m < NR; ++m) {
+            const float2 g2 = make_float2(gp[m], gp[m]);
+            acc[m][0] = __ffma2_rn(g2, o01, m + 1 < NR ? acc[m + 1][0] : make_float2(0.f, 0.f));
+            acc[m][1] = __ffma2_rn(g2, o23, m + 1 < NR ? acc[m + 1][1] : make_float2(0.f, 0.f));
+        }
         const int y_done = y0 + i - 2 * RP;  // output row completed by this input row
         const bool write = y_done >= y0 && x < nx;
-        float* orow = out + ((long long)y_done * nx + x) * nl + j0 - G::RLa;
-        float4 v = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+        float4 v = make_float4(acc[0][0].x, acc[0][0].y, acc[0][1].x, acc[0][1].y);
         if constexpr (NOISE) {
             if (write && owns)
                 v = add_noise4(v, ((long long)y_done * nx + x) * nl + jl, P.noise_inv_s2n, P.seed_lo, P.seed_hi);
