@@ -63,15 +63,6 @@ PFN_encodeTiled_t get_encode_tiled() {
     return fn;
 }
 
-// Round-to-nearest-even FP32 -> BF16 (bit manipulation; NaN kept quiet).
-uint16_t f32_to_bf16(float f) {
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    if ((u & 0x7fffffffu) > 0x7f800000u) return (uint16_t)((u >> 16) | 0x40);
-    u += 0x7fffu + ((u >> 16) & 1u);
-    return (uint16_t)(u >> 16);
-}
-
 void gauss_kernel(double sigma, int r, float* out) {
     std::vector<double> k(2 * r + 1);
     double s = 0.0;
@@ -379,83 +370,32 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
     // grid of one metallicity repeats its entry). One block per age band,
     // node-major, pad zero node rows on both sides, in the storage dtype: FP32
     // pairs, or two BF16 / FP16 bit patterns (first | second << 16) that the
-    // kernels widen to FP32 exactly ----
+    // kernels widen to FP32 exactly; laid out on the device (k_build_pairs) ----
     G.qdt = (S.dtype == RUBIX_F32) ? 0 : (S.dtype == RUBIX_BF16 ? 1 : 2);
     static_assert(kDepHeader % 128 == 0, "slab must start 16-byte aligned");
     {
-        const int da = (S.n_age > 1) ? 1 : 0;
         const size_t rows = (size_t)S.n_ls + 2 * (size_t)G.pad;
         G.band_stride = (long long)((rows * G.pitch + 3) / 4 * 4);
-        const size_t total = (size_t)G.band_stride * G.n_bands, entry = G.qdt ? 4 : 8;
-        std::vector<unsigned char> host(total * entry, 0);
-        // the adjoint's entries, FP32: the template and its difference to the
-        // next age's, so that its sums of age derivatives do not cancel
-        std::vector<float2> adj(with_adjoint ? total : 0, make_float2(0.f, 0.f));
-        auto bits16 = [&](float f) -> uint32_t {
-            if (S.dtype == RUBIX_BF16) return f32_to_bf16(f);
-            const __half hv = __float2half_rn(f);
-            uint16_t b;
-            std::memcpy(&b, &hv, 2);
-            return b;
-        };
-        auto widen16 = [&](uint32_t u) -> float {
-            if (S.dtype == RUBIX_F16) {
-                const uint16_t h16 = (uint16_t)u;
-                __half hv;
-                std::memcpy(&hv, &h16, 2);
-                return __half2float(hv);
+        const size_t total = (size_t)G.band_stride * G.n_bands, nt = (size_t)S.n_age * S.n_Z * S.n_ls;
+        std::vector<float> tf(nt);
+        for (size_t i = 0; i < nt; ++i) tf[i] = (float)ssp->spectra[i];
+        float* d_t = nullptr;
+        const bool ok = cudaMalloc(&h->d_pair, total * (G.qdt ? 4 : 8)) == cudaSuccess &&
+                        (!with_adjoint || dalloc_sync(&h->d_pair_adj, total) == cudaSuccess) &&
+                        dalloc_sync(&d_t, nt) == cudaSuccess;
+        cudaError_t e = cudaSuccess;
+        if (ok) {
+            G.pair = h->d_pair;
+            e = cudaMemcpy(d_t, tf.data(), nt * sizeof(float), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) {
+                launch_build_pairs(G, best.apb, S.n_age, S.n_Z, d_t, h->d_pair, h->d_pair_adj, nullptr);
+                e = cudaDeviceSynchronize();
             }
-            u <<= 16;
-            float f;
-            std::memcpy(&f, &u, 4);
-            return f;
-        };
-        // every template value once, as stored, then node by node (both passes
-        // write in order; the second reads n_age * n_Z streams)
-        const size_t nt = (size_t)S.n_age * S.n_Z;
-        std::vector<uint16_t> t16(G.qdt ? nt * S.n_ls : 0);
-        std::vector<float> tf(!G.qdt || with_adjoint ? nt * S.n_ls : 0);
-        for (size_t i = 0; i < nt * S.n_ls; ++i) {
-            float f = (float)ssp->spectra[i];
-            if (G.qdt) {
-                t16[i] = (uint16_t)bits16(f);
-                f = widen16(t16[i]);
-            }
-            if (!tf.empty()) tf[i] = f;
         }
-        for (int b = 0; b < G.n_bands; ++b)
-            for (int k = 0; k < S.n_ls; ++k) {
-                size_t at = (size_t)b * G.band_stride + (size_t)(k + G.pad) * G.pitch;
-                for (int ia = b * best.apb; ia < std::min((b + 1) * best.apb, ca); ++ia)
-                    for (int z = 0; z < nzc; ++z, ++at) {
-                        const size_t t0 = ((size_t)ia * S.n_Z + std::min(z, S.n_Z - 1)) * S.n_ls + k;
-                        const size_t t1 = t0 + (size_t)da * S.n_Z * S.n_ls;
-                        if (G.qdt) {
-                            const uint32_t u = t16[t0] | ((uint32_t)t16[t1] << 16);
-                            std::memcpy(&host[at * 4], &u, 4);
-                        } else {
-                            const float v[2] = {tf[t0], tf[t1]};
-                            std::memcpy(&host[at * 8], v, 8);
-                        }
-                        if (with_adjoint) adj[at] = make_float2(tf[t0], tf[t1] - tf[t0]);
-                    }
-            }
-        if (cudaMalloc(&h->d_pair, total * entry) != cudaSuccess) {
-            h->d_pair = nullptr;
-            cudaGetLastError();
-            return bail(fail(RUBIX_ERR_OOM, "template alloc"));
-        }
-        if (cudaMemcpy(h->d_pair, host.data(), total * entry, cudaMemcpyHostToDevice) != cudaSuccess)
-            return bail(fail(RUBIX_ERR_CUDA, "template copy"));
-        G.pair = h->d_pair;
-        if (with_adjoint) {
-            if (dalloc_sync(&h->d_pair_adj, total)) {
-                cudaGetLastError();
-                return bail(fail(RUBIX_ERR_OOM, "template alloc"));
-            }
-            if (cudaMemcpy(h->d_pair_adj, adj.data(), total * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess)
-                return bail(fail(RUBIX_ERR_CUDA, "template copy"));
-        }
+        if (d_t) cudaFree(d_t);
+        cudaGetLastError();
+        if (!ok) return bail(fail(RUBIX_ERR_OOM, "template alloc"));
+        if (e != cudaSuccess) return bail(fail(RUBIX_ERR_CUDA, "template copy: %s", cudaGetErrorString(e)));
     }
     if (cudaDeviceSynchronize() != cudaSuccess)
         return bail(fail(RUBIX_ERR_CUDA, "SSP state: %s", cudaGetErrorString(cudaGetLastError())));

@@ -199,6 +199,13 @@ inline __host__ __device__ const void* band_ptr(const void* pair, int qdt, long 
     return static_cast<const char*>(pair) + (long long)band * band_stride * (qdt ? 4 : 8);
 }
 
+// Lays the templates t ([n_age][n_Z][n_ls] FP32) out as age pairs: `pair`
+// (SlabParams::pair) and, if not null, `adj` with entries (T, T(next age) - T) of
+// the same (storage-rounded) values, so that the adjoint's sums of age
+// derivatives do not cancel.
+int launch_build_pairs(const SlabParams& G, int apb, int n_age, int n_Z, const float* t, void* pair, float2* adj,
+                       cudaStream_t st);
+
 struct DepositParams : SlabParams {
     DepJob jobs[kMaxJobs];
     int n_jobs;

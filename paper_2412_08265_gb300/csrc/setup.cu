@@ -165,6 +165,49 @@ int launch_setup(const SetupParams& P, long long n_total, cudaStream_t st) {
 }
 
 // ----------------------------------------------------------------------------
+// Template layout (once per SSP grid): consecutive threads write consecutive
+// entries of a node row and read n_age * n_Z rows of templates (25 MB written
+// for the 50 x 10 x 3721 grid; on the host this took milliseconds).
+// ----------------------------------------------------------------------------
+__global__ void k_build_pairs(const SlabParams G, int apb, int n_age, int n_Z, const float* __restrict__ t,
+                              void* __restrict__ pair, float2* __restrict__ adj) {
+    const int nzc = max(n_Z, 2), ca = max(n_age - 1, 1);
+    const long long total = G.band_stride * G.n_bands;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int band = (int)(i / G.band_stride);
+        const long long r = i - band * G.band_stride;
+        const int k = (int)(r / G.pitch) - G.pad, e = (int)(r % G.pitch);
+        const int ia = band * apb + e / nzc, iz = min(e % nzc, n_Z - 1);
+        float v0 = 0.f, v1 = 0.f;  // zero rows outside the templates, zero entries past the band's
+        if (k >= 0 && k < G.n_ls && e < apb * nzc && ia < ca) {
+            v0 = t[((long long)ia * n_Z + iz) * G.n_ls + k];
+            v1 = t[((long long)min(ia + 1, n_age - 1) * n_Z + iz) * G.n_ls + k];
+        }
+        if (G.qdt == 1) {
+            const __nv_bfloat16 a = __float2bfloat16_rn(v0), b = __float2bfloat16_rn(v1);
+            static_cast<uint32_t*>(pair)[i] = __bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+            v0 = __bfloat162float(a);
+            v1 = __bfloat162float(b);
+        } else if (G.qdt == 2) {
+            const __half a = __float2half_rn(v0), b = __float2half_rn(v1);
+            static_cast<uint32_t*>(pair)[i] = __half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+            v0 = __half2float(a);
+            v1 = __half2float(b);
+        } else {
+            static_cast<float2*>(pair)[i] = make_float2(v0, v1);
+        }
+        if (adj) adj[i] = make_float2(v0, v1 - v0);
+    }
+}
+
+int launch_build_pairs(const SlabParams& G, int apb, int n_age, int n_Z, const float* t, void* pair, float2* adj,
+                       cudaStream_t st) {
+    k_build_pairs<<<16 * sm_count(), 256, 0, st>>>(G, apb, n_age, n_Z, t, pair, adj);
+    return 1;
+}
+
+// ----------------------------------------------------------------------------
 // Work items: one per <= chunk particles of a spaxel (all age bands), in one
 // launch over a chained scan (common.cuh) of the spaxels' items and partial
 // rows. Empty spaxels get no item: k_rows writes their rows. (Counts, two scans
