@@ -132,7 +132,9 @@ def check(status: int):
 
 
 def _call(name, *args):
-    return check(getattr(load(), name)(*args))
+    # the loaded library's function (argument conversion is its argtypes'); the
+    # lock of load() only until it has been loaded
+    return check(getattr(_lib or load(), name)(*args))
 
 
 # ---------------------------------------------------------------------------
@@ -146,21 +148,18 @@ def rubix_cube_create(ssp: rubix_ssp_grid, tel: rubix_telescope, max_particles: 
 
 def rubix_cube_forward(h: int, p: rubix_particles, noise_seed: int, noise_s2n: float, cube_out: int,
                        cube_on_device: int, stream: int) -> None:
-    _call("rubix_cube_forward", C.c_void_p(h), C.byref(p), C.c_uint64(noise_seed), C.c_float(noise_s2n),
-          C.c_void_p(cube_out), C.c_int32(cube_on_device), C.c_void_p(stream))
+    _call("rubix_cube_forward", h, C.byref(p), noise_seed, noise_s2n, cube_out, cube_on_device, stream)
 
 
 def rubix_cube_forward_tag(h: int) -> int:
     t = C.c_uint64()
-    _call("rubix_cube_forward_tag", C.c_void_p(h), C.byref(t))
+    _call("rubix_cube_forward_tag", h, C.byref(t))
     return int(t.value)
 
 
 def rubix_cube_backward(h: int, forward_tag: int, dL_dcube: int, d_mass: int, d_age: int, d_Z: int,
                         d_vlos: int, d_global: int, stream: int) -> None:
-    _call("rubix_cube_backward", C.c_void_p(h), C.c_uint64(forward_tag), C.c_void_p(dL_dcube),
-          C.c_void_p(d_mass), C.c_void_p(d_age), C.c_void_p(d_Z), C.c_void_p(d_vlos), C.c_void_p(d_global),
-          C.c_void_p(stream))
+    _call("rubix_cube_backward", h, forward_tag, dL_dcube, d_mass, d_age, d_Z, d_vlos, d_global, stream)
 
 
 def rubix_cube_destroy(h: int) -> None:

@@ -19,6 +19,14 @@ from . import capi
 SCALAR_KEYS = ("preprojected", "inclination", "azimuth", "position_angle")
 
 
+def _raw_stream(stream, device) -> int:
+    """The cudaStream_t of `stream`, or of the device's current stream (without
+    building a torch.cuda.Stream, which costs as much as three launches)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
 def _dev_f32(a, device) -> torch.Tensor:
     if isinstance(a, torch.Tensor):
         return a.to(device=device, dtype=torch.float32).contiguous()
@@ -31,6 +39,8 @@ class CubeModel:
     def __init__(self, ssp, telescope, template_dtype: str = "f32", max_particles: int = 1 << 16,
                  device: torch.device | str | None = None):
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
+        if self.device.index is None:
+            self.device = torch.device(self.device.type, torch.cuda.current_device())
         self.tel = telescope
         self.ssp = ssp
         self.template_dtype = template_dtype
@@ -111,10 +121,9 @@ class CubeModel:
             else self.device_particles(p)
         if out is None:
             out = torch.empty(self.cube_shape, dtype=torch.float32, device=self.device)
-        st = stream or torch.cuda.current_stream(self.device)
         cp = self.c_particles(d)
         capi.rubix_cube_forward(self.handle, cp, int(noise_seed), float(noise_s2n), out.data_ptr(), 1,
-                                st.cuda_stream)
+                                _raw_stream(stream, self.device))
         self._last = d  # keep the device arrays alive until the kernels have read them
         self.last_tag = capi.rubix_cube_forward_tag(self.handle)
         return out
@@ -128,11 +137,10 @@ class CubeModel:
         tag = self.last_tag if forward_tag is None else int(forward_tag)
         g = [torch.empty(n, dtype=torch.float32, device=self.device) for _ in range(4)]
         glob = torch.empty(4, dtype=torch.float64, device=self.device) if want_global else None
-        st = stream or torch.cuda.current_stream(self.device)
         dc = dL_dcube.to(torch.float32).contiguous()
         capi.rubix_cube_backward(self.handle, tag, dc.data_ptr(), g[0].data_ptr(), g[1].data_ptr(),
                                  g[2].data_ptr(), g[3].data_ptr(), glob.data_ptr() if glob is not None else 0,
-                                 st.cuda_stream)
+                                 _raw_stream(stream, self.device))
         return (*g, glob)
 
     def spaxel_keys(self, p, stream=None) -> torch.Tensor:
@@ -180,9 +188,11 @@ class RubixCube(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, mass, age, Z, v_los, x, y, model: CubeModel):
-        d = {"x": x.detach().contiguous(), "y": y.detach().contiguous(), "mass": mass.detach().contiguous(),
-             "age": age.detach().contiguous(), "Z": Z.detach().contiguous(),
-             "v_los": v_los.detach().contiguous(), "preprojected": True, "inclination": 0.0}
+        d = {"x": x, "y": y, "mass": mass, "age": age, "Z": Z, "v_los": v_los}
+        for k, v in d.items():
+            # the model keeps these arrays until its next forward: without their graphs
+            d[k] = (v.detach() if v.requires_grad else v).contiguous()
+        d["preprojected"], d["inclination"] = True, 0.0
         cube = model.forward(d)
         ctx.model = model
         ctx.forward_tag = model.last_tag
