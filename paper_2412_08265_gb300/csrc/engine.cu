@@ -413,12 +413,31 @@ struct Buf {
     size_t bytes;
 };
 
+// Particles per work item of a galaxy of n: RUBIX_DEP_CHUNK, or less where that
+// would leave a warp of the deposit fewer than about eight full items a forward,
+// too few to even out their lengths (5e5 particles on the survey grid: 976 us
+// with 256, 872 with 64; 2e5 particles, gradient step with bin means: 3.72 and
+// 3.60 ms; on the mid-size and large galaxies smaller items cost 1 - 5 %). It
+// depends on the request alone, so that its cube does not depend on the plan.
+int item_chunk(const SspState& S, long long n) {
+    const double items = (double)n * S.geo.n_tiles / ((double)S.n_sm * (S.dep_threads / 32) * 8.0);
+    int c = RUBIX_DEP_CHUNK;
+    while (c > RUBIX_DEP_CHUNK / 4 && c > items) c /= 2;
+    return c;
+}
+// The most of n' / item_chunk(n') over n' <= n (the smaller chunks end at a
+// known count).
+long long max_chunks(const SspState& S, long long n) {
+    const long long lim = (long long)RUBIX_DEP_CHUNK * S.n_sm * (S.dep_threads / 32) * 8 / std::max(S.geo.n_tiles, 1) + 1;
+    return std::max(n / RUBIX_DEP_CHUNK, std::min(n, lim) / (RUBIX_DEP_CHUNK / 4));
+}
+
 // Every device buffer of a plan for n particles, with its size.
 std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda, long long n, bool with_out,
                               bool with_grad, bool need_tmp, bool staging, int pitch0) {
     const size_t N = (size_t)std::max(n, 1ll);
-    const long long item_cap = (long long)n_s + n / S.chunk + 2;
-    const long long part_cap = 2 * (n / S.chunk) + 2;
+    const long long item_cap = (long long)n_s + max_chunks(S, n) + 2;
+    const long long part_cap = 2 * max_chunks(S, n) + 2;
     const size_t cube = (size_t)n_s * n_lambda * sizeof(float);
     std::vector<Buf> v;
     if (staging)
@@ -544,8 +563,8 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
     P->pitch0 = cube0_pitch(C.rp, C.rl, tel->n_lambda);
     P->has_conv_map = false;
     P->cap = std::max(n, 1ll);
-    P->item_cap = (long long)P->n_s + P->cap / S->chunk + 2;
-    P->part_cap = 2 * (P->cap / S->chunk) + 2;
+    P->item_cap = (long long)P->n_s + max_chunks(*S, P->cap) + 2;
+    P->part_cap = 2 * max_chunks(*S, P->cap) + 2;
     const bool need_tmp = psf_lsf_needs_tmp(C.rp, C.rl);
     P->bytes = 0;
     const int fail_at = fault_alloc_at();
@@ -731,7 +750,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     IP.seg_off = P.d_seg_off;
     IP.n_s = P.n_s;
     IP.n_bands = S.geo.n_bands;
-    IP.chunk = S.chunk;
+    IP.chunk = item_chunk(S, n);
     IP.item_off = P.d_item_off;
     IP.part_off = P.d_part_off;
     IP.items = P.d_items;

@@ -48,7 +48,7 @@ struct SspState {
     int* d_tile_klo = nullptr;
     unsigned* d_tile_ref = nullptr;
     float2* d_lane_ref = nullptr;
-    int dep_ctas = 0, dep_threads = RUBIX_DEP_THREADS, chunk = RUBIX_DEP_CHUNK;
+    int dep_ctas = 0, dep_threads = RUBIX_DEP_THREADS;
     unsigned* d_err = nullptr;              // device error word (kernel bit flags)
     unsigned long long* d_slow = nullptr;   // (particle, tile) pairs on the global-memory path
 };

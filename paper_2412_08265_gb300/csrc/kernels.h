@@ -25,7 +25,7 @@ int sm_count();
 #ifndef RUBIX_DEP_THREADS
 #define RUBIX_DEP_THREADS 1024
 #endif
-// Deposit geometry: particles per work item, the line-of-sight speed (km/s)
+// Deposit geometry: most particles per work item, the line-of-sight speed (km/s)
 // the shared-memory slab's Doppler halo covers, and a fixed number of age
 // bands (0 = chosen by the cost estimate).
 #ifndef RUBIX_DEP_CHUNK
