@@ -32,33 +32,52 @@ struct AdjSums {
     float sm, sa, sz, sv;
 };
 
-// The slab holds, for each age cell and metallicity, the template and its
-// difference to the next age's: a node's entries are (T0, A0) and (T1, A1) at
-// the cell's two metallicities, and with the particle at (ta, tz) in the cell
+// A node's entries, by kind. Kind 0: the deposit's age pairs, the cell's four
+// corners (T00, T10), (T01, T11), and sums per corner: four corners' rounding
+// errors average in each form. Kinds 1, 2: each template and its difference to
+// the next age's, (T0, A0), (T1, A1), and the second entry's difference to the
+// first taken at the node (lds_diff): the sums of a derivative do not cancel
+// (metallicity gradient to 1e-7 where corner sums give 1e-6; the two packed
+// additions per node it takes cost 6 % on kind 0's shorter rounds).
 //   S = (1 - tz)(T0 + ta A0) + tz (T1 + ta A1),  dS/dta = (1 - tz) A0 + tz A1,
-//   dS/dtz = (T1 - T0) + ta (A1 - A0).
+//   dS/dtz = (T1 - T0) + ta (A1 - A0),  A = T(next age) - T.
 struct Forms {
     float m, a, z;
 };
+template <int KIND>
 __device__ __forceinline__ Forms node_forms(const float2 w, const Quad& q) {
-    const float ty = 1.f - w.y;
+    const float ty = 1.f - w.y, tx = 1.f - w.x;
     Forms F;
-    F.m = fmaf(ty, fmaf(w.x, q.a.y, q.a.x), __fmul_rn(w.y, fmaf(w.x, q.b.y, q.b.x)));
-    F.a = fmaf(ty, q.a.y, __fmul_rn(w.y, q.b.y));
-    F.z = fmaf(w.x, q.b.y - q.a.y, q.b.x - q.a.x);
+    if (KIND == 0) {
+        F.m = fmaf(ty, fmaf(w.x, q.a.y, __fmul_rn(tx, q.a.x)), __fmul_rn(w.y, fmaf(w.x, q.b.y, __fmul_rn(tx, q.b.x))));
+        F.a = fmaf(ty, q.a.y - q.a.x, __fmul_rn(w.y, q.b.y - q.b.x));
+        F.z = fmaf(tx, q.b.x - q.a.x, __fmul_rn(w.x, q.b.y - q.a.y));
+    } else {
+        F.m = fmaf(ty, fmaf(w.x, q.a.y, q.a.x), __fmul_rn(w.y, fmaf(w.x, q.b.y, q.b.x)));
+        F.a = fmaf(ty, q.a.y, __fmul_rn(w.y, q.b.y));
+        F.z = fmaf(w.x, q.b.y - q.a.y, q.b.x - q.a.x);
+    }
     return F;
 }
 
-// The four sums from per-entry sums (times su: U). DIFF: the second entry's
-// sums are of its difference to the first (T1 - T0, A1 - A0).
-template <bool DIFF>
+// The four sums from the sums over corners (kind 0) or over entries and their
+// differences; U is to be scaled by su.
+template <int KIND>
 __device__ __forceinline__ AdjSums entry_sums(const float2 w, float su, float2 U0, float2 U1, float2 V0, float2 V1) {
-    const float ty = DIFF ? 1.f : 1.f - w.y;
     AdjSums S;
-    S.sm = su * fmaf(ty, fmaf(w.x, U0.y, U0.x), __fmul_rn(w.y, fmaf(w.x, U1.y, U1.x)));
-    S.sa = su * fmaf(ty, U0.y, __fmul_rn(w.y, U1.y));
-    S.sz = su * (DIFF ? fmaf(w.x, U1.y, U1.x) : fmaf(w.x, U1.y - U0.y, U1.x - U0.x));
-    S.sv = fmaf(ty, fmaf(w.x, V0.y, V0.x), __fmul_rn(w.y, fmaf(w.x, V1.y, V1.x)));
+    if (KIND == 0) {
+        const float tx = 1.f - w.x, ty = 1.f - w.y;
+        const float w0 = tx * ty, w1 = w.x * ty, w2 = tx * w.y, w3 = w.x * w.y;
+        S.sm = su * fmaf(w0, U0.x, fmaf(w1, U0.y, fmaf(w2, U1.x, __fmul_rn(w3, U1.y))));
+        S.sa = su * fmaf(ty, U0.y - U0.x, __fmul_rn(w.y, U1.y - U1.x));
+        S.sz = su * fmaf(tx, U1.x - U0.x, __fmul_rn(w.x, U1.y - U0.y));
+        S.sv = fmaf(w0, V0.x, fmaf(w1, V0.y, fmaf(w2, V1.x, __fmul_rn(w3, V1.y))));
+    } else {
+        S.sm = su * (fmaf(w.x, U0.y, U0.x) + __fmul_rn(w.y, fmaf(w.x, U1.y, U1.x)));
+        S.sa = su * fmaf(w.y, U1.y, U0.y);
+        S.sz = su * fmaf(w.x, U1.y, U1.x);
+        S.sv = fmaf(w.x, V0.y, V0.x) + __fmul_rn(w.y, fmaf(w.x, V1.y, V1.x));
+    }
     return S;
 }
 
@@ -73,7 +92,7 @@ __device__ __forceinline__ Quad lds_diff(uint32_t addr, const TileCtx& C) {
 // nodes from the slab when every bin of the warp has its node pair there, else
 // from global memory. It reads dL/dcube0 from the spaxel's row (grow) itself,
 // so that the fast path's register copy never has to be kept for this call.
-template <int TW>
+template <int TW, int KIND>
 static __device__ __noinline__ AdjSums adj_general(const float2 w, const float4 g4, const TileCtx C, int lane,
                                             const float* __restrict__ grow, float ls0_over) {
     const int c0_bi = __float_as_int(g4.x);
@@ -94,7 +113,7 @@ static __device__ __noinline__ AdjSums adj_general(const float2 w, const float4 
         if (j >= C.n_lambda) break;
         float f;
         const int k = node_pos(j, bi, g4.y, g4.z, g4.w, f);
-        const Forms p = node_forms(w, quad_at(C, use_slab, e, k)), q = node_forms(w, quad_at(C, use_slab, e, k + 1));
+        const Forms p = node_forms<KIND>(w, quad_at(C, use_slab, e, k)), q = node_forms<KIND>(w, quad_at(C, use_slab, e, k + 1));
         const float Gj = grow[j];
         S.sm = fmaf(Gj, fmaf(f, q.m - p.m, p.m), S.sm);
         S.sa = fmaf(Gj, fmaf(f, q.a - p.a, p.a), S.sa);
@@ -148,12 +167,11 @@ __device__ __forceinline__ AdjSums adj_near1(const float2 w, const TileCtx& C, u
         base += carry ? s30 : s31;
         u += du;
     }
-    return entry_sums<false>(w, 1.f, U01, U23, T01, T23);
+    return entry_sums<0>(w, 1.f, U01, U23, T01, T23);
 }
 
-// Any A: rounds of 32 bins, the sums as in adj_near1 (of the second entry's
-// difference to the first: a cell's metallicities differ by a few per cent, and
-// sums of their difference do not cancel); lane l reads both nodes of its bin. The slope jumps at every node, so the node is decided with all
+// Any A: rounds of 32 bins, the sums as in adj_near1; lane l reads both nodes
+// of its bin. The slope jumps at every node, so the node is decided with all
 // the record's precision, as node_pos decides it (the same operations in
 // packed form; the integer parts stay in the magic sums' low bits).
 template <int TW, int NR>
@@ -192,7 +210,7 @@ __device__ __forceinline__ AdjSums adj_rounds(const float2 w, const float4 g4, c
             T23 = __ffma2_rn(t2, D23, T23);
         }
     }
-    return entry_sums<true>(w, 1.f, U01, U23, T01, T23);
+    return entry_sums<1>(w, 1.f, U01, U23, T01, T23);
 }
 
 // ---------------------------------------------------------------------------
@@ -205,6 +223,7 @@ __device__ __forceinline__ AdjSums adj_rounds(const float2 w, const float4 g4, c
 // sv sums G_j times the bracket, and sm, sa, sz sum G_j times the bin means
 // of the three weighted interpolants (M, and the a- and b-weighted forms).
 // ---------------------------------------------------------------------------
+template <int KIND>
 static __device__ __noinline__ AdjSums adj_mean_bin(const float2 w, const float4 g4, const TileCtx C, int j, float Gj,
                                                     bool use_slab, float ls0_over) {
     AdjSums S{0.f, 0.f, 0.f, 0.f};
@@ -213,7 +232,7 @@ static __device__ __noinline__ AdjSums adj_mean_bin(const float2 w, const float4
     float fa, fb;
     const int ka = node_pos(j, bi, g4.y, g4.z, g4.w, fa);
     const int kb = node_pos(j + 1, bi, g4.y, g4.z, g4.w, fb);
-    auto node = [&](int k) { return node_forms(w, quad_at(C, use_slab, e, k)); };
+    auto node = [&](int k) { return node_forms<KIND>(w, quad_at(C, use_slab, e, k)); };
     const float len = (float)(kb - ka) + (fb - fa);
     if (!(len > 0.f)) return S;
     const int k_first = max(ka, -1), k_last = min(kb, C.n_ls - 1);
@@ -242,7 +261,7 @@ static __device__ __noinline__ AdjSums adj_mean_bin(const float2 w, const float4
 
 // General path of the bin means: bin j0 + 32 r + l on lane l, nodes from the
 // slab when every bin of the warp has its nodes there, else from global memory.
-template <int TW>
+template <int TW, int KIND>
 static __device__ __noinline__ AdjSums adj_mean_general(const float2 w, const float4 g4, const TileCtx C, int lane,
                                                  const float* __restrict__ grow, float ls0_over) {
     const int c0_bi = __float_as_int(g4.x);
@@ -262,7 +281,7 @@ static __device__ __noinline__ AdjSums adj_mean_general(const float2 w, const fl
     for (int o = lane; o < TW; o += 32) {
         const int j = C.j0 + o;
         if (j >= C.n_lambda) break;
-        const AdjSums b = adj_mean_bin(w, g4, C, j, grow[j], use_slab, ls0_over);
+        const AdjSums b = adj_mean_bin<KIND>(w, g4, C, j, grow[j], use_slab, ls0_over);
         S.sm += b.sm;
         S.sa += b.sa;
         S.sz += b.sz;
@@ -334,7 +353,7 @@ __device__ __forceinline__ AdjSums adj_mean_near1(const float2 w, const TileCtx&
             u += du;
         }
     }
-    return entry_sums<false>(w, 0.5f, U01, U23, T01, T23);
+    return entry_sums<0>(w, 0.5f, U01, U23, T01, T23);
 }
 
 // Any dt/dj in [1/2, 2): the forward's two-read edges (mean_rounds_phi) in
@@ -388,7 +407,7 @@ __device__ __forceinline__ AdjSums adj_mean_phi(const float2 w, const float4 g4,
             T = __fadd2_rn(T, __ffma2_rn(make_float2(-gi, -gi), v, br));
         }
     }
-    return entry_sums<true>(w, 1.f, U01, U23, T01, T23);
+    return entry_sums<1>(w, 1.f, U01, U23, T01, T23);
 }
 
 // One particle's four sums over the tile (setup by every lane; warp-uniform path).
@@ -419,8 +438,8 @@ __device__ __forceinline__ AdjSums adj_particle(const float2 w, const float4 g4,
         if (fits) return adj_rounds<TW, NR>(w, g4, C, e, bi, A, u0, lanef, G);
     }
     if (!(g4.z > 0.f)) return AdjSums{0.f, 0.f, 0.f, 0.f};  // the spectrum misses every bin
-    if constexpr (MEAN) return adj_mean_general<TW>(w, g4, C, lane, grow, ls0_over);
-    else return adj_general<TW>(w, g4, C, lane, grow, ls0_over);
+    if constexpr (MEAN) return adj_mean_general<TW, KIND>(w, g4, C, lane, grow, ls0_over);
+    else return adj_general<TW, KIND>(w, g4, C, lane, grow, ls0_over);
 }
 
 template <int R, int KIND, bool MEAN>

@@ -334,7 +334,7 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
     launch_adjoint_setup(A, P.d_wu, st);
     AdjTileParams T{};
     static_cast<SlabParams&>(T) = S.geo;
-    T.pair = S.d_pair_adj;
+    T.pair = S.d_pair_adj ? S.d_pair_adj : S.d_pair;
     T.qdt = 0;
     T.map = P.d_map;
     T.wu = P.d_wu;

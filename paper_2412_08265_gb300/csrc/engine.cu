@@ -379,9 +379,10 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
         const size_t total = (size_t)G.band_stride * G.n_bands, nt = (size_t)S.n_age * S.n_Z * S.n_ls;
         std::vector<float> tf(nt);
         for (size_t i = 0; i < nt; ++i) tf[i] = (float)ssp->spectra[i];
+        const bool own_adj = with_adjoint && !(G.kind == 0 && G.qdt == 0);  // else d_pair serves
         float* d_t = nullptr;
         const bool ok = cudaMalloc(&h->d_pair, total * (G.qdt ? 4 : 8)) == cudaSuccess &&
-                        (!with_adjoint || dalloc_sync(&h->d_pair_adj, total) == cudaSuccess) &&
+                        (!own_adj || dalloc_sync(&h->d_pair_adj, total) == cudaSuccess) &&
                         dalloc_sync(&d_t, nt) == cudaSuccess;
         cudaError_t e = cudaSuccess;
         if (ok) {

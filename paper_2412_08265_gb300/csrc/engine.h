@@ -37,7 +37,7 @@ struct SspState {
     int device = 0, n_sm = 0, smem_optin = 0;
     SspDev ssp{};
     void* d_pair = nullptr;     // age pairs of the templates, one block per age band (SlabParams)
-    float2* d_pair_adj = nullptr;  // the adjoint's form of them (null without backward): (T, T(ia + 1) - T)
+    float2* d_pair_adj = nullptr;  // the adjoint's form of them, where it differs (launch_build_pairs)
     SlabParams geo{};           // the deposit's tiles and slabs
     float* d_la = nullptr;
     float* d_lz = nullptr;

@@ -200,9 +200,8 @@ inline __host__ __device__ const void* band_ptr(const void* pair, int qdt, long 
 }
 
 // Lays the templates t ([n_age][n_Z][n_ls] FP32) out as age pairs: `pair`
-// (SlabParams::pair) and, if not null, `adj` with entries (T, T(next age) - T) of
-// the same (storage-rounded) values, so that the adjoint's sums of age
-// derivatives do not cancel.
+// (SlabParams::pair) and, if not null, `adj`, the adjoint's FP32 entries of the
+// same (storage-rounded) values: the pairs for kind 0, else (T, T(next age) - T).
 int launch_build_pairs(const SlabParams& G, int apb, int n_age, int n_Z, const float* t, void* pair, float2* adj,
                        cudaStream_t st);
 

@@ -197,7 +197,7 @@ __global__ void k_build_pairs(const SlabParams G, int apb, int n_age, int n_Z, c
         } else {
             static_cast<float2*>(pair)[i] = make_float2(v0, v1);
         }
-        if (adj) adj[i] = make_float2(v0, v1 - v0);
+        if (adj) adj[i] = make_float2(v0, G.kind == 0 ? v1 : v1 - v0);
     }
 }
 
