@@ -228,7 +228,7 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
     h->z_cosmo = tel->z_cosmo;
 
     // ---- SSP grid: sizes and node vectors (the templates go to the device as
-    // cell quads, below) ----
+    // age pairs, below) ----
     SspDev& S = h->ssp;
     S.dtype = ssp->storage_dtype;
     S.n_age = ssp->n_age;

@@ -92,7 +92,7 @@ int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, 
                        int* perm_out, int* seg_off, int* scratch, bool long_tiles, unsigned long long* next_chain,
                        int n_next_chain, unsigned* err, cudaStream_t st);
 
-// SSP grid as seen by the kernels (the templates themselves as cell quads).
+// SSP grid as seen by the kernels (the templates themselves: SlabParams).
 struct SspDev {
     int dtype;              // 0 f32, 1 bf16, 2 f16
     int n_age, n_Z, n_t, n_ls;
@@ -279,7 +279,7 @@ struct AdjointParams {
 // Adjoint over the deposit's (wavelength tile, work item, age band)
 // decomposition: per (tile, particle) the four sums
 //   part = (sum_j G S, sum_j G dS/dta', sum_j G dS/dtz', sum_j G dS/dt * t_abs)
-// over the tile's bins (unit mass), from the same shared-memory quad slabs.
+// over the tile's bins (unit mass), from slabs of the same geometry.
 struct AdjTileParams : SlabParams {
     const MapRec* map;          // [n_in] the forward's maps (sorted order)
     const float2* wu;           // [n_in] position (ta, tz) in the SSP cell

@@ -1,6 +1,6 @@
 // tile.cuh -- device helpers shared by the deposit (K4) and the adjoint over
 // the same (wavelength tile, work item, age band) decomposition: work-item
-// search over the cost space, the bin -> SSP node map, and cell quads.
+// search over the cost space, the bin -> SSP node map, and the template slab.
 #pragma once
 
 #include "common.cuh"
