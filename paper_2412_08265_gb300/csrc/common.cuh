@@ -164,10 +164,8 @@ __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
 // waiting for anyone. chain[0] is the ticket, chain[1 + tile] the tile's sum
 // with its top bit set; all are cleared beforehand. The wait has a limit, after
 // which the block takes what it has (a sum too small, never too large) and sets
-// the error word.
+// the error word. (chain_words in sort_layout.h gives the words of a chain.)
 // ----------------------------------------------------------------------------
-inline __host__ __device__ size_t chain_words(long long tiles) { return (size_t)tiles + 1; }
-
 struct ChainShared {
     unsigned ticket;
     unsigned long long warp[32];

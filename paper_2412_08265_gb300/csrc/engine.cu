@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "engine.h"
+#include "sort_layout.h"
 #include "tile.cuh"
 
 namespace rubix {
@@ -450,7 +451,7 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_key, 4 * N},
         {(void**)&P->d_keys_tmp, 4 * N}, {(void**)&P->d_vals_tmp, 4 * N}, {(void**)&P->d_skeys, 4 * N},
         {(void**)&P->d_perm, 4 * N}, {(void**)&P->d_pin, 16 * N},
-        {(void**)&P->d_sort_scratch, 4 * sort_scratch_ints((long long)N)},
+        {(void**)&P->d_sort_scratch, 4 * sort_scratch_ints((long long)N, S.n_sm, false)},
         {(void**)&P->d_items, sizeof(Item) * (size_t)item_cap}, {(void**)&P->d_rec, sizeof(DepRec) * N},
         {(void**)&P->d_map, sizeof(MapRec) * N},
         {(void**)&P->d_prec, sizeof(PartRec) * N},
@@ -710,9 +711,11 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         A.apb = S.apb;
         A.n_bands = S.geo.n_bands;
         P.launches += launch_assign(A, st);
-        P.launches += launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
-                                         P.d_perm, P.d_seg_off, P.d_sort_scratch, false, P.d_chain,
-                                         (int)item_chain_words(P.n_s), S.d_err, st);
+        const int ls = launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
+                                          P.d_perm, P.d_seg_off, P.d_sort_scratch, sort_scratch_ints(P.cap, S.n_sm, false),
+                                          false, P.d_chain, (int)item_chain_words(P.n_s), S.d_err, st);
+        if (ls < 0) return fail(RUBIX_ERR_CUDA, "internal: sort scratch too small for %lld particles", n);
+        P.launches += ls;
     } else {
         CK(cudaMemsetAsync(P.d_chain, 0, 8 * item_chain_words(P.n_s), st));
         CK(cudaMemsetAsync(P.d_seg_off, 0, ((size_t)P.n_s * S.geo.n_bands + 2) * sizeof(int), st));

@@ -83,14 +83,14 @@ struct AssignParams {
 };
 
 int launch_assign(const AssignParams& P, cudaStream_t st);
-// Scratch of a sort of n keys (long_tiles: with the large tiles whatever n is,
-// for less scratch).
-size_t sort_scratch_ints(long long n, bool long_tiles = false);
-// Stable sort of keys in [0, n_keys); seg_off gets n_keys + 1 entries. Also
-// clears next_chain (nullable), the chain of a scan that follows.
+// Stable sort of keys in [0, n_keys); seg_off gets n_keys + 1 entries. scratch
+// holds scratch_ints ints (sort_scratch_ints of sort_layout.h for a capacity);
+// -1, with nothing launched, if the sort needs more. long_tiles: the large tiles
+// whatever n is, for less scratch. Also clears next_chain (nullable), the chain of
+// a scan that follows.
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
-                       int* perm_out, int* seg_off, int* scratch, bool long_tiles, unsigned long long* next_chain,
-                       int n_next_chain, unsigned* err, cudaStream_t st);
+                       int* perm_out, int* seg_off, int* scratch, size_t scratch_ints, bool long_tiles,
+                       unsigned long long* next_chain, int n_next_chain, unsigned* err, cudaStream_t st);
 
 // SSP grid as seen by the kernels (the templates themselves: SlabParams).
 struct SspDev {

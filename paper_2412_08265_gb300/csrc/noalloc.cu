@@ -28,6 +28,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "engine.h"
+#include "sort_layout.h"
 
 namespace rubix {
 
@@ -96,7 +97,7 @@ extern "C" rubix_status rubix_spaxel_sort_noalloc(const rubix_particles* p, cons
     // the sort's scratch layout (tiles, digit buckets, scan tiles) must fit
     // the fixed array; a change of those constants shows up here, not as an
     // overrun
-    if ((long long)sort_scratch_ints(n_or_1(p->n), true) > kNoallocSortInts) {
+    if ((long long)sort_scratch_ints(n_or_1(p->n), 1, true) > kNoallocSortInts) {
         set_last_error("internal: the sort needs more scratch than the no-allocation array holds");
         return RUBIX_ERR_UNSUPPORTED;
     }
@@ -135,8 +136,11 @@ extern "C" rubix_status rubix_spaxel_sort_noalloc(const rubix_particles* p, cons
     A.key = keys;
     A.pin_out = nullptr;
     launch_assign(A, st);
-    launch_sort_by_key(keys, n, n_keys, keys_tmp, vals_tmp, skeys, perm_out, seg_off_out, sort_scratch, true,
-                       nullptr, 0, nullptr, st);
+    if (launch_sort_by_key(keys, n, n_keys, keys_tmp, vals_tmp, skeys, perm_out, seg_off_out, sort_scratch,
+                           (size_t)kNoallocSortInts, true, nullptr, 0, nullptr, st) < 0) {
+        set_last_error("internal: the sort needs more scratch than the no-allocation array holds");
+        return RUBIX_ERR_UNSUPPORTED;
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         char m[160];

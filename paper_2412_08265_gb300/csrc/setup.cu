@@ -6,6 +6,7 @@
 // are cut into work items of at most `chunk` particles.
 #include "common.cuh"
 #include "kernels.h"
+#include "sort_layout.h"
 
 namespace rubix {
 

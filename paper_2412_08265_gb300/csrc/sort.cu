@@ -4,6 +4,7 @@
 // atomics in the per-spaxel sum of spectra.
 #include "common.cuh"
 #include "kernels.h"
+#include "sort_layout.h"
 
 namespace rubix {
 
@@ -139,7 +140,7 @@ __global__ void k_assign(AssignParams P) {
 // ----------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
+static_assert(kScanTile == kScanThreads * kScanItems, "scan tile");
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, long long n, int* __restrict__ out,
                                                        unsigned long long* __restrict__ chain, unsigned* err) {
@@ -166,19 +167,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
 // Per pass: per-tile digit counts (digit-major), exclusive scan, then a stable
 // scatter in which each warp ranks its keys in index order with match.any.
 // ----------------------------------------------------------------------------
-constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kMaxBuckets = 512;
-// Keys per tile: 16 per thread, or 4 while that leaves the tiles fewer than two
-// per SM (each round of a tile is a dependent step: 1e4 keys took 10 us for the
-// counts and 14 us for the scatter in 3 tiles of 4096).
-constexpr int kRoundsLong = 16, kRoundsShort = 4;
-static int sort_rounds(long long n) {
-    return n > 2ll * sm_count() * kSortThreads * kRoundsLong ? kRoundsLong : kRoundsShort;
-}
-static long long sort_tiles(long long n, int rounds) {
-    return (n + (long long)kSortThreads * rounds - 1) / ((long long)kSortThreads * rounds);
-}
 
 // Also clears the chain of the scan that follows.
 template <int ROUNDS>
@@ -340,23 +329,17 @@ __global__ void k_seg_bounds(const int* __restrict__ skeys, long long n, int n_k
     }
 }
 
-size_t sort_scratch_ints(long long n, bool long_tiles) {
-    const long long counts = sort_tiles(n, long_tiles ? kRoundsLong : sort_rounds(n)) * kMaxBuckets;
-    return (size_t)(2 * counts) + 2 * chain_words((counts + kScanTile - 1) / kScanTile) + 2;
-}
-
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
-                       int* perm_out, int* seg_off, int* scratch, bool long_tiles, unsigned long long* next_chain,
-                       int n_next_chain, unsigned* err, cudaStream_t st) {
+                       int* perm_out, int* seg_off, int* scratch, size_t scratch_ints, bool long_tiles,
+                       unsigned long long* next_chain, int n_next_chain, unsigned* err, cudaStream_t st) {
     int launches = 0;
     if (n > 0) {
-        int bits = 1;
-        while ((1ll << bits) < (long long)n_keys) ++bits;   // keys lie in [0, n_keys)
-        const int passes = (bits + 8) / 9;
+        const SortLayout L = sort_layout(n, n_keys, sm_count(), long_tiles);
+        if (L.ints > scratch_ints) return -1;
+        const int bits = L.bits, passes = L.passes, n_tiles = L.n_tiles;  // keys lie in [0, n_keys)
         const int per = (bits + passes - 1) / passes;
-        const bool short_tiles = !long_tiles && sort_rounds(n) == kRoundsShort;
-        const int n_tiles = (int)sort_tiles(n, short_tiles ? kRoundsShort : kRoundsLong);
-        const long long n_counts = (long long)n_tiles << per;
+        const bool short_tiles = L.rounds == kRoundsShort;
+        const long long n_counts = L.n_counts;
         // the chain first, on an 8-byte boundary
         unsigned long long* chain =
             reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(scratch) + 7) & ~(uintptr_t)7);
