@@ -76,7 +76,6 @@ __global__ void k_adj_final(const AdjointParams P, const float4* __restrict__ pa
         const float dZ = fs * pr.mass * dtz * sz / (pr.Z * ln10);
         const float dv = fs * pr.mass * q * sv;
         const int p = P.perm[i];
-        if ((unsigned)p >= (unsigned)P.n_in) continue;  // only after an expired wait in the sort
         if (P.d_mass) P.d_mass[p] = dm;
         if (P.d_age) P.d_age[p] = dage;
         if (P.d_Z) P.d_Z[p] = dZ;

@@ -13,7 +13,7 @@ constexpr double kC_kms = 299792.458;
 
 // Error word written by kernels (bit flags), read by the host after a forward.
 enum DeviceError : unsigned {
-    kErrTmaTimeout = 1u,      // a bounded wait expired (an mbarrier of a slab load, a chained scan)
+    kErrTmaTimeout = 1u,      // a bounded wait expired (the mbarrier of a slab or cube row load)
     kErrBadItem = 2u,         // a work item pointed outside its buffers
     kErrBounds = 4u,          // debug builds: a computed index fell outside its buffer
 };
@@ -162,9 +162,11 @@ __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
 // tile's sum, and add up the sums published before theirs: a block waits only
 // for blocks that hold an earlier ticket, which are running and publish without
 // waiting for anyone. chain[0] is the ticket, chain[1 + tile] the tile's sum
-// with its top bit set; all are cleared beforehand. The wait has a limit, after
-// which the block takes what it has (a sum too small, never too large) and sets
-// the error word. (chain_words in sort_layout.h gives the words of a chain.)
+// with its top bit set; all are cleared beforehand. The wait has a limit (about
+// a millisecond; the blocks of a GPU that was taken away from the process in
+// between may meet it), after which the block adds up the missing tiles itself:
+// the result is the same whatever was waited for. (chain_words in sort_layout.h
+// gives the words of a chain.)
 // ----------------------------------------------------------------------------
 struct ChainShared {
     unsigned ticket;
@@ -208,21 +210,25 @@ __device__ __forceinline__ unsigned long long block_exclusive(unsigned long long
     return r;
 }
 
+constexpr long long kChainWait = 2000000;  // cycles a block waits for the sums before its own
+
 // Exclusive prefix of v over all threads of all tiles before this one (values
-// and sums below 2^63).
+// and sums below 2^63). tile_sum(i) is tile i's sum from the scan's input. quiet
+// (tests): nothing is published.
+template <class TileSum>
 __device__ __forceinline__ unsigned long long chain_exclusive(unsigned long long v, unsigned tile,
-                                                              unsigned long long* chain, ChainShared& sh, unsigned* err) {
+                                                              unsigned long long* chain, ChainShared& sh, bool quiet,
+                                                              TileSum tile_sum) {
     unsigned long long total;
     const unsigned long long e = block_exclusive(v, sh, total);
     volatile unsigned long long* pub = chain + 1;
-    if (threadIdx.x == 0) pub[tile] = total | (1ull << 63);
+    if (threadIdx.x == 0 && !quiet) pub[tile] = total | (1ull << 63);
     unsigned long long before = 0;
     const long long t0 = clock64();
     for (unsigned i = threadIdx.x; i < tile; i += blockDim.x) {
         unsigned long long w = pub[i];
-        while (!(w >> 63) && clock64() - t0 < 4000000000ll) w = pub[i];
-        if (w >> 63) before += w & ~(1ull << 63);
-        else if (err) atomicOr(err, kErrTmaTimeout);
+        while (!(w >> 63) && clock64() - t0 < kChainWait) w = pub[i];
+        before += (w >> 63) ? w & ~(1ull << 63) : tile_sum(i);
     }
     unsigned long long sum;
     block_exclusive(before, sh, sum);

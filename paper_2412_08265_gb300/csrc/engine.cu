@@ -542,6 +542,13 @@ static int fault_alloc_at() {
     return e ? std::atoi(e) : 0;
 }
 
+// RUBIX_FAULT_SCAN=1 (tests): the blocks of the plan's chained scans publish
+// nothing, so that every wait in them runs out.
+static bool fault_scan() {
+    const char* e = std::getenv("RUBIX_FAULT_SCAN");
+    return e && std::atoi(e) != 0;
+}
+
 rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, long long n, Alloc a, bool with_out,
                        bool with_grad) {
     rubix_status st = validate_telescope(tel, S->ssp.dls);
@@ -550,6 +557,7 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
         return fail(RUBIX_ERR_INVALID_ARG, "telescope wavelength grid differs from the SSP state's");
     if (n < 0 || n > (1ll << 30)) return fail(RUBIX_ERR_INVALID_ARG, "particle count out of range");
     P->S = S;
+    P->quiet_scan = fault_scan();
     P->alloc = a;
     P->tel = *tel;
     if (P->tel.flux_scale == 0.0) P->tel.flux_scale = 1.0;
@@ -713,7 +721,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         P.launches += launch_assign(A, st);
         const int ls = launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
                                           P.d_perm, P.d_seg_off, P.d_sort_scratch, sort_scratch_ints(P.cap, S.n_sm, false),
-                                          false, P.d_chain, (int)item_chain_words(P.n_s), S.d_err, st);
+                                          false, P.d_chain, (int)item_chain_words(P.n_s), P.quiet_scan, st);
         if (ls < 0) return fail(RUBIX_ERR_CUDA, "internal: sort scratch too small for %lld particles", n);
         P.launches += ls;
     } else {
@@ -747,7 +755,6 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     SP.s_min = S.geo.s_min;
     SP.s_max = S.geo.s_max;
     SP.prec = P.d_prec;
-    SP.n_total = n;
     SP.n_cap = P.cap;
     P.launches += launch_setup(SP, n, st);
     ItemParams IP{};
@@ -761,6 +768,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     IP.item_cap = P.item_cap;
     IP.split = P.d_split;
     IP.chain = P.d_chain;
+    IP.quiet_scan = P.quiet_scan;
     IP.slow_count = P.alloc.async ? nullptr : S.d_slow;  // one forward at a time on a handle
     IP.err = S.d_err;
     P.launches += launch_items(IP, st);

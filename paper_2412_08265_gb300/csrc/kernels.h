@@ -87,10 +87,10 @@ int launch_assign(const AssignParams& P, cudaStream_t st);
 // holds scratch_ints ints (sort_scratch_ints of sort_layout.h for a capacity);
 // -1, with nothing launched, if the sort needs more. long_tiles: the large tiles
 // whatever n is, for less scratch. Also clears next_chain (nullable), the chain of
-// a scan that follows.
+// a scan that follows. quiet_scan (tests): the scans' blocks publish nothing.
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
                        int* perm_out, int* seg_off, int* scratch, size_t scratch_ints, bool long_tiles,
-                       unsigned long long* next_chain, int n_next_chain, unsigned* err, cudaStream_t st);
+                       unsigned long long* next_chain, int n_next_chain, bool quiet_scan, cudaStream_t st);
 
 // SSP grid as seen by the kernels (the templates themselves: SlabParams).
 struct SspDev {
@@ -120,7 +120,6 @@ struct SetupParams {
     int fb, jc, apb, kind;
     float a_max, s_min, s_max;
     PartRec* prec;           // [n_in]
-    long long n_total;       // particles (perm holds indices below it)
     long long n_cap;         // capacity of rec / prec
 };
 int launch_setup(const SetupParams& P, long long n_total, cudaStream_t st);
@@ -138,6 +137,7 @@ struct ItemParams {
     // split spaxels
     unsigned long long* chain;
     unsigned long long* slow_count;  // nullable: the forward's count of per-bin visits, reset here
+    bool quiet_scan;         // tests: the scan's blocks publish nothing
     unsigned* err;
 };
 size_t item_chain_words(int n_s);

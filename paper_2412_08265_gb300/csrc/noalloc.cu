@@ -137,7 +137,7 @@ extern "C" rubix_status rubix_spaxel_sort_noalloc(const rubix_particles* p, cons
     A.pin_out = nullptr;
     launch_assign(A, st);
     if (launch_sort_by_key(keys, n, n_keys, keys_tmp, vals_tmp, skeys, perm_out, seg_off_out, sort_scratch,
-                           (size_t)kNoallocSortInts, true, nullptr, 0, nullptr, st) < 0) {
+                           (size_t)kNoallocSortInts, true, nullptr, 0, false, st) < 0) {
         set_last_error("internal: the sort needs more scratch than the no-allocation array holds");
         return RUBIX_ERR_UNSUPPORTED;
     }

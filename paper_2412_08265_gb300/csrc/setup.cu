@@ -85,11 +85,7 @@ __global__ void k_setup(SetupParams P) {
     const float t_lastj = (float)(P.resample ? P.n_lambda : P.n_lambda - 1);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_in;
          i += (long long)gridDim.x * blockDim.x) {
-        // (an index out of range: only after an expired wait in the sort, which
-        // the error word reports)
-        const int pi = P.perm[i];
-        PartRec pr{0.f, 1.f, 1.f, 0.f};
-        if ((unsigned)pi < (unsigned)P.n_total) pr = P.pin[pi];
+        const PartRec pr = P.pin[P.perm[i]];
         const float m = pr.mass, age = pr.age, Z = pr.Z;
         int ia, iz;
         float ta, tz, dta, dtz;
@@ -231,7 +227,17 @@ __global__ void __launch_bounds__(kItemTile) k_items(const ItemParams P, int n_t
     }
     const int ni = (e0 - b0 + P.chunk - 1) / P.chunk;
     const int np = ni > 1 ? ni : 0;  // partial rows
-    const unsigned long long pre = chain_exclusive(((unsigned long long)np << 32) | (unsigned)ni, tile, P.chain, sh, P.err);
+    auto tile_sum = [&](unsigned i) {
+        unsigned long long t = 0;
+        const long long first = (long long)i * kItemTile, end = min(first + kItemTile, (long long)P.n_s);
+        for (long long k = first; k < end; ++k) {
+            const int m = (P.seg_off[(k + 1) * nb] - P.seg_off[k * nb] + P.chunk - 1) / P.chunk;
+            t += ((unsigned long long)(m > 1 ? m : 0) << 32) | (unsigned)m;
+        }
+        return t;
+    };
+    const unsigned long long pre =
+        chain_exclusive(((unsigned long long)np << 32) | (unsigned)ni, tile, P.chain, sh, P.quiet_scan, tile_sum);
     if (s > P.n_s) return;
     const int base = (int)(pre & 0xffffffffu), part = (int)(pre >> 32);
     P.item_off[s] = base;

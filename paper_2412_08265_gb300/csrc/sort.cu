@@ -132,8 +132,8 @@ __global__ void k_assign(AssignParams P) {
 }
 
 // ----------------------------------------------------------------------------
-// Exclusive scan of int32 in one launch (ChainedTiles, common.cuh): a tile's
-// blocks publish their sums as soon as they have them and add up those before
+// Exclusive scan of int32 in one launch (chain_exclusive, common.cuh): blocks
+// publish their tile's sum as soon as they have it and add up those before
 // theirs, so that no block waits for more than another block's loads. (Three
 // launches -- block sums, scan of the sums, block scans -- took 8 us of a small
 // galaxy's pass each time.)
@@ -143,7 +143,7 @@ constexpr int kScanItems = 4;
 static_assert(kScanTile == kScanThreads * kScanItems, "scan tile");
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ in, long long n, int* __restrict__ out,
-                                                       unsigned long long* __restrict__ chain, unsigned* err) {
+                                                       unsigned long long* __restrict__ chain, bool quiet) {
     __shared__ ChainShared sh;
     const unsigned tile = chain_ticket(chain, sh);
     const long long base = (long long)tile * kScanTile + (long long)threadIdx.x * kScanItems;
@@ -154,7 +154,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
         v[i] = (base + i < n) ? in[base + i] : 0;
         s += v[i];
     }
-    unsigned long long e = chain_exclusive((unsigned long long)s, tile, chain, sh, err);
+    auto tile_sum = [&](unsigned i) {
+        const long long b = (long long)i * kScanTile, e = min(b + kScanTile, n);
+        unsigned long long t = 0;
+        for (long long k = b; k < e; ++k) t += (unsigned)in[k];
+        return t;
+    };
+    unsigned long long e = chain_exclusive((unsigned long long)s, tile, chain, sh, quiet, tile_sum);
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
         if (base + i < n) out[base + i] = (int)e;
@@ -331,7 +337,7 @@ __global__ void k_seg_bounds(const int* __restrict__ skeys, long long n, int n_k
 
 int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, int* vals_tmp, int* keys_out,
                        int* perm_out, int* seg_off, int* scratch, size_t scratch_ints, bool long_tiles,
-                       unsigned long long* next_chain, int n_next_chain, unsigned* err, cudaStream_t st) {
+                       unsigned long long* next_chain, int n_next_chain, bool quiet_scan, cudaStream_t st) {
     int launches = 0;
     if (n > 0) {
         const SortLayout L = sort_layout(n, n_keys, sm_count(), long_tiles);
@@ -361,7 +367,7 @@ int launch_sort_by_key(const int* keys, long long n, int n_keys, int* keys_tmp, 
                 k_radix_hist<kRoundsShort><<<n_tiles, kSortThreads, 0, st>>>(kin, n, shift, nb, n_tiles, counts, chain, n_chain);
             else
                 k_radix_hist<kRoundsLong><<<n_tiles, kSortThreads, 0, st>>>(kin, n, shift, nb, n_tiles, counts, chain, n_chain);
-            k_scan<<<n_scan, kScanThreads, 0, st>>>(counts, cnt, offs, chain, err);
+            k_scan<<<n_scan, kScanThreads, 0, st>>>(counts, cnt, offs, chain, quiet_scan);
             if (short_tiles)
                 k_radix_scatter<kRoundsShort><<<n_tiles, kSortThreads, 0, st>>>(kin, vin, n, shift, nb, n_tiles, offs, kout, vout);
             else
