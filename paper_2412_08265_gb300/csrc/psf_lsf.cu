@@ -180,9 +180,12 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     float* stages = smt + kHead;
     float* px = stages + kTS * G::stage_floats;  // [2][kTX][kTB] PSF-x output, alternating by row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j0 = blockIdx.x * G::TL, x0 = blockIdx.y * kTX, y0 = blockIdx.z * P.ty;
-    const int y1 = min(y0 + P.ty, P.ny);
+    // wavelength tiles and blocks of columns share grid.x (grid.y ends at 65535:
+    // fields of up to 2^24 spaxels along x)
     const int nx = P.nx, nl = P.n_lambda;
+    const unsigned n_lt = (unsigned)(nl + G::TL - 1) / (unsigned)G::TL;
+    const int j0 = (int)(blockIdx.x % n_lt) * G::TL, x0 = (int)(blockIdx.x / n_lt) * kTX, y0 = blockIdx.y * P.ty;
+    const int y1 = min(y0 + P.ty, P.ny);
     const int n_rows = (y1 - y0) + 2 * RP;  // input rows y0 - RP .. y1 + RP - 1
     float gl[2 * RL + 1], gp[NR];
 #pragma unroll
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     const int jl = j0 - G::RLa + 4 * lane;  // cube bin of the lane's first box bin
     // dense rows: position (modulo 2^32) of input column c0's first bin in input row 0
     const unsigned row_step = (unsigned)nx * (unsigned)nl;
-    const unsigned col0 = (unsigned)D.off + (unsigned)(y0 - RP) * row_step + (unsigned)((x0 - RP + c0) * nl + j0 - G::RLa);
+    const unsigned col0 = (unsigned)D.off + (unsigned)(y0 - RP) * row_step + (unsigned)(x0 - RP + c0) * (unsigned)nl + (unsigned)(j0 - G::RLa);
 
     // rows of `out` that are 16-byte aligned take 16-byte stores (others four
     // 4-byte ones: bringing them into order through shared memory first cost more
@@ -421,9 +424,9 @@ static bool launch_conv(ConvParams P, const CUtensorMap* map, const DenseRows& D
     if (cudaFuncSetAttribute(k_psf_lsf<RP, RL, DENSE, NOISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem) !=
         cudaSuccess)
         return false;
-    dim3 g((P.n_lambda + G::TL - 1) / G::TL, (P.nx + kTX - 1) / kTX, 1);
-    P.ty = rows_per_cta(P.ny, RP, (long long)g.x * g.y);
-    g.z = (P.ny + P.ty - 1) / P.ty;
+    const long long columns = (long long)((P.n_lambda + G::TL - 1) / G::TL) * ((P.nx + kTX - 1) / kTX);
+    P.ty = rows_per_cta(P.ny, RP, columns);
+    const dim3 g((unsigned)columns, (P.ny + P.ty - 1) / P.ty);
     k_psf_lsf<RP, RL, DENSE, NOISE><<<g, kTThreads, G::smem, st>>>(P, *map, D, out);
     return true;
 }
