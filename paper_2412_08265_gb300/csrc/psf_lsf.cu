@@ -13,6 +13,7 @@
 //     y-chunk and applies the PSF along y, then optional Philox noise.
 // All global accesses run along wavelength (the fastest axis): coalesced.
 #include "common.cuh"
+#include "conv_layout.h"
 #include "kernels.h"
 
 namespace rubix {
@@ -392,29 +393,7 @@ bool conv_tma_box(int rp, int rl, unsigned box[2]) {
     return false;
 }
 
-// Output rows per CTA: the split of the rows that fills whole waves of the
-// resident CTAs with the fewest input rows (each CTA reads 2 rp rows more than it
-// writes). One wave of 150-row CTAs is best for 150 x 150 spaxels x 3721 bins; a
-// 25 x 25 x 1000 cube runs 36 CTAs unsplit.
 constexpr int kMaxTY = 600;  // input rows (ty + 2 rp) have a bit each in the kernel's header
-static int rows_per_cta(int ny, int rp, long long columns) {
-    const long long slots = (long long)RUBIX_PSF_TMINB * sm_count();
-    int best = ny;
-    double cost = 1e300;
-    for (int k = 1; k <= ny; ++k) {
-        const int ty = (ny + k - 1) / k;
-        if (ty > kMaxTY) continue;
-        if (ty < 2 * rp && best <= kMaxTY) break;
-        const long long ctas = columns * ((ny + ty - 1) / ty);
-        // the rows of the CTAs one slot takes, and a pipeline start for each
-        const double c = (double)((ctas + slots - 1) / slots) * (ty + 2 * rp + 4);
-        if (c < cost * 0.999) {
-            cost = c;
-            best = ty;
-        }
-    }
-    return best;
-}
 
 template <int RP, int RL, bool DENSE, bool NOISE>
 static bool launch_conv(ConvParams P, const CUtensorMap* map, const DenseRows& D, float* out, cudaStream_t st) {
@@ -425,7 +404,7 @@ static bool launch_conv(ConvParams P, const CUtensorMap* map, const DenseRows& D
         cudaSuccess)
         return false;
     const long long columns = (long long)((P.n_lambda + G::TL - 1) / G::TL) * ((P.nx + kTX - 1) / kTX);
-    P.ty = rows_per_cta(P.ny, RP, columns);
+    P.ty = rows_per_cta(P.ny, RP, columns, (long long)RUBIX_PSF_TMINB * sm_count(), kMaxTY);
     const dim3 g((unsigned)columns, (P.ny + P.ty - 1) / P.ty);
     k_psf_lsf<RP, RL, DENSE, NOISE><<<g, kTThreads, G::smem, st>>>(P, *map, D, out);
     return true;
