@@ -305,7 +305,8 @@ rubix_status rubix_measure_fp32_peak(int32_t packed, double *flops_per_s, double
  *     small requests share launches without waiting behind a larger one;
  *   - the combine, PSF, LSF and noise of each request then run on its stream.
  * The work decomposition of a request never depends on the others, so its
- * cube is bitwise the same alone, in any mix, and from rubix_cube_forward.
+ * cube is bitwise the same alone, in any mix, and from rubix_cube_forward (to
+ * rounding from the latter if the budget is tight: rubix_serve_footprint).
  * Device memory comes from a stream-ordered pool owned by the server, so the
  * loop never synchronises the device.
  * ------------------------------------------------------------------------- */
@@ -333,7 +334,10 @@ rubix_status rubix_serve_submit(rubix_server_t *srv, const rubix_telescope *tel,
                                 uint64_t *ticket);
 
 /* Device bytes a request would hold while on the GPU (what admission counts
- * against hbm_budget_bytes), without submitting it. */
+ * against hbm_budget_bytes), without submitting it. A request that the budget
+ * alone does not hold with the work items rubix_cube_forward would take is run
+ * with larger ones, which need less scratch: its cube then equals that call's to
+ * rounding, and is still bitwise the same alone and in any mix. */
 rubix_status rubix_serve_footprint(rubix_server_t *srv, const rubix_telescope *tel, const rubix_particles *p,
                                    int32_t cube_on_device, size_t *bytes);
 

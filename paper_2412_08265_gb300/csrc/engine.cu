@@ -421,7 +421,8 @@ struct Buf {
 // with 256, 872 with 64; 2e5 particles, gradient step with bin means: 3.72 and
 // 3.60 ms; on the mid-size and large galaxies smaller items cost 1 - 5 %). It
 // depends on the request alone, so that its cube does not depend on the plan.
-int item_chunk(const SspState& S, long long n) {
+int item_chunk(const SspState& S, long long n, bool compact) {
+    if (compact) return RUBIX_DEP_CHUNK;
     const double items = (double)n * S.geo.n_tiles / ((double)S.n_sm * (S.dep_threads / 32) * 8.0);
     int c = RUBIX_DEP_CHUNK;
     while (c > RUBIX_DEP_CHUNK / 4 && c > items) c /= 2;
@@ -429,17 +430,24 @@ int item_chunk(const SspState& S, long long n) {
 }
 // The most of n' / item_chunk(n') over n' <= n (the smaller chunks end at a
 // known count).
-long long max_chunks(const SspState& S, long long n) {
+long long max_chunks(const SspState& S, long long n, bool compact) {
+    if (compact) return n / RUBIX_DEP_CHUNK;
     const long long lim = (long long)RUBIX_DEP_CHUNK * S.n_sm * (S.dep_threads / 32) * 8 / std::max(S.geo.n_tiles, 1) + 1;
     return std::max(n / RUBIX_DEP_CHUNK, std::min(n, lim) / (RUBIX_DEP_CHUNK / 4));
+}
+// Partial rows: ceil(count / chunk) of each split spaxel, each of more than chunk
+// particles.
+long long max_parts(const SspState& S, int n_s, long long n, bool compact) {
+    const long long c = max_chunks(S, n, compact);
+    return c + std::min<long long>(n_s, c) + 2;
 }
 
 // Every device buffer of a plan for n particles, with its size.
 std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda, long long n, bool with_out,
-                              bool with_grad, bool need_tmp, bool staging, int pitch0) {
+                              bool with_grad, bool need_tmp, bool staging, int pitch0, bool compact) {
     const size_t N = (size_t)std::max(n, 1ll);
-    const long long item_cap = (long long)n_s + max_chunks(S, n) + 2;
-    const long long part_cap = 2 * max_chunks(S, n) + 2;
+    const long long item_cap = (long long)n_s + max_chunks(S, n, compact) + 2;
+    const long long part_cap = max_parts(S, n_s, n, compact);
     const size_t cube = (size_t)n_s * n_lambda * sizeof(float);
     std::vector<Buf> v;
     if (staging)
@@ -451,10 +459,9 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
         {(void**)&P->d_key, 4 * N},
         {(void**)&P->d_keys_tmp, 4 * N}, {(void**)&P->d_vals_tmp, 4 * N}, {(void**)&P->d_skeys, 4 * N},
         {(void**)&P->d_perm, 4 * N}, {(void**)&P->d_pin, 16 * N},
-        {(void**)&P->d_sort_scratch, 4 * sort_scratch_ints((long long)N, S.n_sm, false)},
+        {(void**)&P->d_sort_scratch, 4 * sort_scratch_ints((long long)N, S.n_sm, compact)},
         {(void**)&P->d_items, sizeof(Item) * (size_t)item_cap}, {(void**)&P->d_rec, sizeof(DepRec) * N},
         {(void**)&P->d_map, sizeof(MapRec) * N},
-        {(void**)&P->d_prec, sizeof(PartRec) * N},
         {(void**)&P->d_partials, 4 * (size_t)part_cap * n_lambda},
         {(void**)&P->d_seg_off, 4 * ((size_t)n_s * S.geo.n_bands + 2)},
         {(void**)&P->d_item_off, 4 * ((size_t)n_s + 1)}, {(void**)&P->d_part_off, 4 * ((size_t)n_s + 1)},
@@ -465,6 +472,7 @@ std::vector<Buf> plan_buffers(Plan* P, const SspState& S, int n_s, int n_lambda,
     if (need_tmp) v.push_back({(void**)&P->d_tmp, cube});
     if (with_out) v.push_back({(void**)&P->d_out, cube});
     if (with_grad) {
+        v.push_back({(void**)&P->d_prec, sizeof(PartRec) * N});
         v.push_back({(void**)&P->d_contrib, 8 * kGlobal * N});
         v.push_back({(void**)&P->d_dvda, 8 * N});
         v.push_back({(void**)&P->d_red, 8 * 1024});
@@ -509,13 +517,13 @@ bool conv_params(const rubix_telescope* tel, int rows, ConvParams* C) {
 }
 
 size_t plan_bytes(const SspState& S, const rubix_telescope* tel, long long n, bool with_out, bool with_grad,
-                  bool staging) {
+                  bool staging, bool compact) {
     Plan tmp;
     const int rp = conv_radius_psf(tel), rl = conv_radius_lsf(tel);
     const bool need_tmp = psf_lsf_needs_tmp(rp, rl);
     size_t total = 0;
     for (const Buf& b : plan_buffers(&tmp, S, tel->nx * window_rows(tel), tel->n_lambda, n, with_out, with_grad, need_tmp,
-                                     staging, cube0_pitch(rp, rl, tel->n_lambda)))
+                                     staging, cube0_pitch(rp, rl, tel->n_lambda), compact))
         total += round256(b.bytes);
     return total;
 }
@@ -523,7 +531,8 @@ size_t plan_bytes(const SspState& S, const rubix_telescope* tel, long long n, bo
 void plan_release(Plan* P) {
     if (!P->S) return;
     const bool need_tmp = true;
-    for (const Buf& b : plan_buffers(P, *P->S, P->n_s, P->tel.n_lambda, P->cap, true, true, need_tmp, true, P->pitch0)) {
+    for (const Buf& b : plan_buffers(P, *P->S, P->n_s, P->tel.n_lambda, P->cap, true, true, need_tmp, true, P->pitch0,
+                                     P->alloc.compact)) {
         if (*b.ptr) {
             if (P->alloc.async) cudaFreeAsync(*b.ptr, P->alloc.stream);
             else cudaFree(*b.ptr);
@@ -573,14 +582,15 @@ rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, l
     P->pitch0 = cube0_pitch(C.rp, C.rl, tel->n_lambda);
     P->has_conv_map = false;
     P->cap = std::max(n, 1ll);
-    P->item_cap = (long long)P->n_s + max_chunks(*S, P->cap) + 2;
-    P->part_cap = 2 * max_chunks(*S, P->cap) + 2;
+    P->item_cap = (long long)P->n_s + max_chunks(*S, P->cap, a.compact) + 2;
+    P->part_cap = max_parts(*S, P->n_s, P->cap, a.compact);
     const bool need_tmp = psf_lsf_needs_tmp(C.rp, C.rl);
     P->bytes = 0;
     const int fail_at = fault_alloc_at();
     int idx = 0;
     for (const Buf& b :
-         plan_buffers(P, *S, P->n_s, tel->n_lambda, P->cap, with_out, with_grad, need_tmp, a.staging, P->pitch0)) {
+         plan_buffers(P, *S, P->n_s, tel->n_lambda, P->cap, with_out, with_grad, need_tmp, a.staging, P->pitch0,
+                      a.compact)) {
         cudaError_t e;
         if (++idx == fail_at) e = cudaErrorMemoryAllocation;
         else if (!a.async) e = cudaMalloc(b.ptr, round256(b.bytes));
@@ -720,8 +730,8 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         A.n_bands = S.geo.n_bands;
         P.launches += launch_assign(A, st);
         const int ls = launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
-                                          P.d_perm, P.d_seg_off, P.d_sort_scratch, sort_scratch_ints(P.cap, S.n_sm, false),
-                                          false, P.d_chain, (int)item_chain_words(P.n_s), P.quiet_scan, st);
+                                          P.d_perm, P.d_seg_off, P.d_sort_scratch, sort_scratch_ints(P.cap, S.n_sm, P.alloc.compact),
+                                          P.alloc.compact, P.d_chain, (int)item_chain_words(P.n_s), P.quiet_scan, st);
         if (ls < 0) return fail(RUBIX_ERR_CUDA, "internal: sort scratch too small for %lld particles", n);
         P.launches += ls;
     } else {
@@ -761,7 +771,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     IP.seg_off = P.d_seg_off;
     IP.n_s = P.n_s;
     IP.n_bands = S.geo.n_bands;
-    IP.chunk = item_chunk(S, n);
+    IP.chunk = item_chunk(S, n, P.alloc.compact);
     IP.item_off = P.d_item_off;
     IP.part_off = P.d_part_off;
     IP.items = P.d_items;

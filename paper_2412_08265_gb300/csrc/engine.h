@@ -82,6 +82,7 @@ struct Alloc {
     cudaStream_t stream = nullptr;
     cudaMemPool_t pool = nullptr;
     bool staging = true;
+    bool compact = false;  // work items of RUBIX_DEP_CHUNK particles and long sort tiles, for less scratch
 };
 
 // One galaxy's forward model on the device: its telescope (spatial grid,
@@ -129,7 +130,7 @@ struct Plan {
 // Device bytes plan_init would take for n particles (with_out: plus a device
 // cube for host output; with_grad: plus backward scratch).
 size_t plan_bytes(const SspState& S, const rubix_telescope* tel, long long n, bool with_out, bool with_grad,
-                  bool staging = true);
+                  bool staging, bool compact);
 rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, long long max_particles, Alloc a,
                        bool with_out, bool with_grad);
 rubix_status plan_grow(Plan* P, long long n);  // synchronous plans only

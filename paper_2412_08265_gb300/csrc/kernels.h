@@ -119,7 +119,7 @@ struct SetupParams {
     // the deposit's geometry: fixed-point shifts, band entries, path limits
     int fb, jc, apb, kind;
     float a_max, s_min, s_max;
-    PartRec* prec;           // [n_in]
+    PartRec* prec;           // [n_in], for the adjoint (nullable)
     long long n_cap;         // capacity of rec / prec
 };
 int launch_setup(const SetupParams& P, long long n_total, cudaStream_t st);

@@ -54,6 +54,7 @@ struct Request {
     float* out = nullptr;
     bool out_dev = false, out_pinned = false;
     size_t bytes = 0;
+    bool compact = false;
     double work = 0;           // estimated GPU work: deposits + kVoxelWork per cube voxel
     Clock::time_point t_submit, t_done;
     ReqState state = kQueued;
@@ -144,6 +145,7 @@ void admit(rubix_server* srv, const ReqPtr& r) {
     a.stream = sl.stream;
     a.pool = srv->pool;
     a.staging = !r->p.on_device;
+    a.compact = r->compact;
     rubix_status s = plan_init(&r->plan, srv->S, &r->tel, std::max<int64_t>(r->p.n, 1), a, !r->out_dev, false);
     if (s == RUBIX_OK) {
         r->dout = r->out_dev ? r->out : r->plan.d_out;
@@ -380,6 +382,17 @@ done:
     return RUBIX_OK;
 }
 
+// Footprint of a request, and whether it is a compact plan's: one that the budget
+// does not hold with small work items (up to four times the partial rows and sort
+// tiles of a galaxy of some 1e5 particles) takes those of 256 particles.
+static size_t request_bytes(const rubix_server* srv, const rubix_telescope* tel, const rubix_particles* p, bool with_out,
+                            bool* compact) {
+    const long long n = std::max<int64_t>(p->n, 1);
+    const size_t b = plan_bytes(*srv->S, tel, n, with_out, false, !p->on_device, false);
+    *compact = b > srv->budget;
+    return *compact ? plan_bytes(*srv->S, tel, n, with_out, false, !p->on_device, true) : b;
+}
+
 extern "C" rubix_status rubix_serve_submit(rubix_server_t* srv, const rubix_telescope* tel, const rubix_particles* p,
                                            uint64_t noise_seed, float noise_s2n, float* cube_out,
                                            int32_t cube_on_device, uint64_t* ticket) {
@@ -403,7 +416,7 @@ extern "C" rubix_status rubix_serve_submit(rubix_server_t* srv, const rubix_tele
         r->out_pinned = cudaPointerGetAttributes(&at, cube_out) == cudaSuccess && at.type == cudaMemoryTypeHost;
         cudaGetLastError();
     }
-    r->bytes = plan_bytes(*srv->S, tel, std::max<int64_t>(p->n, 1), !r->out_dev, false, !p->on_device);
+    r->bytes = request_bytes(srv, tel, p, !r->out_dev, &r->compact);
     r->work = ((double)p->n + kVoxelWork * (double)tel->nx * tel->ny) * tel->n_lambda;
     r->t_submit = Clock::now();
     std::lock_guard<std::mutex> lk(srv->mu);
@@ -429,7 +442,8 @@ extern "C" rubix_status rubix_serve_footprint(rubix_server_t* srv, const rubix_t
     if (s != RUBIX_OK) return s;
     s = validate_telescope(tel, srv->S->ssp.dls);
     if (s != RUBIX_OK) return s;
-    *bytes = plan_bytes(*srv->S, tel, std::max<int64_t>(p->n, 1), cube_on_device == 0, false, !p->on_device);
+    bool compact;
+    *bytes = request_bytes(srv, tel, p, cube_on_device == 0, &compact);
     return RUBIX_OK;
 }
 

@@ -149,7 +149,7 @@ __global__ void k_setup(SetupParams P) {
         r.ef = (unsigned)(8 * e) | (path << 30);
         P.map[i] = mr;
         P.rec[i] = r;
-        P.prec[i] = pr;
+        if (P.prec) P.prec[i] = pr;
     }
 }
 
