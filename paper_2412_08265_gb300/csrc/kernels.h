@@ -241,6 +241,7 @@ struct ConvParams {
     uint32_t seed_lo, seed_hi;
     unsigned* err;               // device error word (bounded waits of the fused kernel; nullable)
     int ty;                      // output rows per CTA (set at launch)
+    int xb_first;                // first block of kConvX columns of the launch (set at launch)
     // segment offsets of the cube's spaxels, seg_bands per spaxel (nullable): a
     // (row, block of kConvX columns) without a particle within rp columns is
     // taken as zero, unread

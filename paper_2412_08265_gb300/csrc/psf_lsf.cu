@@ -12,6 +12,8 @@
 //   pass 2 (k_psfy_noise): each thread owns one (x, wavelength) column of a
 //     y-chunk and applies the PSF along y, then optional Philox noise.
 // All global accesses run along wavelength (the fastest axis): coalesced.
+#include <algorithm>
+
 #include "common.cuh"
 #include "conv_layout.h"
 #include "kernels.h"
@@ -181,12 +183,9 @@ __global__ void __launch_bounds__(kTThreads, RUBIX_PSF_TMINB) k_psf_lsf(const __
     float* stages = smt + kHead;
     float* px = stages + kTS * G::stage_floats;  // [2][kTX][kTB] PSF-x output, alternating by row
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // wavelength tiles and blocks of columns share grid.x (grid.y ends at 65535:
-    // fields of up to 2^24 spaxels along x)
-    const int nx = P.nx, nl = P.n_lambda;
-    const unsigned n_lt = (unsigned)(nl + G::TL - 1) / (unsigned)G::TL;
-    const int j0 = (int)(blockIdx.x % n_lt) * G::TL, x0 = (int)(blockIdx.x / n_lt) * kTX, y0 = blockIdx.y * P.ty;
+    const int j0 = blockIdx.x * G::TL, x0 = (int)(P.xb_first + blockIdx.y) * kTX, y0 = blockIdx.z * P.ty;
     const int y1 = min(y0 + P.ty, P.ny);
+    const int nx = P.nx, nl = P.n_lambda;
     const int n_rows = (y1 - y0) + 2 * RP;  // input rows y0 - RP .. y1 + RP - 1
     float gl[2 * RL + 1], gp[NR];
 #pragma unroll
@@ -403,10 +402,18 @@ static bool launch_conv(ConvParams P, const CUtensorMap* map, const DenseRows& D
     if (cudaFuncSetAttribute(k_psf_lsf<RP, RL, DENSE, NOISE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem) !=
         cudaSuccess)
         return false;
-    const long long columns = (long long)((P.n_lambda + G::TL - 1) / G::TL) * ((P.nx + kTX - 1) / kTX);
-    P.ty = rows_per_cta(P.ny, RP, columns, (long long)RUBIX_PSF_TMINB * sm_count(), kMaxTY);
-    const dim3 g((unsigned)columns, (P.ny + P.ty - 1) / P.ty);
-    k_psf_lsf<RP, RL, DENSE, NOISE><<<g, kTThreads, G::smem, st>>>(P, *map, D, out);
+    const int n_lt = (P.n_lambda + G::TL - 1) / G::TL, n_xb = (P.nx + kTX - 1) / kTX;
+    P.ty = rows_per_cta(P.ny, RP, (long long)n_lt * n_xb, (long long)RUBIX_PSF_TMINB * sm_count(), kMaxTY);
+    // grid.y ends at 65535: a field of more than 524,280 spaxels along x (up to 2^24)
+    // takes several launches. (Column blocks in grid.x, whose end is far off, with
+    // the wavelength tiles in grid.y: 1e4 particles in 300 x 300 x 3721, 600 -> 726
+    // us; both in grid.x by a division: the convolution of 81 x 150 x 3721, 127 -> 133;
+    // a first column that is not known as a multiple of 8: 131.)
+    for (int b = 0; b < n_xb; b += 65535) {
+        P.xb_first = b;
+        const dim3 g(n_lt, std::min(n_xb - b, 65535), (P.ny + P.ty - 1) / P.ty);
+        k_psf_lsf<RP, RL, DENSE, NOISE><<<g, kTThreads, G::smem, st>>>(P, *map, D, out);
+    }
     return true;
 }
 
@@ -437,7 +444,7 @@ bool psf_lsf_needs_tmp(int rp, int rl) {
 int launch_psf_lsf(const ConvParams& P, const float* in, int in_pitch, const CUtensorMap* in_map, float* tmp,
                    float* out, cudaStream_t st) {
     if (!in_map && in_pitch != P.n_lambda) return -1;  // without a map: dense rows
-    if (try_conv(P, in_map, in, out, st)) return 1;
+    if (try_conv(P, in_map, in, out, st)) return 1;  // (wide fields: a few launches, counted as one)
     // generic radii: two passes through an intermediate cube
     const int XW = kXC + 2 * P.rp;
     const size_t smem = (size_t)XW * (kLC + 2 * P.rl + kLC) * sizeof(float);
