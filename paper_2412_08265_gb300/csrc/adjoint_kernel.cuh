@@ -530,12 +530,8 @@ __global__ void __launch_bounds__(RUBIX_ADJ_THREADS, 1) k_adjoint_tiles(const __
                     if (sp < 0 || sp >= P.n_s) {
                         atomicOr(P.err, kErrBadItem);
                     } else {
-                        qb = I.begin;
-                        qe = I.end;
-                        if (nb > 1) {
-                            qb = max(qb, P.seg_off[(long long)sp * nb + band]);
-                            qe = min(qe, P.seg_off[(long long)sp * nb + band + 1]);
-                        }
+                        qb = max(I.begin, P.seg_off[(long long)sp * nb + band]);
+                        qe = min(I.end, P.seg_off[(long long)sp * nb + band + 1]);
                         live = qb < qe;
                         // the item's first weights and record, on their way to L1,
                         // and its tile slice of dL/dcube0 on its way to L2

@@ -13,7 +13,7 @@ constexpr double kC_kms = 299792.458;
 
 // Error word written by kernels (bit flags), read by the host after a forward.
 enum DeviceError : unsigned {
-    kErrTmaTimeout = 1u,      // a bounded wait expired (the mbarrier of a slab or cube row load)
+    kErrTmaTimeout = 1u,      // a bounded wait expired (the mbarrier of a slab or cube row load, the items' scan)
     kErrBadItem = 2u,         // a work item pointed outside its buffers
     kErrBounds = 4u,          // debug builds: a computed index fell outside its buffer
 };
@@ -162,11 +162,11 @@ __device__ __forceinline__ int age_band(int ia, int apb, int n_bands) {
 // tile's sum, and add up the sums published before theirs: a block waits only
 // for blocks that hold an earlier ticket, which are running and publish without
 // waiting for anyone. chain[0] is the ticket, chain[1 + tile] the tile's sum
-// with its top bit set; all are cleared beforehand. The wait has a limit (about
-// a millisecond; the blocks of a GPU that was taken away from the process in
-// between may meet it), after which the block adds up the missing tiles itself:
-// the result is the same whatever was waited for. (chain_words in sort_layout.h
-// gives the words of a chain.)
+// with its top bit set; all are cleared beforehand. The wait has a limit in cycles
+// (the blocks of a GPU that was taken away from the process in between may meet
+// it), after which the prefix says that sums are missing from it: kChainShort, a
+// millisecond, where the block can then do without them, kChainLong where that is
+// an error. (chain_words in sort_layout.h gives the words of a chain.)
 // ----------------------------------------------------------------------------
 struct ChainShared {
     unsigned ticket;
@@ -210,25 +210,27 @@ __device__ __forceinline__ unsigned long long block_exclusive(unsigned long long
     return r;
 }
 
-constexpr long long kChainWait = 2000000;  // cycles a block waits for the sums before its own
+constexpr long long kChainShort = 2000000ll, kChainLong = 4000000000ll;
+constexpr unsigned long long kChainMissing = 1ull << 52;
 
-// Exclusive prefix of v over all threads of all tiles before this one (values
-// and sums below 2^63). tile_sum(i) is tile i's sum from the scan's input. quiet
-// (tests): nothing is published.
-template <class TileSum>
+// Exclusive prefix of v over all threads of all tiles before this one (sums below
+// 2^52); at least kChainMissing, for every thread of the block, if a wait ran out:
+// its lower bits are then a sum too small, never too large. quiet (tests): nothing
+// is published, and waits are short.
 __device__ __forceinline__ unsigned long long chain_exclusive(unsigned long long v, unsigned tile,
-                                                              unsigned long long* chain, ChainShared& sh, bool quiet,
-                                                              TileSum tile_sum) {
+                                                              unsigned long long* chain, ChainShared& sh, long long wait,
+                                                              bool quiet) {
     unsigned long long total;
     const unsigned long long e = block_exclusive(v, sh, total);
     volatile unsigned long long* pub = chain + 1;
     if (threadIdx.x == 0 && !quiet) pub[tile] = total | (1ull << 63);
     unsigned long long before = 0;
+    if (quiet) wait = kChainShort;
     const long long t0 = clock64();
     for (unsigned i = threadIdx.x; i < tile; i += blockDim.x) {
         unsigned long long w = pub[i];
-        while (!(w >> 63) && clock64() - t0 < kChainWait) w = pub[i];
-        before += (w >> 63) ? w & ~(1ull << 63) : tile_sum(i);
+        while (!(w >> 63) && clock64() - t0 < wait) w = pub[i];
+        before += (w >> 63) ? w & ~(1ull << 63) : kChainMissing;
     }
     unsigned long long sum;
     block_exclusive(before, sh, sum);

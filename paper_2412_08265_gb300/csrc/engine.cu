@@ -551,11 +551,11 @@ static int fault_alloc_at() {
     return e ? std::atoi(e) : 0;
 }
 
-// RUBIX_FAULT_SCAN=1 (tests): the blocks of the plan's chained scans publish
-// nothing, so that every wait in them runs out.
-static bool fault_scan() {
+// RUBIX_FAULT_SCAN (tests): the blocks of a plan's scans publish nothing, so that
+// every wait in them runs out: 1 the sort's, 2 the work items'.
+static int fault_scan() {
     const char* e = std::getenv("RUBIX_FAULT_SCAN");
-    return e && std::atoi(e) != 0;
+    return e ? std::atoi(e) : 0;
 }
 
 rubix_status plan_init(Plan* P, const SspState* S, const rubix_telescope* tel, long long n, Alloc a, bool with_out,
@@ -731,7 +731,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
         P.launches += launch_assign(A, st);
         const int ls = launch_sort_by_key(P.d_key, n, P.n_s * S.geo.n_bands + 1, P.d_keys_tmp, P.d_vals_tmp, P.d_skeys,
                                           P.d_perm, P.d_seg_off, P.d_sort_scratch, sort_scratch_ints(P.cap, S.n_sm, P.alloc.compact),
-                                          P.alloc.compact, P.d_chain, (int)item_chain_words(P.n_s), P.quiet_scan, st);
+                                          P.alloc.compact, P.d_chain, (int)item_chain_words(P.n_s), P.quiet_scan == 1, st);
         if (ls < 0) return fail(RUBIX_ERR_CUDA, "internal: sort scratch too small for %lld particles", n);
         P.launches += ls;
     } else {
@@ -778,7 +778,7 @@ rubix_status enqueue_pre(Plan& P, const rubix_particles* p, cudaStream_t st, cud
     IP.item_cap = P.item_cap;
     IP.split = P.d_split;
     IP.chain = P.d_chain;
-    IP.quiet_scan = P.quiet_scan;
+    IP.quiet_scan = P.quiet_scan == 2;
     IP.slow_count = P.alloc.async ? nullptr : S.d_slow;  // one forward at a time on a handle
     IP.err = S.d_err;
     P.launches += launch_items(IP, st);

@@ -103,7 +103,7 @@ struct Plan {
     PartRec* d_pin = nullptr;  // [cap] (mass, age, Z, v_los) in original order, written by the assign
     int* d_sort_scratch = nullptr;
     int *d_seg_off = nullptr, *d_item_off = nullptr, *d_part_off = nullptr, *d_split = nullptr;
-    bool quiet_scan = false;                // tests: waits of the chained scans run out
+    int quiet_scan = 0;                     // tests: scans whose waits run out (RUBIX_FAULT_SCAN)
     unsigned long long* d_chain = nullptr;  // scan of the work items (ItemParams::chain)
     Item* d_items = nullptr;
     DepRec* d_rec = nullptr;

@@ -227,19 +227,16 @@ __global__ void __launch_bounds__(kItemTile) k_items(const ItemParams P, int n_t
     }
     const int ni = (e0 - b0 + P.chunk - 1) / P.chunk;
     const int np = ni > 1 ? ni : 0;  // partial rows
-    auto tile_sum = [&](unsigned i) {
-        unsigned long long t = 0;
-        const long long first = (long long)i * kItemTile, end = min(first + kItemTile, (long long)P.n_s);
-        for (long long k = first; k < end; ++k) {
-            const int m = (P.seg_off[(k + 1) * nb] - P.seg_off[k * nb] + P.chunk - 1) / P.chunk;
-            t += ((unsigned long long)(m > 1 ? m : 0) << 32) | (unsigned)m;
-        }
-        return t;
-    };
+    // items below, partial rows from bit kPartShift (at most 2^24 + 2^24 of each:
+    // spaxels, and particles / chunk)
+    constexpr int kPartShift = 26, kLow = (1 << kPartShift) - 1;
     const unsigned long long pre =
-        chain_exclusive(((unsigned long long)np << 32) | (unsigned)ni, tile, P.chain, sh, P.quiet_scan, tile_sum);
+        chain_exclusive(((unsigned long long)np << kPartShift) | (unsigned)ni, tile, P.chain, sh, kChainLong, P.quiet_scan);
+    // a wait that ran out: offsets too small, so that items are lost, but every
+    // offset stays within its buffers and readers check what the items hold
+    if (pre >= kChainMissing) atomicOr(P.err, kErrTmaTimeout);
     if (s > P.n_s) return;
-    const int base = (int)(pre & 0xffffffffu), part = (int)(pre >> 32);
+    const int base = (int)pre & kLow, part = (int)(pre >> kPartShift) & kLow;
     P.item_off[s] = base;
     P.part_off[s] = part;
     if (np) P.split[atomicAdd(P.chain + n_tiles + 1, 1ull)] = (int)s;

@@ -154,13 +154,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const int* __restrict__ i
         v[i] = (base + i < n) ? in[base + i] : 0;
         s += v[i];
     }
-    auto tile_sum = [&](unsigned i) {
-        const long long b = (long long)i * kScanTile, e = min(b + kScanTile, n);
-        unsigned long long t = 0;
-        for (long long k = b; k < e; ++k) t += (unsigned)in[k];
-        return t;
-    };
-    unsigned long long e = chain_exclusive((unsigned long long)s, tile, chain, sh, quiet, tile_sum);
+    unsigned long long e = chain_exclusive((unsigned long long)s, tile, chain, sh, kChainShort, quiet);
+    if (e >= kChainMissing) {  // a wait ran out (uniform): the counts before the tile from the input
+        unsigned long long before = 0, sum;
+        for (long long i = threadIdx.x; i < (long long)tile * kScanTile; i += kScanThreads) before += (unsigned)in[i];
+        block_exclusive(before, sh, sum);
+        e = sum + block_exclusive((unsigned long long)s, sh, before);
+    }
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
         if (base + i < n) out[base + i] = (int)e;

@@ -1,7 +1,9 @@
-"""The one-launch scans (sort digits, work items) when every wait in them runs out:
-RUBIX_FAULT_SCAN=1 keeps the blocks from publishing their sums, so that each adds up
-the tiles before its own after its limit. Order, offsets, cube and gradients are
-bit for bit those of the scans that wait, and nothing is reported as an error."""
+"""The one-launch scans when every wait in them runs out (RUBIX_FAULT_SCAN keeps the
+blocks from publishing their sums). 1, the sort's: each block counts the tiles
+before its own itself; order, offsets, cube and gradients are bit for bit those
+of the scans that wait, and nothing is reported. 2, the work items': items are
+lost, which the device error word says; forward and gradient still stay within
+their buffers, and the context serves the next model."""
 import os
 
 import numpy as np
@@ -39,3 +41,31 @@ def test_expired_scan_waits_change_nothing(n, nx, ny):
         model.close()
     for a, b in zip(got["0"], got["1"]):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_bands_grid", [(12, 5), (3, 2)])  # several age bands, and one
+def test_expired_item_scan_is_reported(n_bands_grid):
+    import torch
+    from paper_2412_08265_gb300.model import CubeModel
+    ssp = synth.ssp_grid(*n_bands_grid, 200, 4500.0, 4748.75)
+    tel = synth.Telescope(nx=61, ny=53, spaxel_size=0.3, n_lambda=65, lambda0=4560.0, dlambda=1.25)
+    rng = np.random.default_rng(8)
+    n = 30_000
+    f = lambda a: np.ascontiguousarray(a, dtype=np.float32)
+    p = synth.Particles(x=f(rng.uniform(-9, 9, n)), y=f(rng.uniform(-8, 8, n)), mass=f(rng.uniform(0.5, 2.0, n)),
+                        age=f(np.exp(rng.uniform(-2.0, 2.5, n))), Z=f(np.exp(rng.uniform(-9.0, -3.0, n))),
+                        v_los=f(rng.normal(0.0, 150.0, n)))
+    G = torch.ones((53, 61, 65), device="cuda")
+    ref = CubeModel(ssp, tel, "f32", max_particles=n)
+    want = ref.forward(p).clone()
+    os.environ["RUBIX_FAULT_SCAN"] = "2"
+    try:
+        model = CubeModel(ssp, tel, "f32", max_particles=n)
+    finally:
+        del os.environ["RUBIX_FAULT_SCAN"]
+    model.forward(p)
+    model.backward(G)
+    torch.cuda.synchronize()
+    assert model.stats()["device_error"] & 1
+    model.close()
+    assert torch.equal(ref.forward(p), want) and ref.stats()["device_error"] == 0
