@@ -1,6 +1,9 @@
-// conv_layout.h -- output rows per CTA of the fused PSF/LSF kernel (psf_lsf.cu):
-// host arithmetic without a GPU.
+// conv_layout.h -- grids of the passes after the deposit, as host arithmetic
+// without a GPU: blocks of the row pass (rows.cu), output rows per CTA of the fused
+// PSF/LSF kernel (psf_lsf.cu).
 #pragma once
+
+#include <algorithm>
 
 namespace rubix {
 
@@ -28,6 +31,17 @@ inline int rows_per_cta(int ny, int rp, long long columns, long long slots, int 
         }
     }
     return best;
+}
+
+constexpr int kRowThreads = 256;
+constexpr int kCombineBins = 128;  // bins of one row per combine unit: 4 per lane of one warp
+
+// Blocks of the row pass: a warp per spaxel (zero rows) or per combine unit (rows of
+// at most max_split split spaxels), up to eight blocks per SM.
+inline int row_blocks(long long n_s, long long max_split, int n_lambda, int n_sm) {
+    const long long units = std::min(max_split, n_s) * ((n_lambda + kCombineBins - 1) / kCombineBins);
+    const long long warps = std::max(n_s, units), per = kRowThreads / 32;
+    return (int)std::min((warps + per - 1) / per, 8ll * n_sm);
 }
 
 }  // namespace rubix

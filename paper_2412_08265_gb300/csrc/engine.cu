@@ -834,6 +834,7 @@ int enqueue_post(Plan& P, float* target, float* out, uint64_t noise_seed, float 
     RP.part_off = P.d_part_off;
     RP.split = P.d_split;
     RP.n_split = P.d_chain + item_chain_words(P.n_s) - 1;
+    RP.max_split = P.last_n / item_chunk(*P.S, P.last_n, P.alloc.compact);
     RP.partials = P.d_partials;
     RP.cube = target;
     int l = launch_rows(RP, st);

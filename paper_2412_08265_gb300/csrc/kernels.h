@@ -225,6 +225,7 @@ struct RowParams {
     const int* part_off;
     const int* split;                    // the split spaxels
     const unsigned long long* n_split;   // their number
+    long long max_split;                 // the most there can be
     const float* partials;
     float* cube;
 };

@@ -2,6 +2,7 @@
 // sum of Sec. 3): rows of spaxels without particles, and rows of split
 // spaxels, summed from their work items' partial rows.
 #include "common.cuh"
+#include "conv_layout.h"
 #include "kernels.h"
 #include "twosum.cuh"
 
@@ -56,8 +57,6 @@ __device__ __forceinline__ void zero_rows(const RowParams& P, long long w0, long
 // which on this GPU runs at 1/64 of the FP32 rate.
 // ----------------------------------------------------------------------------
 
-constexpr int kCombineBins = 128;  // bins of one row per combine unit: 4 per lane of one warp
-
 // One unit = kCombineBins bins of one split spaxel's row, taken by one warp
 // (lane l sums bins l, l + 32, l + 64, l + 96 of the unit: four independent
 // loads per partial row in flight), so that the rows of a very high-count
@@ -99,7 +98,7 @@ __device__ __forceinline__ void combine_rows(const RowParams& P, long long warp,
 }
 
 // The split spaxels' rows first: they take longest.
-__global__ void __launch_bounds__(256) k_rows(const __grid_constant__ RowParams P) {
+__global__ void __launch_bounds__(kRowThreads) k_rows(const __grid_constant__ RowParams P) {
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -110,10 +109,7 @@ __global__ void __launch_bounds__(256) k_rows(const __grid_constant__ RowParams 
 int launch_rows(const RowParams& P, cudaStream_t st) {
     const long long n_s = (long long)P.nx * P.ny;
     if (n_s < 1) return 0;
-    long long nb = (n_s * 32 + 255) / 256;
-    const long long cap = 8ll * sm_count();
-    if (nb > cap) nb = cap;
-    k_rows<<<(int)nb, 256, 0, st>>>(P);
+    k_rows<<<row_blocks(n_s, P.max_split, P.n_lambda, sm_count()), kRowThreads, 0, st>>>(P);
     return 1;
 }
 

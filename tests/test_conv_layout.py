@@ -1,7 +1,9 @@
-"""The row split of the fused PSF/LSF kernel (csrc/conv_layout.h, host arithmetic):
-it is the best of all splits of the rows into equal parts, and it is found in a
-number of steps that stays small however many rows there are (every launch asks
-for it). Compiled and run on the host; no GPU."""
+"""Grids of the passes after the deposit (csrc/conv_layout.h, host arithmetic;
+compiled and run on the host, no GPU). The row split of the fused PSF/LSF kernel is
+the best of all splits of the rows into equal parts, and it is found in a number of
+steps that stays small however many rows there are (every launch asks for it). The
+row pass has a warp for every unit of work up to its eight blocks per SM, also
+where few spaxels hold many particles."""
 import os
 import subprocess
 
@@ -44,10 +46,43 @@ int main() {
 """
 
 
-def test_row_split_is_the_best_and_cheap_to_find(tmp_path):
+ROWS = r"""
+#include <cstdio>
+#include <initializer_list>
+#include "conv_layout.h"
+using namespace rubix;
+int main() {
+    for (long long n_s : {1ll, 5ll, 64ll, 625ll, 1600ll, 22500ll, 1ll << 24})
+        for (long long max_split : {0ll, 1ll, 3ll, 100ll, 4000ll, 80000ll, 1ll << 22})
+            for (int n_lambda : {1, 128, 129, 1000, 3721, 8192})
+                for (int n_sm : {1, 152}) {
+                    const long long blocks = row_blocks(n_s, max_split, n_lambda, n_sm), full = 8ll * n_sm;
+                    const long long split = max_split < n_s ? max_split : n_s;
+                    const long long units = split * ((n_lambda + kCombineBins - 1) / kCombineBins);
+                    const long long warps = blocks * (kRowThreads / 32);
+                    if (blocks < 1 || blocks > full) return 1;
+                    if (blocks < full && (warps < n_s || warps < units)) {
+                        std::printf("%lld spaxels, %lld split, %d bins: %lld blocks\n", n_s, max_split, n_lambda, blocks);
+                        return 2;
+                    }
+                }
+    return 0;
+}
+"""
+
+
+def _run(tmp_path, program):
     src, exe = tmp_path / "layout.cpp", tmp_path / "layout"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     r = subprocess.run(["g++", "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+def test_row_pass_has_a_warp_per_unit(tmp_path):
+    _run(tmp_path, ROWS)
+
+
+def test_row_split_is_the_best_and_cheap_to_find(tmp_path):
+    _run(tmp_path, PROGRAM)
