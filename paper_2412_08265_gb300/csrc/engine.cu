@@ -253,111 +253,43 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
         S.lz_nodes = h->d_lz;
     }
 
-    // ---- deposit tiling: wavelength tiles and the slab staged per tile and age
-    // band: a band's age pairs (an odd number of 8-byte entries per node) over
-    // the nodes of the tile's R rounds plus a Doppler halo of
-    // +-RUBIX_DEP_VHALO. Among the band sizes that fit, take the one with the
-    // lowest estimated cost per particle: n_tiles * (per-particle setup + R
-    // rounds + bands). ----
+    // ---- deposit tiling: wavelength tiles and the slab staged per tile and age band ----
+    const SlabLayout L = slab_layout(S.n_age, S.n_Z, S.ls0, S.dls, tel->n_lambda, tel->lambda0, tel->dlambda, tel->z_cosmo,
+                                     ((long long)h->smem_optin - kDepHeader) / (long long)sizeof(float2),
+                                     RUBIX_DEP_VHALO / kC_kms, RUBIX_DEP_BANDS);
     const int ca = std::max(S.n_age - 1, 1);
-    const double A0 = tel->dlambda / ((1.0 + tel->z_cosmo) * S.dls);
-    const double beta = RUBIX_DEP_VHALO / kC_kms;
-    const double a_lo = A0 / (1.0 + beta), a_hi = A0 / (1.0 - beta);
-    const double lam_max = (tel->lambda0 + (tel->n_lambda - 1) * tel->dlambda) / (1.0 + tel->z_cosmo);
-    const int shift = (int)std::ceil(lam_max / S.dls * beta / (1.0 - beta));
-    const long long budget = ((long long)h->smem_optin - kDepHeader) / (long long)sizeof(float2);
-    const int nzc = std::max(S.n_Z, 2);  // entries per age cell and node
+    h->apb = L.apb;
     SlabParams& G = h->geo;
-    // kind 0 covers dt/dj in (30/31, 1] (and the two-read rounds just above 1)
-    // when the halo's range reaches it; kind 1 dt/dj in [1/2, 1); else kind 2
-    G.kind = (a_lo > 30.0 / 31.0 && a_lo < 1.0) ? 0 : ((a_lo >= 0.5 && a_hi < 0.999) ? 1 : 2);
-    const int B = kind_bins(G.kind);
-    struct Geo { int apb, bands, pitch, slab_w, R, need; double cost; };
-    Geo best{0, 0, 0, 0, 0, 0, 1e300};
-#define RUBIX_R(r) r,
-    const int rounds[] = {RUBIX_ROUNDS(RUBIX_R)};
-#undef RUBIX_R
-    for (int apb = ca; apb >= 1; --apb) {
-        const int bands = (ca + apb - 1) / apb;
-        if (bands > kMaxBands) break;
-        if (RUBIX_DEP_BANDS > 0 && bands != std::min(RUBIX_DEP_BANDS, ca)) continue;
-        const int pitch = (apb * nzc) | 1;
-        const int slab_max = (int)std::min<long long>(budget / pitch, 1 << 14) / 4 * 4;
-        for (int r : rounds) {
-            // bins of the last lane of the last round, deposit (also a mean
-            // round more) and adjoint (rounds of 32 bins, of 31 edges for means)
-            const int last = std::max({B * (r - 1) + 31, (B - 1) * r + r + 1, (B * r + 31) / 32 * 32 - 1});
-            const int need = (int)std::ceil((last + 1) * std::max(a_hi, 1.0)) + 3;
-            if (need + 2 * shift + 8 > slab_max) continue;
-            // a slab twice the halo wide at most: more would only be staged
-            const int slab_w = std::min(slab_max, (need + 4 * shift + 11) / 4 * 4);
-            const int n_tiles = (tel->n_lambda + B * r - 1) / (B * r);
-            const double cost = n_tiles * (40.0 + 15.0 * r + 6.0 * bands);
-            if (cost < best.cost) best = Geo{apb, bands, pitch, slab_w, r, need, cost};
-        }
-    }
-    // no slab fits (very wide Doppler halo): global-memory path only (need = 0 =
-    // slab_w fails every kernel's test for a fast path)
-    if (best.R == 0) best = Geo{ca, 1, (ca * nzc) | 1, 0, 1, 0, 0.0};
-    h->apb = best.apb;
-    G.n_bands = best.bands;
-    G.pitch = best.pitch;
-    G.slab_w = best.slab_w;
-    G.need = best.need;
-    G.a_max = (float)a_hi;
-    G.tile_w = B * best.R;
-    G.n_tiles = (tel->n_lambda + G.tile_w - 1) / G.tile_w;
+    G.kind = L.kind;
+    G.n_bands = L.n_bands;
+    G.pitch = L.pitch;
+    G.slab_w = L.slab_w;
+    G.need = L.need;
+    G.a_max = L.a_max;
+    G.tile_w = L.tile_w;
+    G.n_tiles = L.n_tiles;
     G.n_lambda = tel->n_lambda;
     G.n_ls = S.n_ls;
     G.es = S.n_Z > 1 ? 1 : 2;
     G.pad = G.slab_w + 8;
     for (int m = 0; m < 2; ++m) {
-        G.ib[m] = (float)std::floor((B - m) * A0 + 0.5);
-        G.fbr[m] = (float)((B - m) * A0 - G.ib[m]);
+        G.ib[m] = L.ib[m];
+        G.fbr[m] = L.fbr[m];
     }
-    G.a0_1m = (float)(1.0 - A0);
-    // fixed point of the Doppler shifts: fb bits after the point, such that a
-    // position anywhere in a slab's margin fits 32 bits and the shift per bin
-    // (|g| <= A0 beta / (1 - beta), times 2^(fb + 13)) 31
-    G.fb = 26;
-    while (G.fb > 0 && ((G.slab_w - G.need + 4.0) * std::ldexp(1.0, G.fb) >= 4294967296.0 ||
-                        A0 * beta / (1.0 - beta) * std::ldexp(1.0, G.fb + 13) >= 2147483648.0))
-        --G.fb;
-    G.jc = tel->n_lambda > 4096 ? 4096 : 0;
+    G.a0_1m = L.a0_1m;
+    G.fb = L.fb;
+    G.jc = L.jc;
+    G.s_min = L.s_min;
+    G.s_max = L.s_max;
     G.cost_c0 = RUBIX_DEP_COSTC0;
-    for (int b = 0; b < kMaxBands; ++b) G.band_e0[b] = std::min(b * best.apb, ca - 1) * nzc;
-    std::vector<int> klo(G.n_tiles, 0);
-    std::vector<unsigned> tref(2 * (size_t)G.n_tiles, 0u);
-    std::vector<float2> lref(32);
-    G.s_min = -1e30f;
-    G.s_max = 1e30f;
-    for (int t = 0; t < G.n_tiles; ++t) {
-        // nodes the tile's fast path reads: K0 .. K0 + need - 1 with K0 within
-        // +-shift of the zero-velocity position t00 of its first bin
-        const int j0 = t * G.tile_w;
-        const double t00 = ((tel->lambda0 + j0 * tel->dlambda) / (1.0 + tel->z_cosmo) - S.ls0) / S.dls;
-        const double k = std::floor((t00 - shift - 1.0 - 0.5 * (G.slab_w - G.need - 2 * shift - 8)) / 4.0) * 4.0;
-        klo[t] = (int)std::max(-1e6, std::min(k, 1e6));
-        for (int m = 0; m < 2; ++m) {
-            const double c = t00 - 0.5 * A0 * m - klo[t];  // at rest, from the slab's first node
-            if (G.slab_w > 0 && std::abs(t00) < 9e5)
-                tref[(size_t)m * G.n_tiles + t] = (unsigned)std::llround(std::ldexp(c, G.fb));
-            else
-                G.s_max = -1e30f;  // no slab, or bins absurdly far from the templates: per-bin path
-            // a particle's first node K0 in [0, slab_w - need) for every tile
-            G.s_min = std::max(G.s_min, (float)(0.01 - c));
-            G.s_max = std::min(G.s_max, (float)(G.slab_w - G.need - 0.01 - c));
-        }
-    }
-    for (int l = 0; l < 32; ++l) {
-        const double w = std::floor(l * A0);
-        lref[l] = make_float2((float)w, (float)(l * A0 - w));
-    }
+    for (int b = 0; b < kMaxBands; ++b) G.band_e0[b] = std::min(b * L.apb, ca - 1) * L.nzc;
+    std::vector<float2> lref;
+    for (int l = 0; l < 32; ++l) lref.push_back(make_float2(L.lane_node[l], L.lane_rest[l]));
     if (dalloc_sync(&h->d_tile_klo, G.n_tiles) || dalloc_sync(&h->d_tile_ref, 2 * (size_t)G.n_tiles) ||
         dalloc_sync(&h->d_lane_ref, 32))
         return bail(fail(RUBIX_ERR_OOM, "tile alloc"));
-    cudaMemcpy(h->d_tile_klo, klo.data(), klo.size() * 4, cudaMemcpyHostToDevice);
-    cudaMemcpy(h->d_tile_ref, tref.data(), tref.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(h->d_tile_klo, L.klo.data(), L.klo.size() * 4, cudaMemcpyHostToDevice);
+    cudaMemcpy(h->d_tile_ref, L.tile_ref.data(), L.tile_ref.size() * 4, cudaMemcpyHostToDevice);
     cudaMemcpy(h->d_lane_ref, lref.data(), 32 * sizeof(float2), cudaMemcpyHostToDevice);
     G.tile_ref = h->d_tile_ref;
     G.lane_ref = h->d_lane_ref;
@@ -390,7 +322,7 @@ rubix_status ssp_state_create(const rubix_ssp_grid* ssp, const rubix_telescope* 
             G.pair = h->d_pair;
             e = cudaMemcpy(d_t, tf.data(), nt * sizeof(float), cudaMemcpyHostToDevice);
             if (e == cudaSuccess) {
-                launch_build_pairs(G, best.apb, S.n_age, S.n_Z, d_t, h->d_pair, h->d_pair_adj, nullptr);
+                launch_build_pairs(G, L.apb, S.n_age, S.n_Z, d_t, h->d_pair, h->d_pair_adj, nullptr);
                 e = cudaDeviceSynchronize();
             }
         }

@@ -6,14 +6,14 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "slab_layout.h"
+
 namespace rubix {
 
 struct DepRec;
 struct MapRec;
 struct PartRec;
 struct Item;
-
-constexpr int kMaxBands = 32;
 
 // Streaming multiprocessors of the current device (cached per device); grid
 // caps of the grid-stride kernels are multiples of it.
@@ -37,8 +37,6 @@ int sm_count();
 #ifndef RUBIX_DEP_BANDS
 #define RUBIX_DEP_BANDS 0
 #endif
-// Rounds per wavelength tile that the deposit and the adjoint are built for.
-#define RUBIX_ROUNDS(X) X(1) X(2) X(3) X(4) X(6) X(8) X(10) X(11) X(12)
 // Cost of a work item in particle units, for the static split of the
 // (tile, item) cost space over CTAs.
 #ifndef RUBIX_DEP_COSTC0

@@ -33,15 +33,6 @@ __device__ __forceinline__ int node_pos(int j, int bi, float bf, float a_hi, flo
     return bi + (int)pi + (int)fl;
 }
 
-// Geometry of the rounds: a warp takes a particle's tile in rounds of kBins
-// consecutive bins, lane l owning bin j0 + kBins r + l. The kind follows from
-// the bin step in template nodes A = dt/dj (chosen once per wavelength grid):
-//   0: A near 1 (1 - A in [0, 1/31)): 31 bins, lanes on consecutive nodes;
-//   1: A in [1/2, 1): 30 bins, each lane on its bin's node, the next node's
-//      value from lane l + 1 or l + 2;
-//   2: any A: 32 bins, each lane reads both of its bin's nodes.
-constexpr int kind_bins(int kind) { return kind == 0 ? 31 : kind == 1 ? 30 : 32; }
-
 struct TileCtx {
     int j0, klo, slab_w, pitch, e0, es, n_lambda, n_ls, pad;
     uint32_t slab;         // shared-space address of the slab
