@@ -108,12 +108,20 @@ static __device__ __noinline__ AdjSums adj_general(const float2 w, const float4 
     }
     const bool use_slab = __all_sync(0xffffffffu, ok);
     AdjSums S{0.f, 0.f, 0.f, 0.f};
-    for (int o = lane; o < TW; o += 32) {
-        const int j = C.j0 + o;
-        if (j >= C.n_lambda) break;
+    for (int o0 = 0; o0 < TW && C.j0 + o0 < C.n_lambda; o0 += 32) {
+        const int j = C.j0 + o0 + lane;
+        const bool in = o0 + lane < TW && j < C.n_lambda;
         float f;
         const int k = node_pos(j, bi, g4.y, g4.z, g4.w, f);
-        const Forms p = node_forms<KIND>(w, quad_at(C, use_slab, e, k)), q = node_forms<KIND>(w, quad_at(C, use_slab, e, k + 1));
+        Forms p{0.f, 0.f, 0.f};
+        if (in) p = node_forms<KIND>(w, quad_at(C, use_slab, e, k));
+        // the next node's forms are the next lane's own where that lane is on it
+        // (as in the deposit's per-bin path)
+        const int kn = __shfl_down_sync(0xffffffffu, in ? k : INT_MIN, 1);
+        Forms q{__shfl_down_sync(0xffffffffu, p.m, 1), __shfl_down_sync(0xffffffffu, p.a, 1),
+                __shfl_down_sync(0xffffffffu, p.z, 1)};
+        if (!in) continue;
+        if (lane == 31 || kn != k + 1) q = node_forms<KIND>(w, quad_at(C, use_slab, e, k + 1));
         const float Gj = grow[j];
         S.sm = fmaf(Gj, fmaf(f, q.m - p.m, p.m), S.sm);
         S.sa = fmaf(Gj, fmaf(f, q.a - p.a, p.a), S.sa);

@@ -3,6 +3,8 @@
 // search over the cost space, the bin -> SSP node map, and the template slab.
 #pragma once
 
+#include <climits>
+
 #include "common.cuh"
 #include "kernels.h"
 
