@@ -19,12 +19,19 @@ from . import capi
 SCALAR_KEYS = ("preprojected", "inclination", "azimuth", "position_angle")
 
 
+# torch's own shortcut (not public: not there in every build of torch) to the
+# cudaStream_t of a device's current stream, without building a torch.cuda.Stream,
+# which costs as much as three launches
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _raw_stream(stream, device) -> int:
-    """The cudaStream_t of `stream`, or of the device's current stream (without
-    building a torch.cuda.Stream, which costs as much as three launches)."""
+    """The cudaStream_t of `stream`, or of the device's current stream."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(device.index)
+    if _current_raw_stream is not None:
+        return _current_raw_stream(device.index)
+    return torch.cuda.current_stream(device).cuda_stream
 
 
 def _dev_f32(a, device) -> torch.Tensor:
