@@ -380,12 +380,18 @@ def run_serving(args, dev, ssp):
             "clocks": clk, **res}
 
 
+def request_class_bytes(count: int, side: int) -> float:
+    """Bytes that `count` requests of side x side x 3721 bins cannot do without:
+    their FP32 cubes written once. (What is moved beyond that depends on the
+    galaxy: rows out of the PSF's reach are written by the convolution alone.)"""
+    return 4.0 * count * side * side * 3721
+
+
 def _serve_classes(torch, server, dev, args):
     """The two ends of the request mix, each as a saturated stream through the
-    served configuration: small galaxies in large cubes (HBM-bound: the
-    deposit writes every voxel, the PSF/LSF reads and writes it again, 12 B per
-    voxel) and large galaxies in small cubes (the deposit's FP32 work, 16 flop
-    per deposit); each with its fraction of the matching peak."""
+    served configuration: small galaxies in large cubes (the cubes' stores:
+    request_class_bytes) and large galaxies in small cubes (the deposit's FP32
+    work, 16 flop per deposit); each with its fraction of the matching peak."""
     from paper_2412_08265_gb300 import synth
     peaks = measured_peaks()
     hbm = float(peaks.get("hbm_gbs") or 6800.0)
@@ -408,8 +414,7 @@ def _serve_classes(torch, server, dev, args):
         _, mk = _drive(torch, srv, dev, reqs, [d] * count, np.zeros(count))
         srv.close()
         deposits = float(count) * n_in * 3721
-        voxels = float(count) * side * side * 3721
-        gbs = 12.0 * voxels / mk / 1e9
+        gbs = request_class_bytes(count, side) / mk / 1e9
         tfl = 16.0 * deposits / mk / 1e12
         out[name] = {"requests": count, "particles": n_p, "cube_side": side, "makespan_s": mk,
                      "requests_per_s": count / mk, "deposits_per_s": deposits / mk,
