@@ -115,7 +115,11 @@ typedef struct rubix_telescope {
                                      * ny-row field are modelled (0, 0 = all rows). Spaxel keys
                                      * are computed on the whole field, so a row-sharded galaxy
                                      * (each shard its own rows) gets bitwise the unsharded
-                                     * assignment; particles of other rows are dropped. The
+                                     * assignment; particles of other rows are dropped. Give
+                                     * every shard the same particle list: the grouping of a
+                                     * spaxel's sum follows the call's particle count, so
+                                     * that with lists cut down per shard the rows equal the
+                                     * unsharded cube's to rounding, not bitwise. The
                                      * cube then has row_hi - row_lo rows, PSF and LSF see zero
                                      * padding at its edges, noise is keyed by the window's own
                                      * voxel index. */
@@ -145,8 +149,8 @@ typedef struct rubix_cube rubix_cube_t;
 typedef struct rubix_server rubix_server_t;
 
 /* Create a forward-model handle for one SSP grid and one telescope.
- * Copies the SSP grid to the device in its storage dtype (rows padded to 16 B)
- * and reserves scratch for up to `max_particles` particles (grown on demand).
+ * Copies the SSP grid to the device in its storage dtype (as pairs of
+ * neighbouring ages) and reserves scratch for up to `max_particles` particles (grown on demand).
  * Errors: INVALID_ARG (bad sizes, non-increasing nodes, NULL pointers),
  * OOM, CUDA. On error *out is NULL. Uses the current CUDA device. */
 rubix_status rubix_cube_create(const rubix_ssp_grid *ssp, const rubix_telescope *tel,

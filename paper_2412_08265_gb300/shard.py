@@ -5,11 +5,14 @@ strong and weak scaling runs). Here a galaxy's field is split by spaxel rows:
 shard i models rows [lo_i, hi_i) only (the telescope's row window; spaxel
 keys are still computed on the whole field, so every particle lands in the
 same spaxel as unsharded, bit for bit). The deposit needs nothing from other
-shards. The PSF reaches r_psf rows across a block boundary, so before
-convolving, each shard takes the r_psf rows on each side from its
-neighbours' deposited (pre-PSF) rows -- one point-to-point exchange step --
-and convolves its extended block; its own rows of the result are then
-exactly the unsharded cube's rows (the LSF is along wavelength, local). At
+shards; every shard is given the whole particle list (a spaxel's sum is
+grouped by the list's length, so that a list cut down to the shard's own rows
+would give the same rows to rounding only). The PSF reaches r_psf rows across a
+block boundary, so before convolving, each shard takes the r_psf rows on each
+side from its neighbours' deposited (pre-PSF) rows -- one point-to-point
+exchange step -- and convolves its extended block; its own rows of the result
+are then exactly the unsharded cube's rows (the LSF is along wavelength,
+local). At
 the field's top and bottom there is no neighbour: the extended block simply
 ends there, which is the unsharded cube's zero padding.
 
