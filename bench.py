@@ -40,7 +40,7 @@ REL_ERR_BOUND = {"f32": 1e-5, "bf16": 2e-3}
 CSRC = os.path.join(ROOT, "paper_2412_08265_gb300", "csrc")
 # sources of the deposit kernel's code: a recorded DRAM traffic figure holds
 # only for the kernel built from the same sources
-DEPOSIT_SOURCES = ("deposit.cu", "deposit_kernel.cuh", "tile.cuh", "common.cuh")
+DEPOSIT_SOURCES = ("deposit.cu", "deposit_kernel.cuh", "slab_layout.h", "tile.cuh", "common.cuh")
 
 
 def deposit_sources_sha() -> str:

@@ -314,7 +314,6 @@ extern "C" rubix_status rubix_cube_backward(rubix_cube_t* h, uint64_t forward_ta
     A.prec = P.d_prec;
     A.perm = P.d_perm;
     A.seg_off = P.d_seg_off;
-    A.sorted_keys = P.d_skeys;
     A.n_s = P.n_s;
     A.n_bands = S.geo.n_bands;
     A.n_lambda = P.tel.n_lambda;

@@ -4,9 +4,11 @@
 // instrument's wavelength grid and added to the spaxel it falls in).
 //
 // K3 (k_setup, setup.cu) has turned each in-field particle, in sorted order,
-// into a 32-byte record: its four mass-scaled bilinear corner weights, its
-// SSP cell (whose four corner templates it interpolates) and the affine map
-// t(j) = B + jA from output bin j to the fractional SSP node position.
+// into a 32-byte record (DepRec): its four mass-scaled bilinear corner weights,
+// its cell's entry in the age band, its Doppler shift against a particle at rest in
+// fixed point, and which rounds it takes; and into a 16-byte record (MapRec) with
+// the full affine map t(j) = B + jA from output bin j to the fractional SSP node
+// position, for the per-bin path and the adjoint.
 //
 // The templates are kept, for the deposit, as age pairs: entry (ia, iz) of a
 // node holds T(ia, iz) and T(ia+1, iz), so that a cell's four corners are two
@@ -26,7 +28,7 @@
 // contiguous; band 0 writes the item's row and later bands continue it.
 //
 // One warp takes one particle at a time, R rounds of kBins bins (kinds in
-// tile.cuh). A lane forms M = sum_c w_c T_c at its node and interpolates to the
+// slab_layout.h). A lane forms M = sum_c w_c T_c at its node and interpolates to the
 // next node's value, which it takes from another lane by one shuffle (kinds 0
 // and 1) or from its own second read. Node positions of the rounds do not
 // depend on one another (tile.cuh), so that the rounds' loads can all be in
@@ -669,7 +671,7 @@ __global__ void __launch_bounds__(RUBIX_DEP_THREADS, 1) k_deposit(const __grid_c
 }
 
 // The kernel of a kind for R rounds per tile (one translation unit per kind);
-// nullptr for an R that is not built (kRoundsBuilt in kernels.h).
+// nullptr for an R that is not built (RUBIX_ROUNDS in slab_layout.h).
 typedef void (*DepositFn)(const DepositParams);
 template <int KIND>
 DepositFn deposit_fn(int R, bool means) {

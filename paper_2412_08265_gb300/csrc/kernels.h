@@ -171,7 +171,7 @@ struct SlabParams {
     int n_ls, pad, pitch, es;   // es: entries per cell index (tile.cuh)
     int n_bands;
     int band_e0[kMaxBands];     // first entry of each age band
-    int kind;                   // bins per round and how lanes reach their nodes (tile.cuh)
+    int kind;                   // bins per round and how lanes reach their nodes (slab_layout.h)
     int n_lambda;
     int tile_w;                 // output bins per tile = rounds x kind_bins(kind)
     int n_tiles;
@@ -266,7 +266,6 @@ struct AdjointParams {
     const PartRec* prec;       // [n_in] sorted order
     const int* perm;           // sorted position -> particle index
     const int* seg_off;        // [n_s * n_bands + 2]
-    const int* sorted_keys;    // [n] key per sorted position (spaxel * n_bands + band)
     int n_s, n_bands, n_lambda;
     double l0, dl, z_cosmo, flux_scale;
     const float* G0;           // [n_s][n_lambda] dL/dcube0

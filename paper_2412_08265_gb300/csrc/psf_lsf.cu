@@ -133,9 +133,10 @@ __global__ void __launch_bounds__(256) k_psfy_noise(const ConvParams P, const fl
 // in the same order for both forms (PSF x, LSF, PSF y; each over its taps in
 // order), so they give the same bits.
 //
-// Bound by shared-memory loads and the barrier per row, at about half of the
-// copy bandwidth. The dense form replaced a kernel of 4-byte cp.async copies
-// (81 x 150 spaxels x 3721 bins: 0.32 ms).
+// Bound by instruction issue (75 % of the slots; shared-memory wavefronts 67 %) and
+// the barrier per row: 150 x 150 spaxels x 3721 bins in 164 us, the dense form 81 x
+// 150 x 3721 in 127 us = 0.42 of the copy bandwidth (a kernel of 4-byte cp.async
+// copies took 323 us).
 // ----------------------------------------------------------------------------
 #ifndef RUBIX_PSF_TSTAGES
 #define RUBIX_PSF_TSTAGES 4

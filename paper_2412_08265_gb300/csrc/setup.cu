@@ -1,9 +1,10 @@
 // setup.cu -- K3 of the deposit path (Sec. 3: each star's SSP lookup and
 // Doppler shift, prepared once per particle): every in-field particle, in
-// sorted order, becomes a 32-byte record (its four mass-scaled bilinear
-// corner weights, its SSP cell and the affine map t(j) = B + jA from output
-// bin j to the fractional SSP node position), and each spaxel's particles
-// are cut into work items of at most `chunk` particles.
+// sorted order, becomes a 32-byte record for the deposit (its four mass-scaled
+// bilinear corner weights, its cell, its Doppler shift in fixed point, the rounds it
+// takes) and a 16-byte one with the affine map t(j) = B + jA from output bin j to
+// the fractional SSP node position, and each spaxel's particles are cut into work
+// items of at most `chunk` particles.
 #include "common.cuh"
 #include "kernels.h"
 #include "sort_layout.h"

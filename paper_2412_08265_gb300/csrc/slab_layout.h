@@ -20,7 +20,9 @@ constexpr int kMaxBands = 32;
 //   0: A near 1 (1 - A in [0, 1/31)): 31 bins, lanes on consecutive nodes;
 //   1: A in [1/2, 1): 30 bins, each lane on its bin's node, the next node's
 //      value from lane l + 1 or l + 2;
-//   2: any A: 32 bins, each lane reads both of its bin's nodes.
+//   2: any A: 32 bins, each lane reads both of its bin's nodes; at bin centres, for
+//      A in (1.03, 1.95) and CTAs with many work items, lanes read consecutive nodes
+//      instead and each bin takes its two from them by shuffles (rounds_gather).
 constexpr int kind_bins(int kind) { return kind == 0 ? 31 : kind == 1 ? 30 : 32; }
 
 struct SlabLayout {
